@@ -30,14 +30,21 @@ namespace lens {
 namespace {
 
 constexpr int kIpmThreads = 256;
-constexpr int kChunksPerGrab = 8;  // 32-cell chunks per fetch of the chunk counter
+// 32-cell chunks per fetch of the chunk counter: at most 8 (a single address
+// serves all warps, and a fetch per chunk made it the bound of a pass without
+// B and C work), fewer where that would leave a resident warp under 8 fetches:
+// with 8 always, the 900 chunks of a refinement level went to 112 of 4864
+// warps (308 us of a 200^2-pixel window's map) and the 7.8e3 chunks of a 500^2
+// grid to 976.
+constexpr int kMaxGrab = 8;
+constexpr int kBlocksPerSm = 4;
 
 constexpr int kWarps = kIpmThreads / 32;
 
 // One warp per round of 32 cells of a grid chunk (or of a cell list, or of
 // sub-cells given as four corners each), rounds handed out by a counter.
 template <bool QUADS, bool LIST = false>
-__global__ void __launch_bounds__(kIpmThreads, 4) k_ipm_cells(IpmArgs A) {
+__global__ void __launch_bounds__(kIpmThreads, kBlocksPerSm) k_ipm_cells(IpmArgs A) {
   __shared__ WarpCells sh[kWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t nchunks = (A.ncells + 31) >> 5;
@@ -45,15 +52,15 @@ __global__ void __launch_bounds__(kIpmThreads, 4) k_ipm_cells(IpmArgs A) {
   Ledger led;
   // Chunks of 32 cells are handed out by a counter (qcount[1]), so the
   // warps of a block finish together however the large cells fall; one
-  // fetch takes kChunksPerGrab chunks (a single address serves all warps, and
-  // a fetch per chunk made it the bound of a pass without B and C work).
+  // fetch takes A.grab chunks.
   unsigned* next = reinterpret_cast<unsigned*>(A.qcount) + 1;
   unsigned g_u = 0;
   if (lane == 0) g_u = atomicAdd(next, 1u);
-  int left = kChunksPerGrab;
-  for (int64_t ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * kChunksPerGrab; ch < nchunks;) {
+  const int grab = A.grab;
+  int left = grab;
+  for (int64_t ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * grab; ch < nchunks;) {
     // the following grab is fetched while this one is processed
-    if (lane == 0 && left == kChunksPerGrab) g_u = atomicAdd(next, 1u);
+    if (lane == 0 && left == grab) g_u = atomicAdd(next, 1u);
     const int64_t idx = ch * 32 + lane;
     const bool has = idx < A.ncells;
     int64_t c = idx;
@@ -78,8 +85,8 @@ __global__ void __launch_bounds__(kIpmThreads, 4) k_ipm_cells(IpmArgs A) {
     if (--left > 0) {
       ++ch;
     } else {
-      left = kChunksPerGrab;
-      ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * kChunksPerGrab;
+      left = grab;
+      ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * grab;
     }
   }
   block_add_stats<kWarps>(A.stats, led, A.wcell);
@@ -147,6 +154,8 @@ void ipm_launch(IpmArgs& A, bool quads, int* qcount, cudaStream_t s,
   LENS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t chunk_blocks = (A.ncells + kIpmThreads - 1) / kIpmThreads;
   const unsigned g = (unsigned)std::min<int64_t>(chunk_blocks, (int64_t)sms * 8);
+  A.grab = (int)std::max<int64_t>(
+      1, std::min<int64_t>(kMaxGrab, (A.ncells >> 5) / ((int64_t)sms * kBlocksPerSm * kWarps * 8)));
   if (quads) k_ipm_cells<true><<<g, kIpmThreads, 0, s>>>(A);
   else if (A.cell_list) k_ipm_cells<false, true><<<g, kIpmThreads, 0, s>>>(A);
   else k_ipm_cells<false><<<g, kIpmThreads, 0, s>>>(A);
