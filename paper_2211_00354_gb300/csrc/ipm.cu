@@ -41,6 +41,14 @@ constexpr int kBlocksPerSm = 4;
 
 constexpr int kWarps = kIpmThreads / 32;
 
+// c / nx for a cell id c < 2^30: with L = ceil(log2 nx) and M = floor(2^(30+L)
+// / nx) + 1 < 2^32, M nx - 2^(30+L) <= nx <= 2^L, so c M / 2^(30+L) exceeds c / nx by
+// less than 1 / nx and the floors agree (a 32-bit division takes ~20 instructions
+// of the ~350 that a round of single-pixel cells has).
+__device__ __forceinline__ int64_t cell_row(const IpmArgs& A, uint32_t c) {
+  return (int64_t)(((uint64_t)c * A.div_m) >> A.div_s);
+}
+
 // One warp per round of 32 cells of a grid chunk (or of a cell list, or of
 // sub-cells given as four corners each), rounds handed out by a counter.
 template <bool QUADS, bool LIST = false>
@@ -71,13 +79,12 @@ __global__ void __launch_bounds__(kIpmThreads, kBlocksPerSm) k_ipm_cells(IpmArgs
 #pragma unroll
         for (int k = 0; k < 4; ++k) q4[k] = A.yc[4 * c + k];
       } else {
-        // cell index < 2^30 and nx < 2^31: 32-bit division
-        const uint32_t j32 = (uint32_t)c / (uint32_t)A.nx;
-        const int64_t j = j32, i = c - j * A.nx;
-        q4[0] = A.yc[j * W + i];
-        q4[1] = A.yc[j * W + i + 1];
-        q4[2] = A.yc[(j + 1) * W + i + 1];
-        q4[3] = A.yc[(j + 1) * W + i];
+        const int64_t j = cell_row(A, (uint32_t)c);
+        const PixCorner* y0 = A.yc + (c + j);  // j W + i = c + j
+        q4[0] = y0[0];
+        q4[1] = y0[1];
+        q4[2] = y0[W + 1];
+        q4[3] = y0[W];
       }
     }
     ipm_round<false>(A, sh[w], lane, has, c, q4, led);
@@ -108,13 +115,12 @@ __global__ void __launch_bounds__(kIpmThreads) k_ipm_ext(IpmArgs A) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) q4[k] = A.yc[4 * c + k];
     } else {
-      const uint32_t j32 = (uint32_t)c / (uint32_t)A.nx;
-      const int64_t j = j32, i = c - j * A.nx;
-      const int64_t W = A.nx + 1;
-      q4[0] = A.yc[j * W + i];
-      q4[1] = A.yc[j * W + i + 1];
-      q4[2] = A.yc[(j + 1) * W + i + 1];
-      q4[3] = A.yc[(j + 1) * W + i];
+      const int64_t j = cell_row(A, (uint32_t)c), W = A.nx + 1;
+      const PixCorner* y0 = A.yc + (c + j);
+      q4[0] = y0[0];
+      q4[1] = y0[1];
+      q4[2] = y0[W + 1];
+      q4[3] = y0[W];
     }
     ext_cell(A, q4, cut_x[w], cut_y[w], lane, led);
   }
@@ -154,6 +160,10 @@ void ipm_launch(IpmArgs& A, bool quads, int* qcount, cudaStream_t s,
   LENS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t chunk_blocks = (A.ncells + kIpmThreads - 1) / kIpmThreads;
   const unsigned g = (unsigned)std::min<int64_t>(chunk_blocks, (int64_t)sms * 8);
+  int L = 0;
+  while ((1ll << L) < A.nx) ++L;
+  A.div_s = 30 + L;
+  A.div_m = A.nx > 0 ? (uint32_t)((1ull << A.div_s) / (uint64_t)A.nx + 1) : 0;
   A.grab = (int)std::max<int64_t>(
       1, std::min<int64_t>(kMaxGrab, (A.ncells >> 5) / ((int64_t)sms * kBlocksPerSm * kWarps * 8)));
   if (quads) k_ipm_cells<true><<<g, kIpmThreads, 0, s>>>(A);

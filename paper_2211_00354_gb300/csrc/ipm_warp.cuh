@@ -36,6 +36,7 @@ struct IpmArgs {
   float wcell;          // cell area in units of the grid's cell (1, or 4^-level for sub-cells)
   int* rq; int* rqcount;  // refinement: cells over the cap are queued here (NULL: dropped)
   int grab;               // k_ipm_cells: chunks of 32 cells per fetch of the chunk counter
+  uint32_t div_m; int div_s;  // c / nx as (c div_m) >> div_s for cell ids c < 2^30
   const int* cell_list;   // k_ipm_cells: the cells to map (ids into yc's grid), or NULL: all
 };
 
@@ -57,9 +58,7 @@ struct WarpCells {
   int4 box[32];           // ix0, iy0, cx0, cy0 (box clipped to the map at cx0, cy0)
   int2 ext[32];           // clipped box width (+ whole-box flag and height
                           // of a small cell), 1 / A_P (float bits)
-  int cum[32], cum2[32];
-  // owner lane of each (cell, pixel) task of the small cells (<= 32 x 16)
-  unsigned char own[32 * kSmallBox * kSmallBox];
+  int who[32], who2[32];  // rank among the lanes with tasks -> lane
   float4 seg[128];        // crossing segments: xa, xb, dy / 2, first pixel (int bits)
   int4 sst[32];           // starts of a row task's segments 1..3 in its pixel list
   int2 rbi[32];           // row task: map offset of (row, box x0), 1 / A_P (float bits)
@@ -188,31 +187,44 @@ __device__ __forceinline__ int winding4(const float* qx, const float* qy, float 
   return w;
 }
 
-// Inclusive warp scan of per-lane counts; cum[] receives the 32 inclusive
-// sums, the return value is the warp total.
-__device__ __forceinline__ int warp_counts(int cnt, int* cum, int lane) {
-  int incl = cnt;
+// The warp's tasks, flattened: lane L brings cnt of them, at flat indices
+// start .. start + cnt - 1.  begin() scans the counts and lists the lanes
+// that have any; owner(f0, ...) gives lane i the owner of task f0 + i: the
+// starts that fall in the window f0 .. f0 + 31 are gathered into one word, so
+// an owner's rank is a population count and its lane one load (a binary
+// search over the counts took five dependent loads, a byte table up to
+// fifteen stores a lane).
+struct WarpTasks {
+  int cnt, start, total;
+  __device__ __forceinline__ void begin(int n, int* who, int lane) {
+    int incl = n;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    cnt = n;
+    start = incl - n;
+    const unsigned m = __ballot_sync(0xffffffffu, n > 0);
+    if (n > 0) who[__popc(m & ((1u << lane) - 1u))] = lane;
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    __syncwarp();
   }
-  cum[lane] = incl;
-  __syncwarp();
-  return __shfl_sync(0xffffffffu, incl, 31);
-}
-// Owner of flat task f: the first lane whose inclusive count exceeds f, and
-// f's offset within that lane's tasks.
-__device__ __forceinline__ int warp_owner(const int* cum, int f, int& off) {
-  int L = 0;
-#pragma unroll
-  for (int st = 16; st > 0; st >>= 1)
-    if (cum[L + st - 1] <= f) L += st;
-  off = f - (L ? cum[L - 1] : 0);
-  return L;
-}
+  // off: the task's index within its owner's (all lanes call; the result is
+  // meaningless for f0 + lane >= total)
+  __device__ __forceinline__ int owner(int f0, const int* who, int lane, int& off) const {
+    const unsigned rel = (unsigned)(start - f0);
+    const unsigned word = __reduce_or_sync(0xffffffffu, cnt > 0 && rel < 32u ? 1u << rel : 0u);
+    const int before = __popc(__ballot_sync(0xffffffffu, cnt > 0 && start < f0));
+    const int rank = before + __popc(word & (0xffffffffu >> (31 - lane))) - 1;
+    const int L = who[rank & 31];
+    off = f0 + lane - __shfl_sync(0xffffffffu, start, L);
+    return L;
+  }
+};
 
-
+__device__ __forceinline__ int min4(int a, int b, int c, int d) { return __vimin3_s32(a, b, min(c, d)); }
+__device__ __forceinline__ int max4(int a, int b, int c, int d) { return __vimax3_s32(a, b, max(c, d)); }
 
 __device__ __forceinline__ void unpack4(float (&a)[4], const float4 v) {
   a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
@@ -406,14 +418,11 @@ __device__ __forceinline__ void ipm_round(const IpmArgs& A, WarpCells& sh, int l
   int nsmall = 0, nrows = 0;
   bool f64 = false;
   if (has) {
-    bool far = false;
-    int ix0 = kFar, ix1 = -kFar, iy0 = kFar, iy1 = -kFar;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      far |= (q4[k].iu == kFar) | (q4[k].iv == kFar);
-      ix0 = min(ix0, q4[k].iu); ix1 = max(ix1, q4[k].iu);
-      iy0 = min(iy0, q4[k].iv); iy1 = max(iy1, q4[k].iv);
-    }
+    const int ix0 = min4(q4[0].iu, q4[1].iu, q4[2].iu, q4[3].iu);
+    const int ix1 = max4(q4[0].iu, q4[1].iu, q4[2].iu, q4[3].iu);
+    const int iy0 = min4(q4[0].iv, q4[1].iv, q4[2].iv, q4[3].iv);
+    const int iy1 = max4(q4[0].iv, q4[1].iv, q4[2].iv, q4[3].iv);
+    const bool far = ix1 == kFar || iy1 == kFar;
     if (!far && (ix1 < 0 || iy1 < 0 || ix0 > npx - 1 || iy0 > npy - 1)) {
       led.fout += 1.f;
     } else if (far || (A.ip.cap > 0 && ((int64_t)ix1 - ix0 + 1 > A.ip.cap ||
@@ -438,12 +447,10 @@ __device__ __forceinline__ void ipm_round(const IpmArgs& A, WarpCells& sh, int l
         f64 = true;
         led.nq += 1;
       } else if (ix0 == ix1 && iy0 == iy1) {
-        atomicAdd(&A.map[(int64_t)iy0 * npx + ix0], A.scale_f);
+        atomicAdd(&A.map[iy0 * npx + ix0], A.scale_f);  // npx * npy < 2^31
         led.fin += 1.f;
         led.nupd += 1;
       } else {
-        const int cx0 = max(ix0, 0), cx1 = min(ix1, npx - 1);
-        const int cy0 = max(iy0, 0), cy1 = min(iy1, npy - 1);
         float slk[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -452,33 +459,54 @@ __device__ __forceinline__ void ipm_round(const IpmArgs& A, WarpCells& sh, int l
           const float ey = qy[(k + 1) & 3] - qy[k];
           slk[k] = fabsf(ey) > 1e-30f ? __fdividef(qx[(k + 1) & 3] - qx[k], ey) : 0.f;
         }
-        sh.qx[lane] = make_float4(qx[0], qx[1], qx[2], qx[3]);
-        sh.qy[lane] = make_float4(qy[0], qy[1], qy[2], qy[3]);
-        sh.sl[lane] = make_float4(slk[0], slk[1], slk[2], slk[3]);
-        sh.box[lane] = make_int4(ix0, iy0, cx0, cy0);
-        const bool smallc = ix1 - ix0 < kSmallBox && iy1 - iy0 < kSmallBox;
-        // A small cell whose pixel box lies inside the map puts all of its
-        // area there: its fractions sum to 1 (winding-weighted areas add up
-        // to the signed area), so the last pixel of the box is not
-        // evaluated and takes 1 minus the others (added whole here, each
-        // other pixel's fraction subtracted from it in B).
-        const bool whole = smallc && cx0 == ix0 && cy0 == iy0 && cx1 == ix1 && cy1 == iy1;
         // |A_loc| > 0: the cell is well conditioned
-        sh.ext[lane] = make_int2((cx1 - cx0 + 1) | (whole ? (cy1 - cy0 + 1) << 3 : 0),
-                                    __float_as_int(frcp_fast(A_loc)));
-        if (whole) {
-          atomicAdd(&A.map[(int64_t)cy1 * npx + cx1], A.scale_f);
+        const float inv = frcp_fast(A_loc);
+        if ((unsigned)(ix1 - ix0) + (unsigned)(iy1 - iy0) == 1u && min(ix0, iy0) >= 0 && ix1 < npx &&
+            iy1 < npy) {
+          // two pixels side by side, both in the map: the whole-box cell of
+          // B with its one overlap taken here (most multi-pixel cells of a
+          // strongly compressed map are such: the list and staging of B cost
+          // about as much as the overlap)
+          float* last = A.map + (iy1 * npx + ix1);
+          atomicAdd(last, A.scale_f);
           led.fin += 1.f;
           led.nupd += 1;
+          const float fr = pixel_area_f(qx, qy, slk, 0.f, 0.f) * inv;
+          if (fr != 0.f) {
+            atomicAdd(&A.map[iy0 * npx + ix0], A.scale_f * fr);
+            atomicAdd(last, -A.scale_f * fr);
+            led.nupd += 1;
+          }
         } else {
-          // every fraction that lands in the map is moved from fout to fin
-          led.fout += 1.f;
-        }
-        if (smallc) {
-          nsmall = (cx1 - cx0 + 1) * (cy1 - cy0 + 1) - (whole ? 1 : 0);
-        } else {
-          nrows = cy1 - cy0 + 1;
-          led.nq += 1;
+          const int cx0 = max(ix0, 0), cx1 = min(ix1, npx - 1);
+          const int cy0 = max(iy0, 0), cy1 = min(iy1, npy - 1);
+          sh.qx[lane] = make_float4(qx[0], qx[1], qx[2], qx[3]);
+          sh.qy[lane] = make_float4(qy[0], qy[1], qy[2], qy[3]);
+          sh.sl[lane] = make_float4(slk[0], slk[1], slk[2], slk[3]);
+          sh.box[lane] = make_int4(ix0, iy0, cx0, cy0);
+          const bool smallc = ix1 - ix0 < kSmallBox && iy1 - iy0 < kSmallBox;
+          // A small cell whose pixel box lies inside the map puts all of its
+          // area there: its fractions sum to 1 (winding-weighted areas add up
+          // to the signed area), so the last pixel of the box is not
+          // evaluated and takes 1 minus the others (added whole here, each
+          // other pixel's fraction subtracted from it in B).
+          const bool whole = smallc && cx0 == ix0 && cy0 == iy0 && cx1 == ix1 && cy1 == iy1;
+          sh.ext[lane] = make_int2((cx1 - cx0 + 1) | (whole ? (cy1 - cy0 + 1) << 3 : 0),
+                                   __float_as_int(inv));
+          if (whole) {
+            atomicAdd(&A.map[cy1 * npx + cx1], A.scale_f);
+            led.fin += 1.f;
+            led.nupd += 1;
+          } else {
+            // every fraction that lands in the map is moved from fout to fin
+            led.fout += 1.f;
+          }
+          if (smallc) {
+            nsmall = (cx1 - cx0 + 1) * (cy1 - cy0 + 1) - (whole ? 1 : 0);
+          } else {
+            nrows = cy1 - cy0 + 1;
+            led.nq += 1;
+          }
         }
       }
     }
@@ -508,19 +536,12 @@ __device__ __forceinline__ void ipm_round(const IpmArgs& A, WarpCells& sh, int l
   }
   // ---- B: pixels of small cells (skipped by a round without any) ----------
   if (__any_sync(0xffffffffu, nsmall > 0)) {
-    const int tot1 = warp_counts(nsmall, sh.cum, lane);
-    {
-      // each lane marks its tasks with its index: one byte load finds a
-      // task's cell
-      const int st = sh.cum[lane] - nsmall;
-      for (int i = 0; i < nsmall; ++i) sh.own[st + i] = (unsigned char)lane;
-      __syncwarp();
-    }
-    for (int f0 = 0; f0 < tot1; f0 += 32) {
-      const int f = f0 + lane;
-      if (f < tot1) {
-        const int L = sh.own[f];
-        const int off = f - (L ? sh.cum[L - 1] : 0);
+    WarpTasks T;
+    T.begin(nsmall, sh.who, lane);
+    for (int f0 = 0; f0 < T.total; f0 += 32) {
+      int off;
+      const int L = T.owner(f0, sh.who, lane, off);
+      if (f0 + lane < T.total) {
         const int4 bx = sh.box[L];
         const int2 ex = sh.ext[L];
         const int wd = ex.x & 7, hg = ex.x >> 3;  // hg > 0: a whole-box cell of hg rows
@@ -550,13 +571,13 @@ __device__ __forceinline__ void ipm_round(const IpmArgs& A, WarpCells& sh, int l
   }
   // ---- C: rows of large cells (skipped by a round without any) -------------
   if (!__any_sync(0xffffffffu, nrows > 0)) return;
-  const int tot2 = warp_counts(nrows, sh.cum2, lane);
-  for (int f0 = 0; f0 < tot2; f0 += 32) {
-    const int f = f0 + lane;
-    int cnt = 0;
-    if (f < tot2) {
-      int r;
-      const int L = warp_owner(sh.cum2, f, r);
+  WarpTasks R;
+  __syncwarp();  // B is done with the task list
+  R.begin(nrows, sh.who, lane);
+  for (int f0 = 0; f0 < R.total; f0 += 32) {
+    int cnt = 0, r;
+    const int L = R.owner(f0, sh.who, lane, r);
+    if (f0 + lane < R.total) {
       const int4 bx = sh.box[L];
       const int2 ex = sh.ext[L];
       const int ix0 = bx.x, cx0 = bx.z;
@@ -612,14 +633,12 @@ __device__ __forceinline__ void ipm_round(const IpmArgs& A, WarpCells& sh, int l
       sh.rbi[lane] = make_int2(py * npx + ix0, __float_as_int(inv));
     }
     // crossed pixels of these 32 rows, spread over the lanes
-    int* cum = sh.cum;  // the small-cell counts are no longer needed
-    __syncwarp();
-    const int totp = warp_counts(cnt, cum, lane);
-    for (int g0 = 0; g0 < totp; g0 += 32) {
-      const int g = g0 + lane;
-      if (g < totp) {
-        int off;
-        const int L = warp_owner(cum, g, off);
+    WarpTasks X;
+    X.begin(cnt, sh.who2, lane);
+    for (int g0 = 0; g0 < X.total; g0 += 32) {
+      int off;
+      const int L = X.owner(g0, sh.who2, lane, off);
+      if (g0 + lane < X.total) {
         // segment k of row task L: the last one starting at or before off
         // (an empty segment shares its start with the next one)
         const int4 ss = sh.sst[L];
