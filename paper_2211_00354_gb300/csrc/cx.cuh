@@ -90,6 +90,17 @@ struct fcomp2 {
     hi = s;
     lo = __fadd2_rn(lo, e);
   }
+  // the same sum by Knuth's two-sum: six paired operations and no compares or
+  // selects, for loops whose issue slots are scarcer than the FMA pipe's cycles
+  __device__ __forceinline__ void add_knuth(float2 x) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 s = __fadd2_rn(hi, x);
+    const float2 b = __ffma2_rn(hi, m1, s);                      // s - hi
+    const float2 a = __ffma2_rn(b, m1, s);                       // s - b
+    const float2 e = __fadd2_rn(__ffma2_rn(a, m1, hi), __ffma2_rn(b, m1, x));
+    hi = s;
+    lo = __fadd2_rn(lo, e);
+  }
 };
 
 // Spread the low 32 bits of x to the even bit positions of a 64-bit word.

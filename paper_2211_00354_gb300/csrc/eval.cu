@@ -302,8 +302,8 @@ __global__ void k_grid_rects(const int* __restrict__ leaves, int64_t nleaf,
                              const int* __restrict__ level, const int* __restrict__ ix,
                              const int* __restrict__ iy, double lo_x, double lo_y, double size,
                              double x0, double y0, double h, int64_t nx, int64_t row0,
-                             int64_t nrows, int tile, int64_t* __restrict__ rect,
-                             int64_t* __restrict__ tiles) {
+                             int64_t nrows, int tile, bool quads,
+                             int64_t* __restrict__ rect, int64_t* __restrict__ tiles) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= nleaf) return;
   const int B = leaves[k];
@@ -316,7 +316,9 @@ __global__ void k_grid_rects(const int* __restrict__ leaves, int64_t nleaf,
   const int64_t j1 = first_at_or_above(y0, h, row0, row0 + nrows, by1);
   const int64_t ni = i1 > i0 ? i1 - i0 : 0, nj = j1 > j0 ? j1 - j0 : 0;
   rect[4 * k] = i0; rect[4 * k + 1] = ni; rect[4 * k + 2] = j0; rect[4 * k + 3] = nj;
-  tiles[k] = (ni * nj + tile - 1) / tile;
+  // rays, or 2 x 2 blocks of them
+  const int64_t units = quads ? ((ni + 1) >> 1) * ((nj + 1) >> 1) : ni * nj;
+  tiles[k] = (units + tile - 1) / tile;
 }
 
 // algorithmic work of one grid band: rays, ray-star pairs, ray-box M2P evals.
@@ -476,14 +478,16 @@ void grid_impl(Plan& P, const GridRows& g, double* y, double* jac, PixCorner* pi
                const IpmParams* ip, cudaStream_t s) {
   const int64_t nl = P.n_active_leaves;
   if (nl == 0 || g.nrows <= 0) return;
-  const int tile = tile_rays(P);
+  // the float32 form without a Jacobian takes its rays in 2 x 2 blocks
+  const bool quads = P.prec == LENS_FP32_BULK && !jac;
+  const int tile = quads ? kEval32Threads : tile_rays(P);
   Scratch rect(&P.da, sizeof(int64_t) * 4 * nl);
   Scratch tiles(&P.da, sizeof(int64_t) * (nl + 1));
   Scratch toff(&P.da, sizeof(int64_t) * (nl + 1));
   k_grid_rects<<<grid_for(nl, 128), 128, 0, s>>>(P.active_leaves, nl, P.box_level, P.box_ix,
                                                  P.box_iy, P.root_lo[0], P.root_lo[1],
                                                  P.root_size, g.x0, g.y0, g.h, g.nx, g.row0,
-                                                 g.nrows, tile, rect.as<int64_t>(),
+                                                 g.nrows, tile, quads, rect.as<int64_t>(),
                                                  tiles.as<int64_t>());
   LENS_LAUNCHED("k_grid_rects");
   LENS_CUDA(cudaMemsetAsync(tiles.as<int64_t>() + nl, 0, sizeof(int64_t), s));
@@ -535,7 +539,7 @@ void evaluate_grid_fused(Plan& P, const GridRows& g, PixCorner* edge, const IpmP
   k_grid_rects<<<grid_for(nl, 128), 128, 0, s>>>(P.active_leaves, nl, P.box_level, P.box_ix,
                                                  P.box_iy, P.root_lo[0], P.root_lo[1],
                                                  P.root_size, g.x0, g.y0, g.h, g.nx, g.row0,
-                                                 g.nrows, tile_rays(P), rect.as<int64_t>(),
+                                                 g.nrows, tile_rays(P), false, rect.as<int64_t>(),
                                                  tiles.as<int64_t>());
   LENS_LAUNCHED("k_grid_rects");
   if (P.work) {

@@ -311,7 +311,8 @@ __device__ __forceinline__ void grid_offset(const E32Args& A, const LeafGrid& lg
   dy = oy.hi; dyl = oy.lo;
 }
 
-template <bool JAC, bool GRID, bool PIX, bool UM = false>
+// Arbitrary rays, and grid rays with the Jacobian (without it: k_eval_quads).
+template <bool JAC, bool GRID, bool UM = false>
 __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
   __shared__ E32Smem sm;
   const int tid = threadIdx.x;
@@ -332,10 +333,8 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
   } else {
     nr_leaf = A.ray_off[k + 1] - A.ray_off[k];
   }
-  // the grid path without the Jacobian sums its near field in grid units
-  constexpr bool GU = GRID && !JAC;
+  static_assert(JAC || !GRID, "grid rays without the Jacobian run k_eval_quads");
   float dx[kRpt], dy[kRpt], dxl[kRpt], dyl[kRpt];
-  float gxr[kRpt], gyr[kRpt];  // GU: the rays' integer grid coordinates from the leaf's origin
   int64_t oidx[kRpt];
   bool ok[kRpt];
   fcomp n1[kRpt], n2[kRpt], nj1[kRpt], nj2[kRpt];
@@ -358,7 +357,6 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
     const int64_t loc = tbase + (int64_t)q * S + tid;
     ok[q] = tid < S && loc < nr_leaf;
     dx[q] = dy[q] = dxl[q] = dyl[q] = 0.f;
-    gxr[q] = gyr[q] = 0.f;
     oidx[q] = 0;
     n1[q] = {0.f, 0.f}; n2[q] = {0.f, 0.f}; nj1[q] = {0.f, 0.f}; nj2[q] = {0.f, 0.f};
     if (!ok[q]) continue;
@@ -368,8 +366,6 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
       const uint32_t dj = l32 / n32, di = l32 - dj * n32;
       oidx[q] = (j0 + (int64_t)dj - A.grow0) * A.gnx1 + i0 + (int64_t)di;
       grid_offset(A, lg, di, dj, dx[q], dxl[q], dy[q], dyl[q]);
-      gxr[q] = (float)(lg.ri + (int)di);
-      gyr[q] = (float)(lg.rj + (int)dj);
     } else {
       const int64_t ridx = A.perm[A.ray_off[k] + loc];
       oidx[q] = ridx;
@@ -390,12 +386,10 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
     const int nf = (int)min64(kChunk, nstar - f0);
     const int nfg = (nf + kGroup - 1) / kGroup * kGroup;
     __syncthreads();
-    stage_stars<GU>(sm, A, star0 + f0, nf, nfg, tid, lg.rx, lg.ry);
+    stage_stars<false>(sm, A, star0 + f0, nf, nfg, tid);
     __syncthreads();
     if (!live) continue;  // uniform over the warp; the barriers are above
-    if constexpr (GU) {
-      p2p_paired<UM, true>(sm, nfg, gxr, gyr, dxl, dyl, N1, N2);
-    } else if (!JAC) {
+    if constexpr (!JAC) {
       p2p_paired<UM>(sm, nfg, dx, dy, dxl, dyl, N1, N2);
     } else {
       for (int lo = 0; lo < nfg; lo += kGroup) {
@@ -488,22 +482,15 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
 #pragma unroll
     for (int h = 0; h < kRpt / 2; ++h) {
       ff2 T1, T2;
-      l2p_lens_pair<GU>(sm, A, ir, h, dx, dy, dxl, dyl, N1[h], N2[h], FX[h], FY[h], T1, T2);
-      if (PIX) {
-        PixCorner pc[2];
-        pix_pair(A, lg, T1, T2, pc);
-        if (ok[2 * h]) A.pix[oidx[2 * h]] = pc[0];
-        if (ok[2 * h + 1]) A.pix[oidx[2 * h + 1]] = pc[1];
-      } else {
+      l2p_lens_pair<false>(sm, A, ir, h, dx, dy, dxl, dyl, N1[h], N2[h], FX[h], FY[h], T1, T2);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int q = 2 * h + c;
-          if (!ok[q]) continue;
-          const ff t1 = c ? ff{T1.hi.y, T1.lo.y} : ff{T1.hi.x, T1.lo.x};
-          const ff t2 = c ? ff{T2.hi.y, T2.lo.y} : ff{T2.hi.x, T2.lo.x};
-          A.y[2 * oidx[q]] = lp.K1 + ff_to_double(t1);
-          A.y[2 * oidx[q] + 1] = lp.K2 + ff_to_double(t2);
-        }
+      for (int c = 0; c < 2; ++c) {
+        const int q = 2 * h + c;
+        if (!ok[q]) continue;
+        const ff t1 = c ? ff{T1.hi.y, T1.lo.y} : ff{T1.hi.x, T1.lo.x};
+        const ff t2 = c ? ff{T2.hi.y, T2.lo.y} : ff{T2.hi.x, T2.lo.x};
+        A.y[2 * oidx[q]] = lp.K1 + ff_to_double(t1);
+        A.y[2 * oidx[q] + 1] = lp.K2 + ff_to_double(t2);
       }
     }
   } else {
@@ -529,37 +516,240 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
       ff T2 = ff_mul(A.bf, ff{dy[q], dyl[q]});
       T2 = ff_add(T2, f.y);
       T2 = ff_add(T2, ff{-n2[q].hi, -n2[q].lo});
-      if (PIX) {
-        PixCorner pc;
-        const ff U = ff_add(lg.U1f, ff_mul(A.iduf, T1));
-        const ff V = ff_add(lg.V1f, ff_mul(A.idvf, T2));
-        bool far = lg.far || !(fabsf(U.hi) < 5.0e8f) || !(fabsf(V.hi) < 5.0e8f);
-        float ku = floorf(U.hi), kv = floorf(V.hi);
-        float fu = (U.hi - ku) + U.lo, fv = (V.hi - kv) + V.lo;
-        if (fu < 0.f) { ku -= 1.f; fu += 1.f; } else if (fu >= 1.f) { ku += 1.f; fu -= 1.f; }
-        if (fv < 0.f) { kv -= 1.f; fv += 1.f; } else if (fv >= 1.f) { kv += 1.f; fv -= 1.f; }
-        // float -> int32 (|k| < 5e8); integer adds only afterwards
-        const int64_t iu = (int64_t)lg.U1i + (int)ku, iv = (int64_t)lg.V1i + (int)kv;
-        far = far || !(iu > -1073741824ll && iu < 1073741824ll && iv > -1073741824ll &&
-                       iv < 1073741824ll);
-        if (!far) {
-          pc.iu = (int)iu; pc.fu = fu; pc.iv = (int)iv; pc.fv = fv;
-        } else {
-          pc.iu = 0x7fffffff; pc.fu = 0.f; pc.iv = 0x7fffffff; pc.fv = 0.f;
-        }
-        A.pix[oidx[q]] = pc;
-        continue;
-      }
       A.y[2 * oidx[q]] = lp.K1 + ff_to_double(T1);
       A.y[2 * oidx[q] + 1] = lp.K2 + ff_to_double(T2);
-      if (JAC) {
-        const double dre = (double)df.x + (double)dfw[q].x + nj1[q].value();
-        const double dim = (double)df.y + (double)dfw[q].y + nj2[q].value();
-        A.jac[4 * oidx[q] + 0] = A.a - dre;
-        A.jac[4 * oidx[q] + 1] = dim;
-        A.jac[4 * oidx[q] + 2] = dim;
-        A.jac[4 * oidx[q] + 3] = A.b + dre;
+      const double dre = (double)df.x + (double)dfw[q].x + nj1[q].value();
+      const double dim = (double)df.y + (double)dfw[q].y + nj2[q].value();
+      A.jac[4 * oidx[q] + 0] = A.a - dre;
+      A.jac[4 * oidx[q] + 1] = dim;
+      A.jac[4 * oidx[q] + 2] = dim;
+      A.jac[4 * oidx[q] + 3] = A.b + dre;
+    }
+  }
+}
+
+// ---- grid rays, two columns by two rows a thread ----------------------------
+// The grid path without the Jacobian (maps, deflected grids), bound by the FMA
+// pipe and issue slots.  A thread takes a 2 x 2 block of a leaf's corner
+// rectangle: columns c and c + ceil(ni / 2) (so that a warp's stores stay
+// contiguous), rows 2 b and 2 b + 1, blocks numbered row by row.  Its four rays
+// share two column and two row coordinates: a star's differences and the
+// row's share of |d|^2 are formed once per pair of columns or rows, 11 paired
+// operations per star and four rays instead of 16, the offsets and the smooth
+// field's products likewise, and a coefficient is loaded once for both rows.
+// Every ray's operations and their order are those of the one-ray-per-slot form
+// (p2p_paired, l2p_lens_pair), so its bits are the same.  Four rays a slot apart
+// against this: high-magnification map 3187 -> 2515 us, clustered map 3810 -> 3180
+// us, 4096^2 halo grid 5293 -> 4115 us.  Not kept: blocks of 64 threads (halo 4620
+// us: the two idle warps of a leaf of ~50 blocks share the staging), several
+// tiles a block with the stars staged once (2450 us, but halo 4410 us).
+constexpr int kQChunk = 256;  // stars staged at a time
+constexpr int kQW = 4;        // far W boxes staged at a time
+static_assert(kQChunk % kGroup == 0, "chunks hold whole groups");
+
+template <bool UM>
+struct QuadSmem {
+  float4 hi[kQChunk], lo[kQChunk];  // -x, -x, -y, -y (grid units): high and low parts
+  float2 m[UM ? 1 : kQChunk];
+  float4 L[kMaxOrder + 1];          // re, re, im, im
+  float4 W[kQW][kMaxOrder + 1];
+  float4 wg[kQW];
+};
+
+template <bool PIX, bool UM>
+__global__ void __launch_bounds__(kT, 7) k_eval_quads(E32Args A) {
+  __shared__ QuadSmem<UM> sm;
+  const int tid = threadIdx.x, p = A.p;
+  const int2 kt = A.tile_leaf[blockIdx.x];
+  const int64_t k = kt.x;
+  for (int l = tid; l <= p; l += kT) {
+    const float2 c = A.fL[k * (int64_t)(p + 1) + l];
+    sm.L[l] = make_float4(c.x, c.x, c.y, c.y);
+  }
+  const LeafGrid lg = A.lgrid[k];
+  const int64_t i0 = A.rect[4 * k], j0 = A.rect[4 * k + 2];
+  const uint32_t ni = (uint32_t)A.rect[4 * k + 1], nj = (uint32_t)A.rect[4 * k + 3];
+  const uint32_t half = (ni + 1) >> 1;
+  const uint32_t nu = half * ((nj + 1) >> 1);  // units of the leaf
+  const int64_t star0 = A.uoff[k];
+  const int nstar = (int)(A.uoff[k + 1] - star0);
+  const int64_t w_beg = A.woff[k], w_end = A.woff[k + 1];
+  const LeafPlan* lp = A.leaf + k;
+  const float ir = lp->ir;
+  const uint32_t u = (uint32_t)kt.y * kT + tid;
+  const bool live = (u & ~31u) < nu;  // uniform over the warp
+  const uint32_t b = u / half, c = u - b * half;
+  const uint32_t di0 = c, di1 = c + half, dj0 = 2 * b, dj1 = 2 * b + 1;
+  const float2 GX = make_float2((float)(lg.ri + (int)di0), (float)(lg.ri + (int)di1));
+  const float2 GY = make_float2((float)(lg.rj + (int)dj0), (float)(lg.rj + (int)dj1));
+  fcomp2 N1[2], N2[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    N1[h] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    N2[h] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  }
+  for (int f0 = 0; f0 < nstar; f0 += kQChunk) {
+    const int nf = min(kQChunk, nstar - f0);
+    const int nfg = (nf + kGroup - 1) / kGroup * kGroup;
+    __syncthreads();
+    for (int f = tid; f < nfg; f += kT) {
+      float4 v = make_float4(1e18f, 0.f, 0.f, 0.f);
+      float mm = 0.f;
+      if (f < nf) {
+        v = A.ust[star0 + f0 + f];
+        if (!UM) mm = A.um[star0 + f0 + f];
       }
+      const ff gx = ff_mul(ff_add(ff{v.x, v.z}, ff_neg(lg.rx)), A.ihf);
+      const ff gy = ff_mul(ff_add(ff{v.y, v.w}, ff_neg(lg.ry)), A.ihf);
+      sm.hi[f] = make_float4(-gx.hi, -gx.hi, -gy.hi, -gy.hi);
+      sm.lo[f] = make_float4(-gx.lo, -gx.lo, -gy.lo, -gy.lo);
+      if (!UM) sm.m[f] = make_float2(mm, mm);
+    }
+    __syncthreads();
+    if (!live) continue;
+    for (int lo = 0; lo < nfg; lo += kGroup) {
+      float2 P1[2], P2[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) { P1[h] = make_float2(0.f, 0.f); P2[h] = make_float2(0.f, 0.f); }
+      const float2 tiny = make_float2(1e-30f, 1e-30f);
+#pragma unroll
+      for (int jj = 0; jj < kGroup; ++jj) {
+        const float4 h4 = sm.hi[lo + jj], l4 = sm.lo[lo + jj];
+        const float2 nx = make_float2(h4.x, h4.y), ny = make_float2(h4.z, h4.w);
+        const float2 nxl = make_float2(l4.x, l4.y), nyl = make_float2(l4.z, l4.w);
+        const float2 d1 = __fadd2_rn(__fadd2_rn(GX, nx), nxl);
+        const float2 d2 = __fadd2_rn(__fadd2_rn(GY, ny), nyl);
+        const float2 q = __ffma2_rn(d2, d2, tiny);
+        const float2 d2r[2] = {make_float2(d2.x, d2.x), make_float2(d2.y, d2.y)};
+        const float2 qr[2] = {make_float2(q.x, q.x), make_float2(q.y, q.y)};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 r2 = __ffma2_rn(d1, d1, qr[h]);
+          const float2 rr = make_float2(frcp_fast(r2.x), frcp_fast(r2.y));
+          const float2 w = UM ? rr : __fmul2_rn(sm.m[lo + jj], rr);
+          P1[h] = __ffma2_rn(w, d1, P1[h]);
+          P2[h] = __ffma2_rn(w, d2r[h], P2[h]);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) { N1[h].add_knuth(P1[h]); N2[h].add_knuth(P2[h]); }
+    }
+  }
+  if (UM && A.m0 != 1.f) {
+    const float2 m2 = make_float2(A.m0, A.m0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      N1[h].hi = __fmul2_rn(N1[h].hi, m2); N1[h].lo = __fmul2_rn(N1[h].lo, m2);
+      N2[h].hi = __fmul2_rn(N2[h].hi, m2); N2[h].lo = __fmul2_rn(N2[h].lo, m2);
+    }
+  }
+  // the rays' offsets from the leaf centre
+  const ff ox0 = ff_add(lg.bx, ff_mul(A.hf, (float)(int)di0));
+  const ff ox1 = ff_add(lg.bx, ff_mul(A.hf, (float)(int)di1));
+  const ff oy[2] = {ff_add(lg.by, ff_mul(A.hf, (float)(int)dj0)),
+                    ff_add(lg.by, ff_mul(A.hf, (float)(int)dj1))};
+  const ff2 OX{make_float2(ox0.hi, ox1.hi), make_float2(ox0.lo, ox1.lo)};
+  // M2P over the far W boxes
+  float2 FX[2], FY[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) { FX[h] = make_float2(0.f, 0.f); FY[h] = make_float2(0.f, 0.f); }
+  for (int64_t e0 = w_beg; e0 < w_end; e0 += kQW) {
+    const int nw = (int)min64(kQW, w_end - e0);
+    __syncthreads();
+    for (int t = tid; t < nw * (p + 1); t += kT) {
+      const int w = t / (p + 1), kk = t - w * (p + 1);
+      const float2 cc = A.fM[(int64_t)A.wlist[e0 + w] * (p + 1) + kk];
+      sm.W[w][kk] = make_float4(cc.x, cc.x, cc.y, cc.y);
+    }
+    if (tid < nw) sm.wg[tid] = A.wgeo[e0 + tid];
+    __syncthreads();
+    if (!live) continue;
+    for (int w = 0; w < nw; ++w) {
+      const float4 gw = sm.wg[w];
+      const float2 gr = f2(gw.z), ngr = f2(-gw.z);
+      const float2 zx = __fadd2_rn(OX.hi, f2(-gw.x));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float2 zy = __fadd2_rn(f2(oy[h].hi), f2(-gw.y));
+        const float2 n2 = __ffma2_rn(zx, zx, __fmul2_rn(zy, zy));
+        const float2 d = make_float2(frcp_fast(n2.x), frcp_fast(n2.y));
+        const float2 ix = __fmul2_rn(zx, d);   // 1/z = (zx d, -zy d)
+        const float2 niy = __fmul2_rn(zy, d);  // -Im(1/z)
+        const float2 iy = make_float2(-niy.x, -niy.y);
+        const float2 qx = __fmul2_rn(ix, gr), qy = __fmul2_rn(iy, gr);
+        const float2 nqy = __fmul2_rn(iy, ngr);
+        float2 sx = make_float2(sm.W[w][p].x, sm.W[w][p].y), sy = make_float2(sm.W[w][p].z, sm.W[w][p].w);
+        for (int kk = p - 1; kk >= 0; --kk) {
+          const float4 cc = sm.W[w][kk];
+          const float2 tx = __ffma2_rn(sy, nqy, make_float2(cc.x, cc.y));
+          const float2 ty = __ffma2_rn(sy, qx, make_float2(cc.z, cc.w));
+          const float2 nsx = __ffma2_rn(sx, qx, tx);
+          sy = __ffma2_rn(sx, qy, ty);
+          sx = nsx;
+        }
+        FX[h] = __ffma2_rn(sx, ix, __ffma2_rn(sy, niy, FX[h]));
+        FY[h] = __ffma2_rn(sx, iy, __ffma2_rn(sy, ix, FY[h]));
+      }
+    }
+  }
+  __syncthreads();  // the local coefficients, where no star or W box was staged
+  if (!live) return;  // no barrier follows
+  // L2P by Horner's rule, both rows at a time (one load of a coefficient)
+  const float2 wx = __fmul2_rn(OX.hi, f2(ir));
+  float2 fx[2], fy[2];
+  {
+    float2 wy[2], nwy[2], sx[2], sy[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      wy[h] = f2(oy[h].hi * ir);
+      nwy[h] = f2(oy[h].hi * -ir);
+      fx[h] = fy[h] = make_float2(0.f, 0.f);
+      sx[h] = make_float2(sm.L[p].x, sm.L[p].y);
+      sy[h] = make_float2(sm.L[p].z, sm.L[p].w);
+    }
+    if (p >= 1) {
+      for (int l = p - 1; l >= 1; --l) {
+        const float4 cc = sm.L[l];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 tx = __ffma2_rn(sy[h], nwy[h], make_float2(cc.x, cc.y));
+          const float2 ty = __ffma2_rn(sy[h], wx, make_float2(cc.z, cc.w));
+          const float2 nsx = __ffma2_rn(sx[h], wx, tx);
+          sy[h] = __ffma2_rn(sx[h], wy[h], ty);
+          sx[h] = nsx;
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        fx[h] = __ffma2_rn(sx[h], wx, __fmul2_rn(sy[h], nwy[h]));
+        fy[h] = __ffma2_rn(sx[h], wy[h], __fmul2_rn(sy[h], wx));
+      }
+    }
+  }
+  // the lens equation, as l2p_lens_pair
+  const ff2 ax = ff2_mul(A.af, OX);
+  const bool okc[2] = {di0 < ni && u < nu, di1 < ni && u < nu};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float2 f1 = __fadd2_rn(fx[h], FX[h]), fi = __fadd2_rn(fy[h], FY[h]);
+    const ff by = ff_mul(A.bf, oy[h]);
+    ff2 T1 = ff2_sub(ax, f1);
+    T1 = ff2_sub(T1, ff2_mul(A.ihf, ff2{N1[h].hi, N1[h].lo}));
+    ff2 T2 = ff2_add(ff2{f2(by.hi), f2(by.lo)}, fi);
+    T2 = ff2_sub(T2, ff2_mul(A.ihf, ff2{N2[h].hi, N2[h].lo}));
+    const uint32_t dj = 2 * b + h;
+    if (dj >= nj) continue;
+    const int64_t o = (j0 + (int64_t)dj - A.grow0) * A.gnx1 + i0 + (int64_t)c;
+    if (PIX) {
+      PixCorner pc[2];
+      pix_pair(A, lg, T1, T2, pc);
+      if (okc[0]) A.pix[o] = pc[0];
+      if (okc[1]) A.pix[o + half] = pc[1];
+    } else {
+      double2* y = reinterpret_cast<double2*>(A.y);
+      const double K1 = lp->K1, K2 = lp->K2;
+      if (okc[0]) y[o] = make_double2(K1 + ff_to_double(ff{T1.hi.x, T1.lo.x}), K2 + ff_to_double(ff{T2.hi.x, T2.lo.x}));
+      if (okc[1]) y[o + half] = make_double2(K1 + ff_to_double(ff{T1.hi.y, T1.lo.y}), K2 + ff_to_double(ff{T2.hi.y, T2.lo.y}));
     }
   }
 }
@@ -963,15 +1153,33 @@ E32Args base_args32(Plan& P) {
   return A;
 }
 
-template <bool GRID, bool PIX>
-void launch32(E32Args& A, int64_t total, bool jac, cudaStream_t s) {
+void launch32_rays(E32Args& A, int64_t total, bool jac, cudaStream_t s) {
   if (total <= 0) return;
   if (total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
   const unsigned g = (unsigned)total;
-  if (jac) k_eval32<true, GRID, PIX><<<g, kT, 0, s>>>(A);
-  else if (A.unit_mass) k_eval32<false, GRID, PIX, true><<<g, kT, 0, s>>>(A);
-  else k_eval32<false, GRID, PIX><<<g, kT, 0, s>>>(A);
+  if (jac) k_eval32<true, false><<<g, kT, 0, s>>>(A);
+  else if (A.unit_mass) k_eval32<false, false, true><<<g, kT, 0, s>>>(A);
+  else k_eval32<false, false><<<g, kT, 0, s>>>(A);
   LENS_LAUNCHED("k_eval32");
+}
+
+void launch32_grid(E32Args& A, int64_t total, cudaStream_t s) {
+  if (total <= 0) return;
+  if (total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
+  const unsigned g = (unsigned)total;
+  if (A.jac) {
+    k_eval32<true, true><<<g, kT, 0, s>>>(A);
+    LENS_LAUNCHED("k_eval32");
+    return;
+  }
+  if (A.pix) {
+    if (A.unit_mass) k_eval_quads<true, true><<<g, kT, 0, s>>>(A);
+    else k_eval_quads<true, false><<<g, kT, 0, s>>>(A);
+  } else {
+    if (A.unit_mass) k_eval_quads<false, true><<<g, kT, 0, s>>>(A);
+    else k_eval_quads<false, false><<<g, kT, 0, s>>>(A);
+  }
+  LENS_LAUNCHED("k_eval_quads");
 }
 
 }  // namespace
@@ -1063,8 +1271,7 @@ void eval32_grid(Plan& P, const GridRows& g, const int64_t* rect, const int2* ti
   // kernel time only: the events follow the wait for the plan's expansions
   std::pair<cudaEvent_t, cudaEvent_t> e;
   if (P.timing) e = event_pair_begin(s);
-  if (px) launch32<true, true>(A, total, false, s);
-  else launch32<true, false>(A, total, jac != nullptr, s);
+  launch32_grid(A, total, s);
   if (P.timing) {
     event_pair_end(e, s);
     P.ev_eval.push_back(e);
@@ -1138,7 +1345,7 @@ void eval32_rays(Plan& P, const double* rays, const int64_t* off, const int* per
   A.tile_leaf = tile_leaf;
   A.rays = rays; A.ray_off = off; A.perm = perm;
   A.y = y; A.jac = jac;
-  launch32<false, false>(A, total, jac != nullptr, s);
+  launch32_rays(A, total, jac != nullptr, s);
 }
 
 }  // namespace lens
