@@ -130,13 +130,51 @@ __global__ void __launch_bounds__(32) k_adj_leaf_moments(AdjArgs A) {
   }
 }
 
-// P2P^T: threads over the U-list stars of the tile's leaf, rays of the tile
-// staged in shared memory.
+// The stars of a leaf's U list, flattened over the block's threads (a leaf's own
+// count is often below the block size): up to kAdjU leaves at a time, their first
+// star and inclusive star counts in shared memory.  f(sj) is called for every
+// star of the list, one thread each.
+struct UStage {
+  int start[kAdjU], incl[kAdjU];
+};
+template <typename F>
+__device__ __forceinline__ void for_u_stars(const AdjArgs& A, int a, UStage& su, F f) {
+  const int64_t u0 = A.U_off[a], nu = A.U_off[a + 1] - u0;
+  for (int64_t ub = 0; ub < nu; ub += kAdjU) {
+    const int nub = (int)min64(kAdjU, nu - ub);
+    __syncthreads();  // the previous group's readers are done (and the caller's staging)
+    if (threadIdx.x < nub) {
+      const int C = A.U_list[u0 + ub + threadIdx.x];
+      su.start[threadIdx.x] = A.start[C];
+      su.incl[threadIdx.x] = A.count[C];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int i = 1; i < nub; ++i) su.incl[i] += su.incl[i - 1];
+    __syncthreads();
+    const int tot = su.incl[nub - 1];
+    for (int q = threadIdx.x; q < tot; q += blockDim.x) {
+      // the group's leaf holding flattened star q: the first with incl > q
+      int lo = 0, hi = nub - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (su.incl[mid] > q) hi = mid; else lo = mid + 1;
+      }
+      f(su.start[lo] + q - (lo ? su.incl[lo - 1] : 0));
+    }
+  }
+}
+
+// P2P^T in float64: threads over the U-list stars of the tile's leaf, the tile's
+// rays staged in shared memory.  Bound by the float64 pipe: 21 operations a pair
+// (with a division and comparisons with 0 on that pipe, ~30), a warp
+// instruction for up to 32 stars (one leaf at a time, ~11).  1.26e5 rays, 2e4
+// stars, leaves of 16: 1781 -> 306 us.
 __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
   __shared__ double2 sz[kAdjTile], sc[kAdjTile];
+  __shared__ UStage su;
   const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
-  const int B = A.leaves[k];
-  const int a = A.aidx[B];
+  const int a = A.aidx[A.leaves[k]];
   const int64_t tile = (int64_t)blockIdx.x - A.tile_off[k];
   const int64_t n = A.ray_off[k + 1] - A.ray_off[k];
   const int64_t r0 = tile * kAdjTile;
@@ -146,30 +184,22 @@ __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
     sz[t] = make_double2(A.rays[2 * ridx], A.rays[2 * ridx + 1]);
     sc[t] = make_double2(-A.gy[2 * ridx], -A.gy[2 * ridx + 1]);
   }
-  __syncthreads();
-  // flatten the U-list stars: walk entries, threads take stars in turn
-  int64_t base = 0;
-  for (int64_t e = A.U_off[a]; e < A.U_off[a + 1]; ++e) {
-    const int C = A.U_list[e];
-    const int s0 = A.start[C], ns = A.count[C];
-    for (int j = threadIdx.x; j < ns; j += blockDim.x) {
-      const int sj = s0 + j;
-      const double2 zj = A.spos[sj];
-      const double mj = A.smass[sj];
-      double2 F = make_double2(0, 0), G = make_double2(0, 0);
-      for (int t = 0; t < nr; ++t) {
-        const double2 d = make_double2(sz[t].x - zj.x, sz[t].y - zj.y);
-        if (d.x == 0.0 && d.y == 0.0) continue;  // self-interaction skipped
-        const double2 inv = cinv(d);
-        const double2 ci = cmul(sc[t], inv);
-        F = F + ci;
-        G = G + cmul(ci, inv);
-      }
-      atomic_add2(A.Phi + sj, F);
-      atomic_add2(A.Psi + sj, make_double2(mj * G.x, mj * G.y));
+  for_u_stars(A, a, su, [&](int sj) {
+    const double2 zj = A.spos[sj];
+    double2 F = make_double2(0, 0), G = make_double2(0, 0);
+#pragma unroll 2
+    for (int t = 0; t < nr; ++t) {
+      const double2 d = make_double2(sz[t].x - zj.x, sz[t].y - zj.y);
+      const double w = rcp_or_zero(d.x * d.x + d.y * d.y);  // 0: self-interaction skipped
+      const double2 inv = make_double2(d.x * w, -d.y * w);
+      const double2 ci = cmul(sc[t], inv);
+      F = F + ci;
+      G = cfma(ci, inv, G);
     }
-    base += ns;
-  }
+    const double mj = A.smass[sj];
+    atomic_add2(A.Phi + sj, F);
+    atomic_add2(A.Psi + sj, make_double2(mj * G.x, mj * G.y));
+  });
 }
 
 // ---- float32 bulk (plans of precision LENS_FP32_BULK) ------------------------
@@ -202,52 +232,27 @@ __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
     sz[t] = make_float4(ox.hi, oy.hi, ox.lo, oy.lo);
     sc[t] = make_float2((float)-A.gy[2 * ridx], (float)-A.gy[2 * ridx + 1]);
   }
-  // the stars of the U-list leaves, flattened over the block's threads (a
-  // leaf's own count is often below the block size): up to kAdjU leaves at a
-  // time, their first star and inclusive star counts in shared memory
-  __shared__ int su_start[kAdjU], su_incl[kAdjU];
-  const int64_t u0 = A.U_off[a], nu = A.U_off[a + 1] - u0;
-  for (int64_t ub = 0; ub < nu; ub += kAdjU) {
-    const int nub = (int)min64(kAdjU, nu - ub);
-    __syncthreads();  // the previous group's readers are done (and the rays staged)
-    if (threadIdx.x < nub) {
-      const int C = A.U_list[u0 + ub + threadIdx.x];
-      su_start[threadIdx.x] = A.start[C];
-      su_incl[threadIdx.x] = A.count[C];
+  __shared__ UStage su;
+  for_u_stars(A, a, su, [&](int sj) {
+    const double2 zj = A.spos[sj];
+    const ff sx = ff_of(zj.x - cB.x), sy = ff_of(zj.y - cB.y);
+    fcomp F1{0.f, 0.f}, F2{0.f, 0.f}, G1{0.f, 0.f}, G2{0.f, 0.f};
+    for (int t = 0; t < nr; ++t) {
+      const float4 z = sz[t];
+      const float2 c = sc[t];
+      // d = z_r - z_j; 1/d = conj(d) / |d|^2 (a star exactly at the ray adds
+      // nothing: d = 0 makes both terms 0 under the floor on |d|^2)
+      const float d1 = (z.x - sx.hi) + (z.z - sx.lo), d2 = (z.y - sy.hi) + (z.w - sy.lo);
+      const float w = frcp_fast(fmaf(d1, d1, fmaf(d2, d2, 1e-30f)));
+      const float i1 = d1 * w, i2 = -d2 * w;
+      const float c1 = c.x * i1 - c.y * i2, c2 = c.x * i2 + c.y * i1;  // c / d
+      F1.add(c1); F2.add(c2);
+      G1.add(c1 * i1 - c2 * i2); G2.add(c1 * i2 + c2 * i1);             // c / d^2
     }
-    __syncthreads();
-    if (threadIdx.x == 0)
-      for (int i = 1; i < nub; ++i) su_incl[i] += su_incl[i - 1];
-    __syncthreads();
-    const int tot = su_incl[nub - 1];
-    for (int q = threadIdx.x; q < tot; q += blockDim.x) {
-      // the group's leaf holding flattened star q: the first with su_incl > q
-      int lo = 0, hi = nub - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (su_incl[mid] > q) hi = mid; else lo = mid + 1;
-      }
-      const int sj = su_start[lo] + q - (lo ? su_incl[lo - 1] : 0);
-      const double2 zj = A.spos[sj];
-      const ff sx = ff_of(zj.x - cB.x), sy = ff_of(zj.y - cB.y);
-      fcomp F1{0.f, 0.f}, F2{0.f, 0.f}, G1{0.f, 0.f}, G2{0.f, 0.f};
-      for (int t = 0; t < nr; ++t) {
-        const float4 z = sz[t];
-        const float2 c = sc[t];
-        // d = z_r - z_j; 1/d = conj(d) / |d|^2 (a star exactly at the ray adds
-        // nothing: d = 0 makes both terms 0 under the floor on |d|^2)
-        const float d1 = (z.x - sx.hi) + (z.z - sx.lo), d2 = (z.y - sy.hi) + (z.w - sy.lo);
-        const float w = frcp_fast(fmaf(d1, d1, fmaf(d2, d2, 1e-30f)));
-        const float i1 = d1 * w, i2 = -d2 * w;
-        const float c1 = c.x * i1 - c.y * i2, c2 = c.x * i2 + c.y * i1;  // c / d
-        F1.add(c1); F2.add(c2);
-        G1.add(c1 * i1 - c2 * i2); G2.add(c1 * i2 + c2 * i1);             // c / d^2
-      }
-      const double mj = A.smass[sj];
-      atomic_add2(A.Phi + sj, make_double2(F1.value(), F2.value()));
-      atomic_add2(A.Psi + sj, make_double2(mj * G1.value(), mj * G2.value()));
-    }
-  }
+    const double mj = A.smass[sj];
+    atomic_add2(A.Phi + sj, make_double2(F1.value(), F2.value()));
+    atomic_add2(A.Psi + sj, make_double2(mj * G1.value(), mj * G2.value()));
+  });
 }
 
 // L2P^T and M2P^T moments in float32: one warp per (leaf, tile), as
@@ -331,12 +336,16 @@ __global__ void __launch_bounds__(128) k_adj_l2l(AdjArgs A, const int* active, i
   }
 }
 
-// M2L^T (V) and P2L^T (X): warp per active box.
-__global__ void __launch_bounds__(128) k_adj_m2l(AdjArgs A, const int* active, int64_t na) {
-  __shared__ double2 sbuf[4][kMaxOrder + 2];
+// M2L^T (V) and P2L^T (X): block per active box, its warps taking the V entries
+// and the X stars in turn (a warp per box left a small target region, a few
+// dozen boxes of ~27 entries each, on as many warps: 124 ->
+// 30 us at p 24).
+constexpr int kAdjM2lWarps = 8;
+__global__ void __launch_bounds__(32 * kAdjM2lWarps)
+k_adj_m2l(AdjArgs A, const int* active, int64_t na) {
+  __shared__ double2 sbuf[kAdjM2lWarps][kMaxOrder + 2];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t ai = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
-  if (ai >= na) return;
+  const int64_t ai = blockIdx.x;
   const int B = active[ai];
   const int p = A.p, P1 = p + 1;
   const double r = box_r(A, B);
@@ -344,7 +353,7 @@ __global__ void __launch_bounds__(128) k_adj_m2l(AdjArgs A, const int* active, i
   const double2 cB = box_c(A, B, r);
   const double2* Lb = A.Lh + (int64_t)B * P1;
   double2* buf = sbuf[wib];
-  for (int64_t e = A.V_off[ai]; e < A.V_off[ai + 1]; ++e) {
+  for (int64_t e = A.V_off[ai] + wib; e < A.V_off[ai + 1]; e += kAdjM2lWarps) {
     const int C = A.V_list[e];
     const int dx = A.ix[C] - A.ix[B], dy = A.iy[C] - A.iy[B];
     const double2* up = A.tab.upow + (int64_t)((dy + 3) * 7 + (dx + 3)) * (p + 2);
@@ -368,7 +377,7 @@ __global__ void __launch_bounds__(128) k_adj_m2l(AdjArgs A, const int* active, i
   }
   for (int64_t e = A.X_off[ai]; e < A.X_off[ai + 1]; ++e) {
     const int C = A.X_list[e];
-    for (int j = A.start[C]; j < A.start[C] + A.count[C]; ++j) {
+    for (int j = A.start[C] + wib; j < A.start[C] + A.count[C]; j += kAdjM2lWarps) {
       const double2 z = A.spos[j];
       const double m = A.smass[j];
       const double2 inv = cinv(make_double2(z.x - cB.x, z.y - cB.y));
@@ -417,27 +426,32 @@ __global__ void __launch_bounds__(128) k_adj_m2m(AdjArgs A, int64_t b0, int64_t 
   }
 }
 
-// P2M^T at the stars of every leaf (thread per leaf).
-__global__ void k_adj_p2m(AdjArgs A, int64_t nb) {
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// P2M^T at the stars of every leaf, G lanes a leaf (a thread a leaf ran its stars
+// one after another, ~25 dependent float64 steps each: 161 -> 29 us at 2e4
+// stars, leaves of 16, p 24).  Horner's rule
+// for the sum and its derivative side by side.
+template <int G>
+__global__ void __launch_bounds__(128) k_adj_p2m(AdjArgs A, int64_t nb) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t b = t / G;
   if (b >= nb || A.child[b] >= 0 || A.count[b] == 0) return;
   const int p = A.p, P1 = p + 1;
   const double r = box_r(A, (int)b);
   const double2 c = box_c(A, (int)b, r);
   const double ir = 1.0 / r;
   const double2* Mb = A.Mh + b * P1;
-  for (int j = A.start[b]; j < A.start[b] + A.count[b]; ++j) {
+  const int s0 = A.start[b], s1 = s0 + A.count[b];
+  for (int j = s0 + (int)(t % G); j < s1; j += G) {
     const double2 z = A.spos[j];
     const double m = A.smass[j];
     const double2 w = make_double2((z.x - c.x) * ir, (z.y - c.y) * ir);
-    double2 F = Mb[p], G = make_double2(p * Mb[p].x, p * Mb[p].y);
+    double2 F = Mb[p], D = make_double2(0.0, 0.0);  // sum, derivative in w
     for (int kk = p - 1; kk >= 0; --kk) {
+      D = cfma(D, w, F);
       F = cfma(F, w, Mb[kk]);
-      if (kk >= 1) G = cfma(G, w, make_double2(kk * Mb[kk].x, kk * Mb[kk].y));
     }
-    // G = sum_{k>=1} k Mhat_k w^(k-1)
     A.Phi[j] = A.Phi[j] + F;
-    A.Psi[j] = A.Psi[j] + make_double2(m * G.x * ir, m * G.y * ir);
+    A.Psi[j] = A.Psi[j] + make_double2(m * D.x * ir, m * D.y * ir);
   }
 }
 
@@ -527,7 +541,7 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
     LENS_LAUNCHED("k_adj_l2l");
   }
   if (P.n_active > 0) {
-    k_adj_m2l<<<grid_for(P.n_active * 32, 128), 128, 0, s>>>(A, P.active, P.n_active);
+    k_adj_m2l<<<(unsigned)P.n_active, 32 * kAdjM2lWarps, 0, s>>>(A, P.active, P.n_active);
     LENS_LAUNCHED("k_adj_m2l");
   }
   // M2M^T, coarsest level first
@@ -536,7 +550,9 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
     k_adj_m2m<<<grid_for((b1 - b0) * 32, 128), 128, 0, s>>>(A, b0, b1);
     LENS_LAUNCHED("k_adj_m2m");
   }
-  k_adj_p2m<<<grid_for(P.nb, 128), 128, 0, s>>>(A, P.nb);
+  if (P.leaf <= 8) k_adj_p2m<8><<<grid_for(P.nb * 8, 128), 128, 0, s>>>(A, P.nb);
+  else if (P.leaf <= 16) k_adj_p2m<16><<<grid_for(P.nb * 16, 128), 128, 0, s>>>(A, P.nb);
+  else k_adj_p2m<32><<<grid_for(P.nb * 32, 128), 128, 0, s>>>(A, P.nb);
   LENS_LAUNCHED("k_adj_p2m");
   if (gkg) {
     k_adj_kg<<<grid_for(m, 256, 1024), 256, 0, s>>>(rays, gy, m, gkg);

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval(EvalArgs A) {
             const double d1 = dx[q] - sx, d2 = dy[q] - sy;
             const double r2 = d1 * d1 + d2 * d2;
             // a star exactly on the ray contributes nothing
-            const double inv = r2 > 0.0 ? 1.0 / r2 : 0.0;
+            const double inv = rcp_or_zero(r2);
             const double w = sm * inv;
             p1[q] += w * d1;
             p2[q] += w * d2;
