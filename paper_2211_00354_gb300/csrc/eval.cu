@@ -431,6 +431,8 @@ __global__ void k_tile_leaf(const int64_t* __restrict__ toff, int64_t nl, int64_
   out[t] = make_int2((int)lo, (int)(t - toff[lo]));
 }
 
+}  // namespace
+
 Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s) {
   if (total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
   Scratch tl(&P.da, sizeof(int2) * (size_t)std::max<int64_t>(total, 1));
@@ -438,6 +440,8 @@ Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cud
   LENS_LAUNCHED("k_tile_leaf");
   return tl;
 }
+
+namespace {
 
 template <bool GRID, bool PIX>
 void launch_eval(Plan& P, EvalArgs& A, int64_t total_tiles, bool jac, cudaStream_t s) {
@@ -568,7 +572,8 @@ void evaluate_grid_pix(Plan& P, const GridRows& g, PixCorner* out, const IpmPara
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s) {
   const int64_t nl = P.n_active_leaves;
   if (nl == 0) fail(LENS_EDOMAIN, "plan has no active leaves");
-  Scratch slot(&P.da, sizeof(int) * m);
+  B.slot = Scratch(&P.da, sizeof(int) * m);
+  const Scratch& slot = B.slot;
   Scratch cnt(&P.da, sizeof(int64_t) * (nl + 1));
   Scratch cur(&P.da, sizeof(int64_t) * (nl + 1));
   Scratch tiles(&P.da, sizeof(int64_t) * (nl + 1));

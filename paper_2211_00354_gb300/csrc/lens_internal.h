@@ -262,11 +262,15 @@ void evaluate_grid(Plan& P, const GridRows& g, double* y, double* jac, cudaStrea
 void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* jac,
                    cudaStream_t s);
 // Rays bucketed by active leaf: perm (ray ids in leaf order), off (per leaf,
-// CSR into perm) and toff (per leaf, first tile of `tile` rays).
+// CSR into perm), toff (per leaf, first tile of `tile` rays) and slot (per ray,
+// its leaf).
 struct RayBuckets {
-  Scratch perm, off, toff;
+  Scratch perm, off, toff, slot;
   int64_t total = 0;  // tiles
 };
+// (leaf, tile within the leaf) of each of `total` tiles (toff: exclusive scan of
+// the leaves' tile counts)
+Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s);
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s);
 
 struct IpmParams {

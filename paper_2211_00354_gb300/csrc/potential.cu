@@ -20,13 +20,20 @@
 //   P2P  over U (the leaf itself included): sum_j m_j ln|z - z_j| (a star
 //        exactly at the ray contributes nothing)
 //   M2P  over W:  a_0 ln|z - c_C| - Re sum_{k>=1} (A_k / k) (r_C / (z - c_C))^k
-// All float64; a thread per ray descends the tree to its leaf, the rays taken
-// in leaf order (bucketed as the deflection's ray path does), so that the
-// lanes of a warp share their leaf's lists and stars.  Divisions by
-// the small integers k take a per-block table of 1/k, and with equal masses
-// the near field's logarithms are taken of products of up to 8 squared
-// distances (flushed early outside [1e-200, 1e200]): one float64 log where
-// there were eight, on GB300's slow float64 pipe.
+// All float64, so what counts is float64 operations (a warp-wide one takes a
+// sub-partition ~77 cycles).  A thread takes a ray, the rays in leaf order
+// (bucketed as the deflection's ray path does), so that the lanes of a warp share
+// their leaf's lists and stars; the leaf's centre, scale, constant and
+// integrated expansion are formed once per leaf.  With equal masses the near
+// field's logarithms are one: the squared distances' exponents add up as
+// integers and their mantissas multiply.  1e5 stars, leaves of 8, 2.6e5 rays: 1392
+// -> 474 us a call (a logarithm per 8 stars, float64 range checks, divisions per ray
+// and a launch per level for the constants before).  Not kept: a block per
+// leaf and 128 of its rays with everything staged in shared memory (744 us
+// against 635 for the same sums: partly filled warps cost as much as full ones).
+// The constant c_B is formed as one increment per active box (its V and X
+// lists and its parent's expansion at its centre), summed up the ancestors of
+// each leaf.
 #include "cx.cuh"
 #include "potential.h"
 
@@ -36,17 +43,15 @@ namespace {
 struct PotArgs {
   int p;
   double lo_x, lo_y, size;
-  int depth;
   const int* level; const int* ix; const int* iy; const int* parent; const int* child;
-  const int* aidx; const int* lidx; const int* start; const int* count; const int* active;
+  const int* aidx; const int* start; const int* count; const int* active;
   const double2* spos; const double* smass;
   const double2* M; const double2* L;
   const int64_t* V_off; const int* V_list; const int64_t* X_off; const int* X_list;
   const int64_t* U_off; const int* U_list; const int64_t* W_off; const int* W_list;
   double* c0;  // per active box
   double ks, g;
-  int um;        // all masses equal to m0
-  double m0;
+  double m0;  // the mass of every star, if all are equal
 };
 
 __device__ __forceinline__ double half_side(const PotArgs& A, int level) {
@@ -55,17 +60,6 @@ __device__ __forceinline__ double half_side(const PotArgs& A, int level) {
 __device__ __forceinline__ double2 centre(const PotArgs& A, int b, double r) {
   return make_double2(A.lo_x + (2.0 * A.ix[b] + 1.0) * r, A.lo_y + (2.0 * A.iy[b] + 1.0) * r);
 }
-// -Re sum_{k=1..p} (A_k / k) v^k, inv[k] = 1/k
-__device__ __forceinline__ double tail(const double2* Ak, int p, double2 v, const double* inv) {
-  double s = 0.0;
-  double2 pw = v;
-  for (int k = 1; k <= p; ++k) {
-    s -= (Ak[k].x * pw.x - Ak[k].y * pw.y) * inv[k];
-    pw = cmul(pw, v);
-  }
-  return s;
-}
-
 // 1/k for k = 0 .. n-1 in shared memory (1/0 unused); block-cooperative
 constexpr int kPotInv = kMaxOrder + 2;
 __device__ __forceinline__ void fill_inv(double* inv, int n) {
@@ -73,9 +67,48 @@ __device__ __forceinline__ void fill_inv(double* inv, int n) {
   __syncthreads();
 }
 
-// own constant of every active box: M2L over V and P2L over X (warp per box)
-__global__ void k_pot_own(PotArgs A, int64_t nact) {
+// sum of ln d2 over positive d2: exponents summed as integers, mantissas
+// multiplied (each in [1, 2), so up to kLogRun of them stay in range); zeros are
+// left out, subnormal and non-finite values take their own logarithm.
+constexpr int kLogRun = 512;
+struct LogSum {
+  double prod = 1.0, rest = 0.0;
+  int e = 0, n = 0;
+  __device__ __forceinline__ void add(double d2) {
+    const int hi = __double2hiint(d2);
+    if ((unsigned)hi - 0x00100000u < 0x7ff00000u - 0x00100000u) {
+      e += (hi >> 20) - 1023;
+      prod *= __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(d2));
+      if (++n == kLogRun) fold();
+    } else if (d2 > 0.0) {
+      rest += log(d2);
+    }
+  }
+  __device__ __forceinline__ void fold() {  // prod back to [1, 2)
+    const int hi = __double2hiint(prod);
+    e += (hi >> 20) - 1023;
+    prod = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(prod));
+    n = 0;
+  }
+  __device__ __forceinline__ double value() const {
+    return rest + fma((double)e, 0.69314718055994530942, log(prod));  // ln 2
+  }
+};
+
+// increment of every active box (warp per box): M2L over V, P2L over X, and
+// the parent's expansion at the box centre.  u^k and ((1+i)/2)^k come from the
+// translation tables.
+constexpr int kLevels = kMaxDepth + 2;
+__global__ void k_pot_own(PotArgs A, FmmTables T, int64_t nact) {
   __shared__ double inv[kPotInv];
+  // ln |(dx, dy)| by dx^2 + dy^2 (at most 18 in a V list), ln(2 r) by level
+  __shared__ double lnd[19], lnr[kLevels];
+  if (threadIdx.x >= 64 && threadIdx.x < 64 + 19) {
+    const int q = threadIdx.x - 64;
+    lnd[q] = q ? 0.5 * log((double)q) : 0.0;
+  }
+  if (threadIdx.x >= 96 && threadIdx.x < 96 + kLevels)
+    lnr[threadIdx.x - 96] = log(2.0 * half_side(A, threadIdx.x - 96));
   fill_inv(inv, A.p + 2);
   const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -87,12 +120,12 @@ __global__ void k_pot_own(PotArgs A, int64_t nact) {
   double acc = 0.0;
   for (int64_t e = A.V_off[a] + lane; e < A.V_off[a + 1]; e += 32) {
     const int C = A.V_list[e];
-    const double2 cC = centre(A, C, r);
-    const double2 t = make_double2(cB.x - cC.x, cB.y - cC.y);
+    const int dx = A.ix[C] - A.ix[B], dy = A.iy[C] - A.iy[B];
     const double2* Ak = A.M + (int64_t)C * P1;
-    const double2 it = cinv(t);
-    acc += Ak[0].x * 0.5 * log(t.x * t.x + t.y * t.y) +
-           tail(Ak, A.p, make_double2(r * it.x, r * it.y), inv);
+    const double2* u = T.upow + (int64_t)((dy + 3) * 7 + dx + 3) * (A.p + 2);
+    // |t| = 2 r |(dx, dy)|
+    acc = fma(Ak[0].x, lnr[A.level[B]] + lnd[dx * dx + dy * dy], acc);
+    for (int k = 1; k <= A.p; ++k) acc -= inv[k] * (Ak[k].x * u[k].x - Ak[k].y * u[k].y);
   }
   for (int64_t e = A.X_off[a]; e < A.X_off[a + 1]; ++e) {
     const int C = A.X_list[e];
@@ -101,123 +134,122 @@ __global__ void k_pot_own(PotArgs A, int64_t nact) {
       acc += A.smass[j] * 0.5 * log(dx * dx + dy * dy);
     }
   }
+  const int Pb = A.parent[B];
+  if (Pb >= 0 && A.aidx[Pb] >= 0) {
+    // d^(l+1) = w^(l+1) i^(m (l+1)), w = (1+i)/2, m = 2, 3, 1, 0 for the quadrants;
+    // w^(l+1) = w w^l
+    const int q = B - A.child[Pb], m = q == 0 ? 2 : q == 1 ? 3 : q == 2 ? 1 : 0;
+    const double2* Bl = A.L + (int64_t)Pb * P1;
+    double s = 0.0;
+    for (int l = lane; l <= A.p; l += 32) {
+      const double2 w0 = T.wpow[l];
+      const double2 w = make_double2(0.5 * (w0.x - w0.y), 0.5 * (w0.x + w0.y));
+      const int ph = (m * (l + 1)) & 3;
+      // Re(B_l w i^ph)
+      const double2 b = Bl[l];
+      const double re = b.x * w.x - b.y * w.y, im = b.x * w.y + b.y * w.x;
+      s += inv[l + 1] * (ph == 0 ? re : ph == 1 ? -im : ph == 2 ? -re : im);
+    }
+    acc = fma(2.0 * r, s, acc);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) A.c0[a] = acc;
 }
 
-// the parent's far field at each box centre, one level at a time (thread per
-// active box of the level)
-__global__ void k_pot_down(PotArgs A, int64_t a0, int64_t a1) {
-  const int64_t a = a0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (a >= a1) return;
-  const int B = A.active[a];
-  const int Pb = A.parent[B];
-  if (Pb < 0) return;
-  const int ap = A.aidx[Pb];
-  if (ap < 0) return;
-  const double rP = half_side(A, A.level[Pb]);
-  const double2 d = make_double2((2.0 * A.ix[B] + 1.0 - 2.0 * (2.0 * A.ix[Pb] + 1.0)) * 0.5,
-                                 (2.0 * A.iy[B] + 1.0 - 2.0 * (2.0 * A.iy[Pb] + 1.0)) * 0.5);
-  const double2* Bl = A.L + (int64_t)Pb * (A.p + 1);
-  // sum_l B_l d^(l+1) / (l+1) by Horner
-  double2 acc = make_double2(Bl[A.p].x / (A.p + 1), Bl[A.p].y / (A.p + 1));
-  for (int l = A.p - 1; l >= 0; --l) {
-    acc = cmul(acc, d);
-    acc.x += Bl[l].x / (l + 1);
-    acc.y += Bl[l].y / (l + 1);
-  }
-  acc = cmul(acc, d);
-  A.c0[a] += A.c0[ap] + rP * acc.x;
+// Per active leaf: centre, half-side and its inverse, c_B (its increment and its
+// active ancestors'), and the integrated expansion B_l / (l + 1); thread per
+// (leaf, coefficient).
+struct LeafPot {
+  double cx, cy, r, ir, c;
+  int a, pad;
+};
+__global__ void k_pot_leaf(PotArgs A, const int* __restrict__ leaves, int64_t nl,
+                           LeafPot* __restrict__ lp, double2* __restrict__ Bi) {
+  __shared__ double inv[kPotInv];
+  fill_inv(inv, A.p + 2);
+  const int P1 = A.p + 1;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t k = t / P1;
+  if (k >= nl) return;
+  const int l = (int)(t - k * P1), b = leaves[k];
+  const double2 v = A.L[(int64_t)b * P1 + l];
+  Bi[t] = make_double2(v.x * inv[l + 1], v.y * inv[l + 1]);
+  if (l > 0) return;
+  LeafPot q;
+  q.r = half_side(A, A.level[b]);
+  const double2 c = centre(A, b, q.r);
+  q.cx = c.x; q.cy = c.y;
+  q.ir = 1.0 / q.r;
+  q.c = 0.0;
+  q.a = A.aidx[b]; q.pad = 0;
+  for (int x = b; x >= 0 && A.aidx[x] >= 0; x = A.parent[x]) q.c += A.c0[A.aidx[x]];
+  lp[k] = q;
 }
 
-__global__ void k_pot_eval(PotArgs A, const double* __restrict__ rays, int64_t m,
-                           const int* __restrict__ perm, double* __restrict__ psi,
-                           int* __restrict__ err) {
+__device__ __forceinline__ double smooth_psi(const PotArgs& A, double x, double y) {
+  return 0.5 * A.ks * (x * x + y * y) + 0.5 * A.g * (x * x - y * y);
+}
+// M2P of one W box: a_0 ln|t| - Re sum_{k>=1} (A_k / k) (r_C / t)^k, the
+// coefficients Ak over k by Horner's rule (coef(k) = A_k / k)
+template <typename F>
+__device__ __forceinline__ double pot_m2p(double a0, int p, double2 t, double rC, F coef) {
+  const double2 it = cinv(t);
+  const double2 v = make_double2(rC * it.x, rC * it.y);
+  double2 s = make_double2(0.0, 0.0);
+  for (int k = p; k >= 1; --k) {
+    s = s + coef(k);
+    s = cmul(s, v);
+  }
+  return fma(a0, 0.5 * log(t.x * t.x + t.y * t.y), -s.x);
+}
+
+// Thread per ray, rays in leaf order (slot[r]: its leaf).
+template <bool UM>
+__global__ void __launch_bounds__(128)
+k_pot_rays(PotArgs A, const double* __restrict__ rays, int64_t m, const int* __restrict__ slot,
+           const int* __restrict__ perm, const LeafPot* __restrict__ lp,
+           const double2* __restrict__ Bi, int wmax, double* __restrict__ psi) {
   __shared__ double inv[kPotInv];
   fill_inv(inv, A.p + 2);
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= m) return;
   const int64_t r = perm[t];
   const double x = rays[2 * r], y = rays[2 * r + 1];
-  const double scale = (double)(1ull << A.depth) / A.size;
-  const double qmax = (double)((1u << A.depth) - 1u);
-  const double fx = floor((x - A.lo_x) * scale), fy = floor((y - A.lo_y) * scale);
-  if (!(fx >= 0.0 && fx <= qmax && fy >= 0.0 && fy <= qmax)) {  // also catches NaN
-    atomicExch(err, 1);
-    psi[r] = NAN;
-    return;
-  }
-  const uint32_t qx = (uint32_t)fx, qy = (uint32_t)fy;
-  int b = 0;
-  for (int l = 0; l < A.depth; ++l) {
-    const int c = A.child[b];
-    if (c < 0) break;
-    const int sh = A.depth - l - 1;
-    b = c + (int)(((qx >> sh) & 1u) | (((qy >> sh) & 1u) << 1));
-  }
-  const int a = A.aidx[b];
-  if (A.lidx[b] < 0 || a < 0) {
-    atomicExch(err, 1);
-    psi[r] = NAN;
-    return;
-  }
-  const double rb = half_side(A, A.level[b]);
-  const double2 cb = centre(A, b, rb);
-  const int P1 = A.p + 1;
+  const int k0 = slot[r];
+  const LeafPot q = lp[k0];
+  const int a = q.a, P1 = A.p + 1;
   // L2P of the integrated local expansion
-  const double2 w = make_double2((x - cb.x) / rb, (y - cb.y) / rb);
-  const double2* Bl = A.L + (int64_t)b * P1;
-  double2 acc = make_double2(Bl[A.p].x * inv[P1], Bl[A.p].y * inv[P1]);
-  for (int l = A.p - 1; l >= 0; --l) {
-    acc = cmul(acc, w);
-    acc.x += Bl[l].x * inv[l + 1];
-    acc.y += Bl[l].y * inv[l + 1];
-  }
+  const double2 w = make_double2((x - q.cx) * q.ir, (y - q.cy) * q.ir);
+  const double2* Bl = Bi + (int64_t)k0 * P1;
+  double2 acc = Bl[A.p];
+  for (int l = A.p - 1; l >= 0; --l) acc = cfma(acc, w, Bl[l]);
   acc = cmul(acc, w);
-  double phi = A.c0[a] + rb * acc.x;
-  // P2P over U (a star exactly at the ray contributes nothing)
-  if (A.um) {
-    double lsum = 0.0, prod = 1.0;
-    int n = 0;
-    for (int64_t e = A.U_off[a]; e < A.U_off[a + 1]; ++e) {
-      const int C = A.U_list[e];
-      for (int j = A.start[C]; j < A.start[C] + A.count[C]; ++j) {
-        const double dx = x - A.spos[j].x, dy = y - A.spos[j].y;
-        const double d2 = dx * dx + dy * dy;
-        if (!(d2 > 0.0)) continue;
-        prod *= d2;
-        if (++n == 8 || !(prod > 1e-200 && prod < 1e200)) {
-          lsum += log(prod);
-          prod = 1.0;
-          n = 0;
-        }
-      }
+  double phi = fma(q.r, acc.x, q.c);
+  // P2P over U (a star exactly at the ray contributes nothing) and over W boxes
+  // of at most wmax stars
+  LogSum ls;
+  const auto p2p = [&](int C) {
+    for (int j = A.start[C]; j < A.start[C] + A.count[C]; ++j) {
+      const double dx = x - A.spos[j].x, dy = y - A.spos[j].y;
+      const double d2 = dx * dx + dy * dy;
+      if (UM) ls.add(d2);
+      else if (d2 > 0.0) phi += A.smass[j] * 0.5 * log(d2);
     }
-    if (n > 0) lsum += log(prod);
-    phi += 0.5 * A.m0 * lsum;
-  } else {
-    for (int64_t e = A.U_off[a]; e < A.U_off[a + 1]; ++e) {
-      const int C = A.U_list[e];
-      for (int j = A.start[C]; j < A.start[C] + A.count[C]; ++j) {
-        const double dx = x - A.spos[j].x, dy = y - A.spos[j].y;
-        const double d2 = dx * dx + dy * dy;
-        if (d2 > 0.0) phi += A.smass[j] * 0.5 * log(d2);
-      }
-    }
-  }
-  // M2P over W
+  };
+  for (int64_t e = A.U_off[a]; e < A.U_off[a + 1]; ++e) p2p(A.U_list[e]);
   for (int64_t e = A.W_off[a]; e < A.W_off[a + 1]; ++e) {
     const int C = A.W_list[e];
+    if (A.count[C] <= wmax) { p2p(C); continue; }
     const double rC = half_side(A, A.level[C]);
     const double2 cC = centre(A, C, rC);
-    const double2 t = make_double2(x - cC.x, y - cC.y);
     const double2* Ak = A.M + (int64_t)C * P1;
-    const double2 it = cinv(t);
-    phi += Ak[0].x * 0.5 * log(t.x * t.x + t.y * t.y) +
-           tail(Ak, A.p, make_double2(rC * it.x, rC * it.y), inv);
+    phi += pot_m2p(Ak[0].x, A.p, make_double2(x - cC.x, y - cC.y), rC, [&](int k) {
+      return make_double2(Ak[k].x * inv[k], Ak[k].y * inv[k]);
+    });
   }
-  psi[r] = phi + 0.5 * A.ks * (x * x + y * y) + 0.5 * A.g * (x * x - y * y);
+  if (UM) phi += 0.5 * A.m0 * ls.value();
+  psi[r] = phi + smooth_psi(A, x, y);
 }
 
 }  // namespace
@@ -225,40 +257,46 @@ __global__ void k_pot_eval(PotArgs A, const double* __restrict__ rays, int64_t m
 void evaluate_potential(Plan& P, const double* rays, int64_t m, double* psi, cudaStream_t s) {
   if (m == 0) return;
   if (P.n_active == 0) fail(LENS_EDOMAIN, "plan has no active boxes");
-  // the rays in leaf order (fails with LENS_EDOMAIN for a ray outside the root)
+  // the rays in leaf order (fails with LENS_EDOMAIN for a ray outside the
+  // target region)
+  const int64_t nl = P.n_active_leaves;
   RayBuckets RB;
   bucket_rays(P, rays, m, 1, RB, s);
   wait_expansions(P, s);
   Scratch c0(&P.da, sizeof(double) * (size_t)P.n_active);
-  Scratch err(&P.da, sizeof(int));
-  LENS_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), s));
+  Scratch lp(&P.da, sizeof(LeafPot) * (size_t)nl);
+  Scratch Bi(&P.da, sizeof(double2) * (size_t)nl * (P.p + 1));
   PotArgs A{};
   A.p = P.p;
-  A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.size = P.root_size; A.depth = P.depth;
+  A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.size = P.root_size;
   A.level = P.box_level; A.ix = P.box_ix; A.iy = P.box_iy; A.parent = P.box_parent;
-  A.child = P.box_child; A.aidx = P.box_aidx; A.lidx = P.box_lidx; A.start = P.box_start;
+  A.child = P.box_child; A.aidx = P.box_aidx; A.start = P.box_start;
   A.count = P.box_count; A.active = P.active; A.spos = P.spos; A.smass = P.smass;
   A.M = P.M; A.L = P.L;
   A.V_off = P.V_off; A.V_list = P.V_list; A.X_off = P.X_off; A.X_list = P.X_list;
   A.U_off = P.U_off; A.U_list = P.U_list; A.W_off = P.W_off; A.W_list = P.W_list;
   A.c0 = c0.as<double>();
   A.ks = P.kappa_s; A.g = P.gamma;
-  A.um = P.equal_mass ? 1 : 0;
   A.m0 = P.mass0;
-  k_pot_own<<<grid_for(P.n_active * 32, 256), 256, 0, s>>>(A, P.n_active);
+  k_pot_own<<<grid_for(P.n_active * 32, 256), 256, 0, s>>>(A, P.tab, P.n_active);
   LENS_LAUNCHED("k_pot_own");
-  for (size_t l = 1; l + 1 < P.active_level_off.size(); ++l) {
-    const int64_t a0 = P.active_level_off[l], a1 = P.active_level_off[l + 1];
-    if (a1 <= a0) continue;
-    k_pot_down<<<grid_for(a1 - a0, 128), 128, 0, s>>>(A, a0, a1);
-    LENS_LAUNCHED("k_pot_down");
-  }
-  k_pot_eval<<<grid_for(m, 128), 128, 0, s>>>(A, rays, m, RB.perm.as<int>(), psi, err.as<int>());
-  LENS_LAUNCHED("k_pot_eval");
-  int herr = 0;
-  LENS_CUDA(cudaMemcpyAsync(&herr, err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+  k_pot_leaf<<<grid_for(nl * (P.p + 1), 128), 128, 0, s>>>(A, P.active_leaves, nl, lp.as<LeafPot>(),
+                                                            Bi.as<double2>());
+  LENS_LAUNCHED("k_pot_leaf");
+  // float64 operations of an M2P (~6 p + 45: the products with 1/k, Horner's rule, a
+  // reciprocal, a logarithm) over those of a star summed directly: 5 with equal
+  // masses, ~35 with a logarithm each
+  const int wmax = (6 * P.p + 45) / (P.equal_mass ? 5 : 35);
+  if (P.equal_mass)
+    k_pot_rays<true><<<grid_for(m, 128), 128, 0, s>>>(A, rays, m, RB.slot.as<int>(),
+                                                      RB.perm.as<int>(), lp.as<LeafPot>(),
+                                                      Bi.as<double2>(), wmax, psi);
+  else
+    k_pot_rays<false><<<grid_for(m, 128), 128, 0, s>>>(A, rays, m, RB.slot.as<int>(),
+                                                       RB.perm.as<int>(), lp.as<LeafPot>(),
+                                                       Bi.as<double2>(), wmax, psi);
+  LENS_LAUNCHED("k_pot_rays");
   LENS_CUDA(cudaStreamSynchronize(s));
-  if (herr) fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
 }
 
 }  // namespace lens
