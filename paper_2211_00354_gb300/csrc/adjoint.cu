@@ -74,6 +74,7 @@ __device__ __forceinline__ double2 box_c(const AdjArgs& A, int b, double r) {
 __global__ void __launch_bounds__(32) k_adj_leaf_moments(AdjArgs A) {
   extern __shared__ double2 acc[];  // [(p+1)][32]
   const int lane = threadIdx.x;
+  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
   const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
   const int B = A.leaves[k];
   const int a = A.aidx[B];
@@ -173,6 +174,7 @@ __device__ __forceinline__ void for_u_stars(const AdjArgs& A, int a, UStage& su,
 __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
   __shared__ double2 sz[kAdjTile], sc[kAdjTile];
   __shared__ UStage su;
+  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
   const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
   const int a = A.aidx[A.leaves[k]];
   const int64_t tile = (int64_t)blockIdx.x - A.tile_off[k];
@@ -217,6 +219,7 @@ __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
 __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
   __shared__ float4 sz[kAdjTile];  // x_hi, y_hi, x_lo, y_lo
   __shared__ float2 sc[kAdjTile];
+  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
   const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
   const int B = A.leaves[k];
   const int a = A.aidx[B];
@@ -260,6 +263,7 @@ __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
 __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
   extern __shared__ float2 acc32[];  // [(p+1)][33]: lane partials, padded
   const int lane = threadIdx.x;
+  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
   const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
   const int B = A.leaves[k];
   const int a = A.aidx[B];
@@ -505,7 +509,7 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
   LENS_CUDA(cudaMemsetAsync(Psi.p, 0, Psi.bytes, s));
   AdjArgs A{};
   A.rays = rays; A.gy = gy;
-  A.perm = RB.perm.as<int>(); A.ray_off = RB.off.as<int64_t>(); A.tile_off = RB.toff.as<int64_t>();
+  A.perm = RB.perm.as<int>(); A.ray_off = RB.off; A.tile_off = RB.toff;
   A.nleaf = P.n_active_leaves;
   A.leaves = P.active_leaves; A.aidx = P.box_aidx; A.level = P.box_level; A.ix = P.box_ix;
   A.iy = P.box_iy; A.start = P.box_start; A.count = P.box_count; A.child = P.box_child;
@@ -516,21 +520,21 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
   A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.size = P.root_size; A.p = P.p;
   A.Lh = Lh.as<double2>(); A.Mh = Mh.as<double2>();
   A.Phi = Phi.as<double2>(); A.Psi = Psi.as<double2>();
-  if (RB.total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many rays in one adjoint call");
-  if (RB.total > 0 && P.prec == LENS_FP32_BULK) {
+  const unsigned tiles = (unsigned)RB.tiles_max;
+  if (P.prec == LENS_FP32_BULK) {
     const size_t smem = sizeof(float2) * (size_t)P1 * 33;
-    k_adj_leaf_moments32<<<(unsigned)RB.total, 32, smem, s>>>(A);
+    k_adj_leaf_moments32<<<tiles, 32, smem, s>>>(A);
     LENS_LAUNCHED("k_adj_leaf_moments32");
-    k_adj_p2p32<<<(unsigned)RB.total, 128, 0, s>>>(A);
+    k_adj_p2p32<<<tiles, 128, 0, s>>>(A);
     LENS_LAUNCHED("k_adj_p2p32");
-  } else if (RB.total > 0) {
+  } else {
     const size_t smem = sizeof(double2) * (size_t)P1 * 32;
     if (smem > 48 * 1024)
       LENS_CUDA(cudaFuncSetAttribute(k_adj_leaf_moments, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
-    k_adj_leaf_moments<<<(unsigned)RB.total, 32, smem, s>>>(A);
+    k_adj_leaf_moments<<<tiles, 32, smem, s>>>(A);
     LENS_LAUNCHED("k_adj_leaf_moments");
-    k_adj_p2p<<<(unsigned)RB.total, 128, 0, s>>>(A);
+    k_adj_p2p<<<tiles, 128, 0, s>>>(A);
     LENS_LAUNCHED("k_adj_p2p");
   }
   // L2L^T, finest level first (levels >= 2 carry L2L)
@@ -563,6 +567,7 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
                                                  gxy, gm);
     LENS_LAUNCHED("k_adj_out");
   }
+  check_rays(RB);
 }
 
 }  // namespace lens

@@ -97,6 +97,35 @@ static cudaMemPool_t library_pool() {
   return pool;
 }
 
+namespace {
+struct HostBlock {
+  int64_t* host = nullptr;
+  int64_t* dev = nullptr;
+  unsigned next = 0;
+  ~HostBlock() { if (host) cudaFreeHost(host); }
+};
+thread_local HostBlock g_host_block;
+}  // namespace
+
+HostSlot host_slot() {
+  HostBlock& b = g_host_block;
+  if (!b.host) {
+    void* h = nullptr;
+    LENS_CUDA(cudaHostAlloc(&h, sizeof(int64_t) * kHostSlots * kHostSlotWords,
+                            cudaHostAllocPortable | cudaHostAllocMapped));
+    void* d = nullptr;
+    const cudaError_t e = cudaHostGetDevicePointer(&d, h, 0);
+    if (e != cudaSuccess) {
+      cudaFreeHost(h);
+      LENS_CUDA(e);
+    }
+    b.host = static_cast<int64_t*>(h);
+    b.dev = static_cast<int64_t*>(d);
+  }
+  const unsigned k = (b.next++ % kHostSlots) * kHostSlotWords;
+  return HostSlot{b.host + k, b.dev + k};
+}
+
 void* DeviceAlloc::alloc(size_t bytes) {
   fault_point_alloc();
   if (bytes == 0) bytes = 16;

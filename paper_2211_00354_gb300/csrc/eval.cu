@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kEvalThreads) k_eval(EvalArgs A) {
   const int tid = threadIdx.x;
   const int p = A.p;
   const int2 kt = A.tile_leaf[blockIdx.x];
+  if (kt.x < 0) return;
   const int64_t k = kt.x;
   const int B = A.leaves[k];
   const int a = A.aidx[B];
@@ -357,14 +358,14 @@ __global__ void k_work_count(const int* __restrict__ leaves, int64_t nleaf,
 __global__ void k_ray_leaf(const double* __restrict__ rays, int64_t m, const int* __restrict__ child,
                            const int* __restrict__ lidx, double lo_x, double lo_y, double scale,
                            int depth, int* __restrict__ slot, int64_t* __restrict__ counts,
-                           int* __restrict__ err) {
+                           int64_t* __restrict__ err) {
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= m) return;
   const double x = rays[2 * r], y = rays[2 * r + 1];
   const double qmax = (double)((1u << depth) - 1u);
   const double fx = floor((x - lo_x) * scale), fy = floor((y - lo_y) * scale);
   if (!(fx >= 0.0 && fx <= qmax && fy >= 0.0 && fy <= qmax)) {  // also catches NaN
-    atomicExch(err, 1);
+    *err = 1;  // host memory: a plain store, whoever comes first
     slot[r] = -1;
     return;
   }
@@ -378,7 +379,7 @@ __global__ void k_ray_leaf(const double* __restrict__ rays, int64_t m, const int
   }
   const int li = lidx[b];
   if (li < 0) {
-    atomicExch(err, 1);
+    *err = 1;
     slot[r] = -1;
     return;
   }
@@ -413,6 +414,48 @@ __global__ void k_tiles_from_counts(const int64_t* __restrict__ counts, int64_t 
   tiles[k] = (counts[k] + tile - 1) / tile;
 }
 
+// off = exclusive scan of the n = nl + 1 counts, toff = of their tile counts, by
+// one block: for up to kOneBlockLeaves leaves (a few steps of the block) one launch instead of
+// three to seven.
+constexpr int kOffThreads = 1024;
+constexpr int64_t kOneBlockLeaves = 16384;
+__global__ void __launch_bounds__(kOffThreads)
+k_ray_offsets(const int64_t* __restrict__ cnt, int64_t n, int tile, int64_t* __restrict__ off,
+              int64_t* __restrict__ toff) {
+  __shared__ int64_t sc[2][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int64_t base = 0, tbase = 0;
+  for (int64_t i0 = 0; i0 < n; i0 += kOffThreads) {
+    const int64_t i = i0 + threadIdx.x;
+    const int64_t c = i < n ? cnt[i] : 0, t = (c + tile - 1) / tile;
+    int64_t x = c, y = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t u = __shfl_up_sync(0xffffffffu, x, o), v = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) { x += u; y += v; }
+    }
+    __syncthreads();  // the previous step's readers of sc are done
+    if (lane == 31) { sc[0][w] = x; sc[1][w] = y; }
+    __syncthreads();
+    if (w < 2) {
+      int64_t v = sc[w][lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+      }
+      sc[w][lane] = v;
+    }
+    __syncthreads();
+    if (i < n) {
+      off[i] = base + (w ? sc[0][w - 1] : 0) + x - c;
+      toff[i] = tbase + (w ? sc[1][w - 1] : 0) + y - t;
+    }
+    base += sc[0][31];
+    tbase += sc[1][31];
+  }
+}
+
 // (leaf, tile within the leaf) of every ray tile, one thread per tile, so
 // that each block of the evaluation kernels finds its leaf with one load.
 // The offsets are an exclusive scan (toff[0] = 0, toff[nl] = total): the
@@ -423,6 +466,7 @@ __global__ void k_tile_leaf(const int64_t* __restrict__ toff, int64_t nl, int64_
                             int2* __restrict__ out) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= total) return;
+  if (t >= toff[nl]) { out[t] = make_int2(-1, 0); return; }
   int64_t lo = 0, hi = nl;
   while (hi - lo > 1) {
     const int64_t mid = (lo + hi) >> 1;
@@ -470,8 +514,11 @@ EvalArgs base_args(Plan& P) {
   return A;
 }
 
-int tile_rays(const Plan& P) {
-  return P.prec == LENS_FP64 ? kEvalThreads * kRptD : kEval32Threads * kEval32Rpt;
+// grid rays a tile; the float32 form without a Jacobian takes its rays in 2 x 2
+// blocks, one a thread
+int tile_rays(const Plan& P, bool jac) {
+  return P.prec == LENS_FP64 ? kEvalThreads * kRptD
+                             : kEval32Threads * (jac ? eval32_rays_per_thread(true) : 1);
 }
 
 }  // namespace
@@ -482,9 +529,8 @@ void grid_impl(Plan& P, const GridRows& g, double* y, double* jac, PixCorner* pi
                const IpmParams* ip, cudaStream_t s) {
   const int64_t nl = P.n_active_leaves;
   if (nl == 0 || g.nrows <= 0) return;
-  // the float32 form without a Jacobian takes its rays in 2 x 2 blocks
   const bool quads = P.prec == LENS_FP32_BULK && !jac;
-  const int tile = quads ? kEval32Threads : tile_rays(P);
+  const int tile = tile_rays(P, jac != nullptr);
   Scratch rect(&P.da, sizeof(int64_t) * 4 * nl);
   Scratch tiles(&P.da, sizeof(int64_t) * (nl + 1));
   Scratch toff(&P.da, sizeof(int64_t) * (nl + 1));
@@ -543,7 +589,7 @@ void evaluate_grid_fused(Plan& P, const GridRows& g, PixCorner* edge, const IpmP
   k_grid_rects<<<grid_for(nl, 128), 128, 0, s>>>(P.active_leaves, nl, P.box_level, P.box_ix,
                                                  P.box_iy, P.root_lo[0], P.root_lo[1],
                                                  P.root_size, g.x0, g.y0, g.h, g.nx, g.row0,
-                                                 g.nrows, tile_rays(P), false, rect.as<int64_t>(),
+                                                 g.nrows, kEval32Threads, false, rect.as<int64_t>(),
                                                  tiles.as<int64_t>());
   LENS_LAUNCHED("k_grid_rects");
   if (P.work) {
@@ -572,54 +618,65 @@ void evaluate_grid_pix(Plan& P, const GridRows& g, PixCorner* out, const IpmPara
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s) {
   const int64_t nl = P.n_active_leaves;
   if (nl == 0) fail(LENS_EDOMAIN, "plan has no active leaves");
+  // counts and cursors (zeroed together), then the offsets
+  const size_t n = (size_t)nl + 1;
+  B.mem = Scratch(&P.da, sizeof(int64_t) * 4 * n);
   B.slot = Scratch(&P.da, sizeof(int) * m);
-  const Scratch& slot = B.slot;
-  Scratch cnt(&P.da, sizeof(int64_t) * (nl + 1));
-  Scratch cur(&P.da, sizeof(int64_t) * (nl + 1));
-  Scratch tiles(&P.da, sizeof(int64_t) * (nl + 1));
-  Scratch err(&P.da, sizeof(int) * 4);
-  B.off = Scratch(&P.da, sizeof(int64_t) * (nl + 1));
   B.perm = Scratch(&P.da, sizeof(int) * m);
-  B.toff = Scratch(&P.da, sizeof(int64_t) * (nl + 1));
-  LENS_CUDA(cudaMemsetAsync(cnt.p, 0, cnt.bytes, s));
-  LENS_CUDA(cudaMemsetAsync(cur.p, 0, cur.bytes, s));
-  LENS_CUDA(cudaMemsetAsync(err.p, 0, err.bytes, s));
+  int64_t* cnt = B.mem.as<int64_t>();
+  int64_t* cur = cnt + n;
+  int64_t* off = cur + n;
+  int64_t* toff = off + n;
+  B.flag = host_slot();
+  B.flag.host[0] = 0;
+  LENS_CUDA(cudaEventCreateWithFlags(&B.leaves_known, cudaEventDisableTiming));
+  LENS_CUDA(cudaMemsetAsync(B.mem.p, 0, sizeof(int64_t) * 2 * n, s));
   const double scale = (double)(1ull << P.depth) / P.root_size;
   k_ray_leaf<<<grid_for(m, 256), 256, 0, s>>>(rays, m, P.box_child, P.box_lidx, P.root_lo[0],
-                                              P.root_lo[1], scale, P.depth, slot.as<int>(),
-                                              cnt.as<int64_t>(), err.as<int>());
+                                              P.root_lo[1], scale, P.depth, B.slot.as<int>(), cnt,
+                                              B.flag.dev);
   LENS_LAUNCHED("k_ray_leaf");
-  exclusive_scan_i64(cnt.as<int64_t>(), B.off.as<int64_t>(), nl + 1, P.da, s);
-  k_ray_scatter<<<grid_for(m, 256), 256, 0, s>>>(slot.as<int>(), m, B.off.as<int64_t>(),
-                                                 cur.as<int64_t>(), B.perm.as<int>());
+  LENS_CUDA(cudaEventRecord(B.leaves_known, s));
+  if (nl <= kOneBlockLeaves) {
+    k_ray_offsets<<<1, kOffThreads, 0, s>>>(cnt, nl + 1, tile, off, toff);
+    LENS_LAUNCHED("k_ray_offsets");
+  } else {
+    exclusive_scan_i64(cnt, off, nl + 1, P.da, s);
+    k_tiles_from_counts<<<grid_for(nl + 1, 256), 256, 0, s>>>(cnt, nl + 1, tile, toff);
+    LENS_LAUNCHED("k_tiles_from_counts");
+    exclusive_scan_i64(toff, toff, nl + 1, P.da, s);
+  }
+  k_ray_scatter<<<grid_for(m, 256), 256, 0, s>>>(B.slot.as<int>(), m, off, cur, B.perm.as<int>());
   LENS_LAUNCHED("k_ray_scatter");
-  k_tiles_from_counts<<<grid_for(nl + 1, 256), 256, 0, s>>>(cnt.as<int64_t>(), nl + 1, tile,
-                                                            tiles.as<int64_t>());
-  LENS_LAUNCHED("k_tiles_from_counts");
-  exclusive_scan_i64(tiles.as<int64_t>(), B.toff.as<int64_t>(), nl + 1, P.da, s);
-  int herr[4] = {0, 0, 0, 0};
-  B.total = 0;
-  LENS_CUDA(cudaMemcpyAsync(&B.total, B.toff.as<int64_t>() + nl, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  LENS_CUDA(cudaMemcpyAsync(herr, err.p, sizeof(herr), cudaMemcpyDeviceToHost, s));
-  LENS_CUDA(cudaStreamSynchronize(s));
-  if (herr[0]) fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
+  B.off = off;
+  B.toff = toff;
+  B.tiles_max = m / tile + std::min(nl, m);
+  if (B.tiles_max > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
+}
+
+void check_rays(const RayBuckets& B) {
+  LENS_CUDA(cudaEventSynchronize(B.leaves_known));
+  if (B.flag.host[0]) fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
 }
 
 void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* jac, cudaStream_t s) {
   if (m == 0) return;
+  const bool f64 = P.prec == LENS_FP64;
+  const int rpt = f64 ? kRptD : eval32_rays_per_thread(jac != nullptr);
   RayBuckets B;
-  bucket_rays(P, rays, m, tile_rays(P), B, s);
-  Scratch tl = tile_leaves(P, B.toff.as<int64_t>(), P.n_active_leaves, B.total, s);
-  if (P.prec == LENS_FP32_BULK) {
-    eval32_rays(P, rays, B.off.as<int64_t>(), B.perm.as<int>(), tl.as<int2>(), B.total, y, jac, s);
-    return;
+  bucket_rays(P, rays, m, (f64 ? kEvalThreads : kEval32Threads) * rpt, B, s);
+  Scratch tl = tile_leaves(P, B.toff, P.n_active_leaves, B.tiles_max, s);
+  if (f64) {
+    wait_expansions(P, s);
+    EvalArgs A = base_args(P);
+    A.tile_leaf = tl.as<int2>();
+    A.rays = rays; A.ray_off = B.off; A.perm = B.perm.as<int>();
+    A.y = y; A.jac = jac;
+    launch_eval<false, false>(P, A, B.tiles_max, jac != nullptr, s);
+  } else {
+    eval32_rays(P, rays, B.off, B.perm.as<int>(), tl.as<int2>(), B.tiles_max, y, jac, s);
   }
-  wait_expansions(P, s);
-  EvalArgs A = base_args(P);
-  A.tile_leaf = tl.as<int2>();
-  A.rays = rays; A.ray_off = B.off.as<int64_t>(); A.perm = B.perm.as<int>();
-  A.y = y; A.jac = jac;
-  launch_eval<false, false>(P, A, B.total, jac != nullptr, s);
+  check_rays(B);
 }
 
 }  // namespace lens

@@ -38,10 +38,9 @@ namespace lens {
 namespace {
 
 constexpr int kT = kEval32Threads;
-constexpr int kRpt = kEval32Rpt;
+constexpr int kRpt = 4;    // rays per thread of the fused map kernel
 constexpr int kGroup = 8;  // stars per float32 partial sum of the near field
 constexpr int kChunk = 512;
-static_assert(kRpt % 2 == 0, "rays are paired for float2 arithmetic");
 constexpr int kWChunk = 8;
 
 struct E32Args {
@@ -137,15 +136,15 @@ __device__ __forceinline__ void stage_stars(E32Smem& sm, const E32Args& A, int64
 // unused): d = (x - s_hi) - s_lo, one paired add fewer per coordinate.  A
 // padding star then lies ~1e18 / h away: its |d|^2 may overflow to infinity,
 // whose reciprocal 0 still makes its term exactly zero.
-template <bool UM, bool GU = false>
-__device__ __forceinline__ void p2p_paired(const E32Smem& sm, int nfg, const float (&dx)[kRpt],
-                                           const float (&dy)[kRpt], const float (&dxl)[kRpt],
-                                           const float (&dyl)[kRpt], fcomp2 (&N1)[kRpt / 2],
-                                           fcomp2 (&N2)[kRpt / 2]) {
+template <bool UM, bool GU = false, int R>
+__device__ __forceinline__ void p2p_paired(const E32Smem& sm, int nfg, const float (&dx)[R],
+                                           const float (&dy)[R], const float (&dxl)[R],
+                                           const float (&dyl)[R], fcomp2 (&N1)[R / 2],
+                                           fcomp2 (&N2)[R / 2]) {
   for (int lo = 0; lo < nfg; lo += kGroup) {
-    float2 P1[kRpt / 2], P2[kRpt / 2], DX[kRpt / 2], DY[kRpt / 2], DXL[kRpt / 2], DYL[kRpt / 2];
+    float2 P1[R / 2], P2[R / 2], DX[R / 2], DY[R / 2], DXL[R / 2], DYL[R / 2];
 #pragma unroll
-    for (int h = 0; h < kRpt / 2; ++h) {
+    for (int h = 0; h < R / 2; ++h) {
       P1[h] = make_float2(0.f, 0.f); P2[h] = make_float2(0.f, 0.f);
       DX[h] = make_float2(dx[2 * h], dx[2 * h + 1]); DY[h] = make_float2(dy[2 * h], dy[2 * h + 1]);
       DXL[h] = make_float2(dxl[2 * h], dxl[2 * h + 1]); DYL[h] = make_float2(dyl[2 * h], dyl[2 * h + 1]);
@@ -156,7 +155,7 @@ __device__ __forceinline__ void p2p_paired(const E32Smem& sm, int nfg, const flo
       const int j = lo + jj;
       const float2 nsx = sm.s_x[j], nsy = sm.s_y[j], nsxl = sm.s_xl[j], nsyl = sm.s_yl[j];
 #pragma unroll
-      for (int h = 0; h < kRpt / 2; ++h) {
+      for (int h = 0; h < R / 2; ++h) {
         const float2 d1 = GU ? __fadd2_rn(__fadd2_rn(DX[h], nsx), nsxl)
                              : __fadd2_rn(__fadd2_rn(DX[h], nsx), __fadd2_rn(DXL[h], nsxl));
         const float2 d2 = GU ? __fadd2_rn(__fadd2_rn(DY[h], nsy), nsyl)
@@ -170,7 +169,7 @@ __device__ __forceinline__ void p2p_paired(const E32Smem& sm, int nfg, const flo
       }
     }
 #pragma unroll
-    for (int h = 0; h < kRpt / 2; ++h) {
+    for (int h = 0; h < R / 2; ++h) {
       N1[h].add(P1[h]);
       N2[h].add(P2[h]);
     }
@@ -192,15 +191,16 @@ __device__ __forceinline__ void stage_w(E32Smem& sm, const E32Args& A, int64_t e
 
 // M2P of the nw staged W boxes, rays (2h, 2h+1) side by side: Horner's rule
 // for f(z) = (1/z) sum_k A_k (r/z)^k, 4 paired multiply-adds per order.
-__device__ __forceinline__ void m2p_paired(const E32Smem& sm, int nw, int p, const float (&dx)[kRpt],
-                                           const float (&dy)[kRpt], float2 (&FX)[kRpt / 2],
-                                           float2 (&FY)[kRpt / 2]) {
+template <int R>
+__device__ __forceinline__ void m2p_paired(const E32Smem& sm, int nw, int p, const float (&dx)[R],
+                                           const float (&dy)[R], float2 (&FX)[R / 2],
+                                           float2 (&FY)[R / 2]) {
   for (int w = 0; w < nw; ++w) {
     const float4 gw = sm.s_wg[w];
     const float2 ngx = make_float2(-gw.x, -gw.x), ngy = make_float2(-gw.y, -gw.y);
     const float2 gr = make_float2(gw.z, gw.z), ngr = make_float2(-gw.z, -gw.z);
 #pragma unroll
-    for (int h = 0; h < kRpt / 2; ++h) {
+    for (int h = 0; h < R / 2; ++h) {
       const float2 zx = __fadd2_rn(make_float2(dx[2 * h], dx[2 * h + 1]), ngx);
       const float2 zy = __fadd2_rn(make_float2(dy[2 * h], dy[2 * h + 1]), ngy);
       const float2 n2 = __ffma2_rn(zx, zx, __fmul2_rn(zy, zy));
@@ -228,10 +228,10 @@ __device__ __forceinline__ void m2p_paired(const E32Smem& sm, int nw, int p, con
 // side by side: T1 = a dx - Re f - near1, T2 = b dy + Im f - near2 (y minus
 // the leaf's float64 constant; alpha = conj(b0 + f + near)).
 // (GU: the near-field sums are in grid units and take the factor 1/h here.)
-template <bool GU = false>
+template <bool GU = false, int R>
 __device__ __forceinline__ void l2p_lens_pair(const E32Smem& sm, const E32Args& A, float ir, int h,
-                                              const float (&dx)[kRpt], const float (&dy)[kRpt],
-                                              const float (&dxl)[kRpt], const float (&dyl)[kRpt],
+                                              const float (&dx)[R], const float (&dy)[R],
+                                              const float (&dxl)[R], const float (&dyl)[R],
                                               const fcomp2& N1h, const fcomp2& N2h, float2 FXh,
                                               float2 FYh, ff2& T1, ff2& T2) {
   const int p = A.p;
@@ -311,13 +311,24 @@ __device__ __forceinline__ void grid_offset(const E32Args& A, const LeafGrid& lg
   dy = oy.hi; dyl = oy.lo;
 }
 
-// Arbitrary rays, and grid rays with the Jacobian (without it: k_eval_quads).
-template <bool JAC, bool GRID, bool UM = false>
+// a b with the contraction written out (left to the compiler it varies with the
+// kernel's other parameters); CROSS: which cross product is rounded first
+template <bool CROSS>
+__device__ __forceinline__ float2 cmul_fma(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -(a.y * b.y)),
+                     CROSS ? fmaf(a.y, b.x, a.x * b.y) : fmaf(a.x, b.y, a.y * b.x));
+}
+
+// Arbitrary rays, and grid rays with the Jacobian (without it: k_eval_quads), R
+// rays a thread.
+template <bool JAC, bool GRID, int R, bool UM = false>
 __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
+  static_assert(JAC || R % 2 == 0, "rays are paired without the Jacobian");
   __shared__ E32Smem sm;
   const int tid = threadIdx.x;
   const int p = A.p;
   const int2 kt = A.tile_leaf[blockIdx.x];
+  if (kt.x < 0) return;
   const int64_t k = kt.x;
   const int64_t tile = kt.y;
   const LeafPlan lp = A.leaf[k];
@@ -334,26 +345,27 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
     nr_leaf = A.ray_off[k + 1] - A.ray_off[k];
   }
   static_assert(JAC || !GRID, "grid rays without the Jacobian run k_eval_quads");
-  float dx[kRpt], dy[kRpt], dxl[kRpt], dyl[kRpt];
-  int64_t oidx[kRpt];
-  bool ok[kRpt];
-  fcomp n1[kRpt], n2[kRpt], nj1[kRpt], nj2[kRpt];
-  fcomp2 N1[kRpt / 2], N2[kRpt / 2];  // paired accumulators of the Jacobian-free path
+  float dx[R], dy[R], dxl[R], dyl[R];
+  int64_t oidx[R];
+  bool ok[R];
+  fcomp n1[R], n2[R], nj1[R], nj2[R];
+  constexpr int H = JAC ? 1 : R / 2;
+  fcomp2 N1[H], N2[H];  // paired accumulators of the Jacobian-free path
 #pragma unroll
-  for (int h = 0; h < kRpt / 2; ++h) {
+  for (int h = 0; h < H; ++h) {
     N1[h] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     N2[h] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   }
-  // A tile holds up to kT kRpt rays; a partial one (a leaf's last tile, or a
+  // A tile holds up to kT R rays; a partial one (a leaf's last tile, or a
   // leaf of few rays) lays them out with stride S, a multiple of 32, so that
   // they fill whole warps: slot q of thread t is ray q S + t of the tile, and a
   // warp with no ray (t >= S) joins the block's staging but skips the sums.
-  const int64_t tbase = tile * (int64_t)(kT * kRpt);
-  const int nt = (int)min64(kT * kRpt, nr_leaf - tbase);
-  const int S = min(kT, ((nt + kRpt - 1) / kRpt + 31) & ~31);
+  const int64_t tbase = tile * (int64_t)(kT * R);
+  const int nt = (int)min64(kT * R, nr_leaf - tbase);
+  const int S = min(kT, ((nt + R - 1) / R + 31) & ~31);
   const bool live = (tid & ~31) < S;
 #pragma unroll
-  for (int q = 0; q < kRpt; ++q) {
+  for (int q = 0; q < R; ++q) {
     const int64_t loc = tbase + (int64_t)q * S + tid;
     ok[q] = tid < S && loc < nr_leaf;
     dx[q] = dy[q] = dxl[q] = dyl[q] = 0.f;
@@ -393,16 +405,16 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
       p2p_paired<UM>(sm, nfg, dx, dy, dxl, dyl, N1, N2);
     } else {
       for (int lo = 0; lo < nfg; lo += kGroup) {
-        float p1[kRpt], p2[kRpt], pj1[kRpt], pj2[kRpt];
+        float p1[R], p2[R], pj1[R], pj2[R];
 #pragma unroll
-        for (int q = 0; q < kRpt; ++q) { p1[q] = 0.f; p2[q] = 0.f; pj1[q] = 0.f; pj2[q] = 0.f; }
+        for (int q = 0; q < R; ++q) { p1[q] = 0.f; p2[q] = 0.f; pj1[q] = 0.f; pj2[q] = 0.f; }
 #pragma unroll
         for (int jj = 0; jj < kGroup; ++jj) {
           const int j = lo + jj;
           const float sx = -sm.s_x[j].x, sy = -sm.s_y[j].x, sxl = -sm.s_xl[j].x, syl = -sm.s_yl[j].x;
           const float smm = sm.s_m[j].x;
 #pragma unroll
-          for (int q = 0; q < kRpt; ++q) {
+          for (int q = 0; q < R; ++q) {
             const float d1 = (dx[q] - sx) + (dxl[q] - sxl);
             const float d2 = (dy[q] - sy) + (dyl[q] - syl);
             // a star exactly on the ray contributes nothing (w * w would
@@ -418,7 +430,7 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
           }
         }
 #pragma unroll
-        for (int q = 0; q < kRpt; ++q) {
+        for (int q = 0; q < R; ++q) {
           n1[q].add(p1[q]); n2[q].add(p2[q]);
           nj1[q].add(pj1[q]); nj2[q].add(pj2[q]);
         }
@@ -430,7 +442,7 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
     if (A.m0 != 1.f) {
       const float2 m2 = make_float2(A.m0, A.m0);
 #pragma unroll
-      for (int h = 0; h < kRpt / 2; ++h) {
+      for (int h = 0; h < H; ++h) {
         N1[h].hi = __fmul2_rn(N1[h].hi, m2); N1[h].lo = __fmul2_rn(N1[h].lo, m2);
         N2[h].hi = __fmul2_rn(N2[h].hi, m2); N2[h].lo = __fmul2_rn(N2[h].lo, m2);
       }
@@ -438,12 +450,12 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
   }
 
   // ---- M2P over the far W boxes --------------------------------------------
-  float2 fw[kRpt], dfw[kRpt];
+  float2 fw[R], dfw[R];
 #pragma unroll
-  for (int q = 0; q < kRpt; ++q) { fw[q] = make_float2(0.f, 0.f); dfw[q] = make_float2(0.f, 0.f); }
-  float2 FX[kRpt / 2], FY[kRpt / 2];
+  for (int q = 0; q < R; ++q) { fw[q] = make_float2(0.f, 0.f); dfw[q] = make_float2(0.f, 0.f); }
+  float2 FX[H], FY[H];
 #pragma unroll
-  for (int h = 0; h < kRpt / 2; ++h) { FX[h] = make_float2(0.f, 0.f); FY[h] = make_float2(0.f, 0.f); }
+  for (int h = 0; h < H; ++h) { FX[h] = make_float2(0.f, 0.f); FY[h] = make_float2(0.f, 0.f); }
   const int64_t w_beg = A.woff[k], w_end = A.woff[k + 1];
   for (int64_t e0 = w_beg; e0 < w_end; e0 += kWChunk) {
     const int nw = (int)min64(kWChunk, w_end - e0);
@@ -451,13 +463,13 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
     stage_w(sm, A, e0, nw, tid);
     __syncthreads();
     if (!live) continue;
-    if (!JAC) {
+    if constexpr (!JAC) {
       m2p_paired(sm, nw, p, dx, dy, FX, FY);
     } else {
       for (int w = 0; w < nw; ++w) {
         const float4 gw = sm.s_wg[w];
 #pragma unroll
-        for (int q = 0; q < kRpt; ++q) {
+        for (int q = 0; q < R; ++q) {
           const float2 z = make_float2(dx[q] - gw.x, dy[q] - gw.y);
           const float2 inv = cinv(z);
           const float2 qq = make_float2(inv.x * gw.z, inv.y * gw.z);
@@ -467,7 +479,7 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
           float2 t = make_float2((float)(p + 1) * sm.s_Wx[w][p].x, (float)(p + 1) * sm.s_Wy[w][p].x);
           for (int kk = p - 1; kk >= 0; --kk)
             t = cfma(t, qq, make_float2((float)(kk + 1) * sm.s_Wx[w][kk].x, (float)(kk + 1) * sm.s_Wy[w][kk].x));
-          const float2 dd = cmul(t, cmul(inv, inv));
+          const float2 dd = cmul_fma<GRID>(t, cmul_fma<false>(inv, inv));
           dfw[q] = make_float2(dfw[q].x - dd.x, dfw[q].y - dd.y);
         }
       }
@@ -480,7 +492,7 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
   const float ir = lp.ir;
   if constexpr (!JAC) {
 #pragma unroll
-    for (int h = 0; h < kRpt / 2; ++h) {
+    for (int h = 0; h < H; ++h) {
       ff2 T1, T2;
       l2p_lens_pair<false>(sm, A, ir, h, dx, dy, dxl, dyl, N1[h], N2[h], FX[h], FY[h], T1, T2);
 #pragma unroll
@@ -496,7 +508,7 @@ __global__ void __launch_bounds__(kT, 7) k_eval32(E32Args A) {
   } else {
     // with the Jacobian: one ray at a time
 #pragma unroll
-    for (int q = 0; q < kRpt; ++q) {
+    for (int q = 0; q < R; ++q) {
       if (!ok[q]) continue;
       float2 f = make_float2(0.f, 0.f), df = make_float2(0.f, 0.f);
       if (p >= 1) {
@@ -1157,9 +1169,10 @@ void launch32_rays(E32Args& A, int64_t total, bool jac, cudaStream_t s) {
   if (total <= 0) return;
   if (total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
   const unsigned g = (unsigned)total;
-  if (jac) k_eval32<true, false><<<g, kT, 0, s>>>(A);
-  else if (A.unit_mass) k_eval32<false, false, true><<<g, kT, 0, s>>>(A);
-  else k_eval32<false, false><<<g, kT, 0, s>>>(A);
+  constexpr int RJ = eval32_rays_per_thread(true), R = eval32_rays_per_thread(false);
+  if (jac) k_eval32<true, false, RJ><<<g, kT, 0, s>>>(A);
+  else if (A.unit_mass) k_eval32<false, false, R, true><<<g, kT, 0, s>>>(A);
+  else k_eval32<false, false, R><<<g, kT, 0, s>>>(A);
   LENS_LAUNCHED("k_eval32");
 }
 
@@ -1168,7 +1181,7 @@ void launch32_grid(E32Args& A, int64_t total, cudaStream_t s) {
   if (total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
   const unsigned g = (unsigned)total;
   if (A.jac) {
-    k_eval32<true, true><<<g, kT, 0, s>>>(A);
+    k_eval32<true, true, eval32_rays_per_thread(true)><<<g, kT, 0, s>>>(A);
     LENS_LAUNCHED("k_eval32");
     return;
   }

@@ -65,12 +65,23 @@ struct Scratch {
   template <class T> T* as() const { return static_cast<T*>(p); }
 };
 
+// A few words of host memory that kernels write through the mapped pointer: the
+// read-back of a size or a flag is then one kernel's store and one wait instead
+// of a copy on top.  One block per host thread (kept until the thread ends),
+// handed out in turn; a slot is read before kHostSlots later ones are taken,
+// since every call that takes one waits for it before it returns.
+constexpr int kHostSlots = 64, kHostSlotWords = 80;
+struct HostSlot {
+  volatile int64_t* host;  // kHostSlotWords words
+  int64_t* dev;
+};
+HostSlot host_slot();
+
 constexpr int kMaxDepth = 28;   // quadtree levels below the root (56-bit keys)
 constexpr int kMaxOrder = 64;   // expansion order cap
 
-// Float32 evaluation kernel geometry (eval32.cu): threads per CTA, rays per thread.
+// Float32 evaluation kernel geometry (eval32.cu): threads per CTA.
 constexpr int kEval32Threads = 128;
-constexpr int kEval32Rpt = 4;
 
 // Per active leaf, float64 constants formed once per plan (eval32.cu).
 struct LeafPlan {
@@ -261,17 +272,30 @@ struct GridRows {  // a band of corner rows of a grid
 void evaluate_grid(Plan& P, const GridRows& g, double* y, double* jac, cudaStream_t s);
 void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* jac,
                    cudaStream_t s);
-// Rays bucketed by active leaf: perm (ray ids in leaf order), off (per leaf,
-// CSR into perm), toff (per leaf, first tile of `tile` rays) and slot (per ray,
-// its leaf).
+// Rays bucketed by active leaf: perm (ray ids in leaf order), slot (per ray, its
+// leaf), off (per leaf, CSR into perm; off[nl] = rays in a leaf) and toff (per
+// leaf, first tile of `tile` rays; toff[nl] = tiles, at most tiles_max).  Nothing
+// is read back: a launch over tiles covers tiles_max and its blocks past
+// toff[nl] return, and check_rays(), called once the work is launched, waits until
+// every ray has its leaf (not for the work) and fails if one lies outside the
+// target region.
 struct RayBuckets {
-  Scratch perm, off, toff, slot;
-  int64_t total = 0;  // tiles
+  Scratch mem, perm, slot;
+  const int64_t* off = nullptr;
+  const int64_t* toff = nullptr;
+  int64_t tiles_max = 0;
+  HostSlot flag{};
+  cudaEvent_t leaves_known = nullptr;  // every ray has its leaf (or raised the flag)
+  RayBuckets() = default;
+  RayBuckets(const RayBuckets&) = delete;
+  RayBuckets& operator=(const RayBuckets&) = delete;
+  ~RayBuckets() { if (leaves_known) cudaEventDestroy(leaves_known); }
 };
-// (leaf, tile within the leaf) of each of `total` tiles (toff: exclusive scan of
-// the leaves' tile counts)
-Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s);
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s);
+void check_rays(const RayBuckets& B);
+// (leaf, tile within the leaf) of each of `total` tiles (toff: exclusive scan of
+// the leaves' tile counts, toff[nl] their sum; a tile past it gets leaf -1)
+Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s);
 
 struct IpmParams {
   double u0, v0, inv_du, inv_dv;  // source-plane window origin, inverse pixel size
@@ -325,6 +349,12 @@ void wait_tree(Plan& P, cudaStream_t s);
 void eval32_grid(Plan& P, const GridRows& g, const int64_t* rect, const int2* tile_leaf,
                  int64_t total, double* y, double* jac, PixCorner* pix, const IpmParams* ip,
                  cudaStream_t s);
+// Rays per thread of k_eval32 (float32 ray path, grid rays with the Jacobian).
+// One with the Jacobian, a pair without, whatever the number of rays: four a thread
+// spilled registers and left leaves of ~100 rays to one warp (1e4 stars, 2e4 rays, with the
+// Jacobian 36 us, one a thread 11; 3e5 stars, 1e6 rays: 399 -> 251 us a call, without it
+// 214 -> 187).
+constexpr int eval32_rays_per_thread(bool jac) { return jac ? 1 : 2; }
 void eval32_rays(Plan& P, const double* rays, const int64_t* off, const int* perm,
                  const int2* tile_leaf, int64_t total, double* y, double* jac, cudaStream_t s);
 // The fused deflection + IPM path (eval32.cu, float32-bulk plans).  A work
