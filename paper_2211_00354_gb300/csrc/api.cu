@@ -456,23 +456,30 @@ lens_status lens_ipm_map_ex(lens_plan* plan, const lens_grid* grid, const lens_b
   cudaStream_t s = S(stream);
   P.da.stream = s;
   const int64_t nx = grid->nx, ny = grid->ny;
-  int64_t max_cells = max_cells_per_chunk;
-  if (max_cells == 0) {
-    size_t fr = 0, tot = 0;
-    LENS_CUDA(cudaMemGetInfo(&fr, &tot));
-    // 16 B per corner + 4 B queue slot per cell, within a quarter of free memory
-    max_cells = (int64_t)std::min<double>((double)fr / 4.0 / 20.0, (double)(1ll << 30));
-  }
-  max_cells = std::min<int64_t>(max_cells, 1ll << 30);
   // The float32 accumulators are flushed into the float64 map once about
   // kFlushCellsPerPixel cells per map pixel have entered them, so a pixel
   // sums a bounded number of float32 increments whatever the grid size
   // (a pixel under n equal increments drifts by up to ~n 2^-25 relative).
   constexpr int64_t kFlushCellsPerPixel = 64;
   const int64_t flush_cells = std::min<int64_t>(kFlushCellsPerPixel * npx * npy, 1ll << 30);
-  max_cells = std::min(max_cells, flush_cells);
-  int64_t rows = std::max<int64_t>(1, max_cells / nx);
-  rows = std::min<int64_t>(rows, ny);
+  const auto rows_for = [&](int64_t max_cells) {
+    max_cells = std::min(std::min<int64_t>(max_cells, 1ll << 30), flush_cells);
+    return std::min<int64_t>(std::max<int64_t>(1, max_cells / nx), ny);
+  };
+  const auto rows_from_memory = [&]() {
+    size_t fr = 0, tot = 0;
+    LENS_CUDA(cudaMemGetInfo(&fr, &tot));
+    // 16 B per corner + 4 B queue slot per cell, within a quarter of free memory
+    return rows_for((int64_t)std::min<double>((double)fr / 4.0 / 20.0, (double)(1ll << 30)));
+  };
+  // A grid (or the part of it between flushes) of at most kSmallCells cells, 84 MB,
+  // is taken at once: the query of the free memory costs the host as much as
+  // a few launches, and is made only if the buffers are then not to be had.
+  constexpr int64_t kSmallCells = 1 << 22;
+  const bool unasked = max_cells_per_chunk == 0 && std::min(flush_cells, nx * ny) <= kSmallCells;
+  int64_t rows = max_cells_per_chunk ? rows_for(max_cells_per_chunk)
+                 : unasked           ? rows_for(1ll << 30)
+                                     : rows_from_memory();
   need(rows * nx <= (1ll << 30) || rows == 1, "grid rows too wide for one chunk");
 
   IpmParams ip{};
@@ -484,8 +491,18 @@ lens_status lens_ipm_map_ex(lens_plan* plan, const lens_grid* grid, const lens_b
   ip.scale = ip.a_cell / ip.s_star;
   ip.npx = npx; ip.npy = npy; ip.cap = bbox_cap_px;
 
-  Scratch corners(&P.da, sizeof(PixCorner) * (size_t)(rows + 1) * (size_t)(nx + 1));
-  Scratch queue(&P.da, sizeof(int) * (size_t)rows * (size_t)nx + sizeof(int) * 4);
+  Scratch corners, queue;
+  for (bool again = unasked;; again = false) {
+    try {
+      corners = Scratch(&P.da, sizeof(PixCorner) * (size_t)(rows + 1) * (size_t)(nx + 1));
+      queue = Scratch(&P.da, sizeof(int) * (size_t)rows * (size_t)nx + sizeof(int) * 4);
+      break;
+    } catch (const Error& e) {
+      if (!again || e.status != LENS_ENOMEM) throw;
+      corners.reset();
+      rows = rows_from_memory();
+    }
+  }
   Scratch sdev(&P.da, sizeof(double) * 16);
   // the map accumulates in float32 (increments are O(1) and a pixel receives
   // ~mu n_0 of them; float32 keeps ~1e-6 relative) and is written out in
@@ -587,8 +604,9 @@ lens_status lens_ipm_map_ex(lens_plan* plan, const lens_grid* grid, const lens_b
   ipm_finish_map(map32.as<float>(), rowdiff.as<float>(), npx, npy, map_out, flushed, false, s);
   mark();
   double hs[16];
-  LENS_CUDA(cudaMemcpyAsync(hs, sdev.p, sizeof(hs), cudaMemcpyDeviceToHost, s));
-  LENS_CUDA(cudaStreamSynchronize(s));
+  int64_t hw[16];
+  read_words(sdev.as<int64_t>(), 16, hw, s);
+  std::memcpy(hs, hw, sizeof(hs));
   double msd = 0, msi = 0;
   for (size_t k = 0; k + 1 < ev.size(); ++k) {
     float ms = 0;

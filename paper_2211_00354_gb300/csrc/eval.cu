@@ -540,11 +540,11 @@ void grid_impl(Plan& P, const GridRows& g, double* y, double* jac, PixCorner* pi
                                                  g.nrows, tile, quads, rect.as<int64_t>(),
                                                  tiles.as<int64_t>());
   LENS_LAUNCHED("k_grid_rects");
-  LENS_CUDA(cudaMemsetAsync(tiles.as<int64_t>() + nl, 0, sizeof(int64_t), s));
-  exclusive_scan_i64(tiles.as<int64_t>(), toff.as<int64_t>(), nl + 1, P.da, s);
+  const ScanJob job{tiles.as<int64_t>(), toff.as<int64_t>()};
+  exclusive_scans(&job, 1, nl, P.da, s);
   int64_t total = 0;
-  LENS_CUDA(cudaMemcpyAsync(&total, toff.as<int64_t>() + nl, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  LENS_CUDA(cudaStreamSynchronize(s));
+  const int64_t* addr[1] = {toff.as<int64_t>() + nl};
+  read_i64(addr, 1, &total, s);
   if (P.work) {
     k_work_count<<<grid_for(nl, 128, 1024), 128, 0, s>>>(P.active_leaves, nl, P.box_aidx,
                                                         rect.as<int64_t>(), P.ustar_cnt,

@@ -966,24 +966,6 @@ __global__ void k_fuse_fill(const int64_t* __restrict__ rect, int64_t nl, int64_
 }
 
 // ---- plan-time preparation ---------------------------------------------------
-// per active leaf: centre, 1/r, r (the tree alone)
-__global__ void k_prep_leaf_geo(const int* __restrict__ leaves, int64_t nl,
-                                const int* __restrict__ level, const int* __restrict__ ix,
-                                const int* __restrict__ iy, double lo_x, double lo_y, double size,
-                                LeafPlan* __restrict__ out) {
-  const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (k >= nl) return;
-  const int B = leaves[k];
-  const double r = size / (double)(2ull << level[B]);
-  LeafPlan lp;
-  lp.cx = lo_x + (2.0 * ix[B] + 1.0) * r;
-  lp.cy = lo_y + (2.0 * iy[B] + 1.0) * r;
-  lp.K1 = 0.0; lp.K2 = 0.0;
-  lp.ir = (float)(1.0 / r);
-  lp.r = (float)r;
-  out[k] = lp;
-}
-
 // per active leaf: the lens equation at the centre with the constant term of
 // the local expansion, and the float32 local coefficients (the expansions)
 __global__ void k_prep_leaf_exp(const int* __restrict__ leaves, int64_t nl, double a, double b,
@@ -1004,16 +986,28 @@ __global__ void k_prep_leaf_exp(const int* __restrict__ leaves, int64_t nl, doub
 // operations per star against ~4(p+1) + 25 for one M2P.
 inline int w_direct_max(int p) { return std::max(1, (p + 1) / 2); }
 
-// Per active leaf: near boxes (U list + small W boxes), their stars, and the
-// far W boxes.
+// Per active leaf: centre, 1/r, r; near boxes (U list + small W boxes), their
+// stars, and the far W boxes.
 __global__ void k_prep_counts(const int* __restrict__ leaves, int64_t nl, const int* __restrict__ aidx,
+                              const int* __restrict__ level, const int* __restrict__ ix,
+                              const int* __restrict__ iy, double lo_x, double lo_y, double size,
+                              LeafPlan* __restrict__ out,
                               const int64_t* __restrict__ W_off,
                               const int* __restrict__ W_list, const int* __restrict__ count,
                               const int64_t* __restrict__ ustar_cnt, int wmax,
                               int64_t* __restrict__ scnt, int64_t* __restrict__ wcnt) {
   const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (k >= nl) return;
-  const int a = aidx[leaves[k]];
+  const int B = leaves[k];
+  const double r = size / (double)(2ull << level[B]);
+  LeafPlan lp;
+  lp.cx = lo_x + (2.0 * ix[B] + 1.0) * r;
+  lp.cy = lo_y + (2.0 * iy[B] + 1.0) * r;
+  lp.K1 = 0.0; lp.K2 = 0.0;
+  lp.ir = (float)(1.0 / r);
+  lp.r = (float)r;
+  out[k] = lp;
+  const int a = aidx[B];
   int64_t ns = ustar_cnt[a], nw = 0;
   for (int64_t e = W_off[a]; e < W_off[a + 1]; ++e) {
     const int c = count[W_list[e]];
@@ -1213,21 +1207,16 @@ void eval32_prepare_tree(Plan& P, cudaStream_t s) {
   const int64_t nl = P.n_active_leaves;
   if (nl == 0) return;
   const int wmax = w_direct_max(P.p);
-  k_prep_leaf_geo<<<grid_for(nl, 128), 128, 0, s>>>(P.active_leaves, nl, P.box_level, P.box_ix,
-                                                    P.box_iy, P.root_lo[0], P.root_lo[1],
-                                                    P.root_size, P.f_leaf);
-  LENS_LAUNCHED("k_prep_leaf_geo");
-  LENS_CUDA(cudaMemsetAsync(P.f_ncnt, 0, sizeof(int64_t) * (nl + 1), s));
-  LENS_CUDA(cudaMemsetAsync(P.f_wcnt, 0, sizeof(int64_t) * (nl + 1), s));
-  k_prep_counts<<<grid_for(nl, 128), 128, 0, s>>>(P.active_leaves, nl, P.box_aidx, P.W_off,
-                                                  P.W_list, P.box_count, P.ustar_cnt, wmax,
+  k_prep_counts<<<grid_for(nl, 128), 128, 0, s>>>(P.active_leaves, nl, P.box_aidx, P.box_level,
+                                                  P.box_ix, P.box_iy, P.root_lo[0], P.root_lo[1],
+                                                  P.root_size, P.f_leaf, P.W_off, P.W_list, P.box_count, P.ustar_cnt, wmax,
                                                   P.f_ncnt, P.f_wcnt);
   LENS_LAUNCHED("k_prep_counts");
-  exclusive_scan_i64(P.f_ncnt, P.f_uoff, nl + 1, P.da, s);
-  exclusive_scan_i64(P.f_wcnt, P.f_woff, nl + 1, P.da, s);
+  const ScanJob jobs[2] = {{P.f_ncnt, P.f_uoff}, {P.f_wcnt, P.f_woff}};
+  exclusive_scans(jobs, 2, nl, P.da, s);
   int64_t tot[2] = {0, 0};
   const int64_t* addr[2] = {P.f_uoff + nl, P.f_woff + nl};
-  read_i64(addr, 2, tot, P.da, s);
+  read_i64(addr, 2, tot, s);
   P.f_ust = P.dalloc_n<float4>(tot[0]);
   P.f_um = P.dalloc_n<float>(tot[0]);
   P.f_wlist = P.dalloc_n<int>(tot[1]);
@@ -1298,16 +1287,14 @@ Scratch eval32_fused(Plan& P, const GridRows& g, const int64_t* rect, PixCorner*
   const int64_t jlast = g.row0 + g.nrows - 2;  // the chunk's last cell row
   Scratch cnt(&P.da, sizeof(int64_t) * (nl + 1)), scnt(&P.da, sizeof(int64_t) * (nl + 1));
   Scratch ioff(&P.da, sizeof(int64_t) * (nl + 1)), soff(&P.da, sizeof(int64_t) * (nl + 1));
-  LENS_CUDA(cudaMemsetAsync(cnt.as<int64_t>() + nl, 0, sizeof(int64_t), s));
-  LENS_CUDA(cudaMemsetAsync(scnt.as<int64_t>() + nl, 0, sizeof(int64_t), s));
   k_fuse_count<<<grid_for(nl, 128), 128, 0, s>>>(rect, nl, g.nx, jlast, cnt.as<int64_t>(),
                                                  scnt.as<int64_t>());
   LENS_LAUNCHED("k_fuse_count");
-  exclusive_scan_i64(cnt.as<int64_t>(), ioff.as<int64_t>(), nl + 1, P.da, s);
-  exclusive_scan_i64(scnt.as<int64_t>(), soff.as<int64_t>(), nl + 1, P.da, s);
+  const ScanJob jobs[2] = {{cnt.as<int64_t>(), ioff.as<int64_t>()}, {scnt.as<int64_t>(), soff.as<int64_t>()}};
+  exclusive_scans(jobs, 2, nl, P.da, s);
   int64_t tot[2] = {0, 0};
   const int64_t* addr[2] = {ioff.as<int64_t>() + nl, soff.as<int64_t>() + nl};
-  read_i64(addr, 2, tot, P.da, s);
+  read_i64(addr, 2, tot, s);
   const int64_t nitems = tot[0];
   nseam = tot[1];
   if (nitems > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many work items in one chunk");

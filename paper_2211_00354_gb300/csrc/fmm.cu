@@ -385,32 +385,37 @@ void fmm_tables(Plan& P, cudaStream_t s) {
   FmmTables& t = P.tab;
   t.p = p;
   t.ldb = p + 2;
+  std::vector<double> t_bin((size_t)(2 * p + 2) * t.ldb, 0.0);
   const int nb = 2 * p + 2;
-  std::vector<double> bin((size_t)nb * t.ldb, 0.0);
-  std::vector<std::vector<double>> full(nb, std::vector<double>(nb, 0.0));
+  const auto full = [&](int n, int k) -> double& { return t_bin[(size_t)n * t.ldb + k]; };
+  std::vector<double>& bin = t_bin;
+  // C(n, k), k < p + 2 (C(n, k) of row n needs only columns up to k of row n - 1)
   for (int n = 0; n < nb; ++n) {
-    full[n][0] = 1.0;
-    for (int k = 1; k <= n; ++k) full[n][k] = full[n - 1][k - 1] + (k <= n - 1 ? full[n - 1][k] : 0.0);
+    full(n, 0) = 1.0;
+    for (int k = 1; k <= n && k < t.ldb; ++k) full(n, k) = full(n - 1, k - 1) + (k <= n - 1 ? full(n - 1, k) : 0.0);
   }
-  for (int n = 0; n < nb; ++n)
-    for (int k = 0; k < t.ldb && k <= n; ++k) bin[(size_t)n * t.ldb + k] = full[n][k];
-  auto cpow = [](double re, double im, int e) {
+  // powers of the child offsets, by repeated products
+  std::vector<std::pair<double, double>> dpow((size_t)4 * P1), wpw((size_t)P1);
+  const auto powers = [&](double re, double im, std::pair<double, double>* out) {
     double pr = 1.0, pi = 0.0;
-    for (int i = 0; i < e; ++i) {
-      double nr = pr * re - pi * im, ni = pr * im + pi * re;
+    for (int i = 0; i <= p; ++i) {
+      out[i] = {pr, pi};
+      const double nr = pr * re - pi * im, ni = pr * im + pi * re;
       pr = nr; pi = ni;
     }
-    return std::pair<double, double>(pr, pi);
   };
+  powers(0.5, 0.5, wpw.data());
   std::vector<double2> m2m((size_t)4 * P1 * P1), l2l((size_t)4 * P1 * P1);
   for (int q = 0; q < 4; ++q) {
     const double dre = ((q & 1) ? 0.5 : -0.5), dim = ((q >> 1) ? 0.5 : -0.5);
+    const std::pair<double, double>* dq = dpow.data() + (size_t)q * P1;
+    powers(dre, dim, dpow.data() + (size_t)q * P1);
     for (int l = 0; l <= p; ++l)
       for (int k = 0; k <= p; ++k) {
         double2 v = make_double2(0.0, 0.0);
         if (k <= l) {
-          auto d = cpow(dre, dim, l - k);
-          const double c = full[l][k] * std::ldexp(1.0, -k);
+          const auto d = dq[l - k];
+          const double c = full(l, k) * std::ldexp(1.0, -k);
           v = make_double2(c * d.first, c * d.second);
         }
         m2m[((size_t)q * P1 + l) * P1 + k] = v;
@@ -419,8 +424,8 @@ void fmm_tables(Plan& P, cudaStream_t s) {
       for (int l = 0; l <= p; ++l) {
         double2 v = make_double2(0.0, 0.0);
         if (l >= j) {
-          auto d = cpow(dre, dim, l - j);
-          const double c = full[l][j] * std::ldexp(1.0, -j);
+          const auto d = dq[l - j];
+          const double c = full(l, j) * std::ldexp(1.0, -j);
           v = make_double2(c * d.first, c * d.second);
         }
         l2l[((size_t)q * P1 + j) * P1 + l] = v;
@@ -447,8 +452,7 @@ void fmm_tables(Plan& P, cudaStream_t s) {
   // ((1+i)/2)^k: Gaussian integers over powers of two, exact in float64
   std::vector<double2> wp((size_t)P1);
   for (int k = 0; k <= p; ++k) {
-    auto w = cpow(0.5, 0.5, k);
-    wp[(size_t)k] = make_double2(w.first, w.second);
+    wp[(size_t)k] = make_double2(wpw[(size_t)k].first, wpw[(size_t)k].second);
   }
   // one host block (kept in the plan until the copy has run: no wait here);
   // bin holds (2p+2)(p+2) doubles, an even count, so the complex tables

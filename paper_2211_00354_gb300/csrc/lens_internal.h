@@ -246,11 +246,20 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits,
                     DeviceAlloc& da, cudaStream_t s, int lo_bit = 0);
 void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, DeviceAlloc& da,
                         cudaStream_t s);
-// host[i] = *addrs[i] (device int64 values, n <= kMaxPick): one small kernel,
-// one copy and one synchronisation instead of a round trip per value (a
-// device-to-pageable copy returns only when it is done)
+// host[i] = *addrs[i] (device int64 values, n <= kMaxPick): one small kernel and
+// one synchronisation instead of a round trip per value
 constexpr int kMaxPick = 64;
-void read_i64(const int64_t* const* addrs, int n, int64_t* host, DeviceAlloc& da, cudaStream_t s);
+void read_i64(const int64_t* const* addrs, int n, int64_t* host, cudaStream_t s);
+// host[i] = dev[i], i < n <= kMaxPick, likewise
+void read_words(const int64_t* dev, int n, int64_t* host, cudaStream_t s);
+// out[i] = sum_{j<i} in[j], i = 0 .. n (n + 1 entries), for up to kMaxScanJobs
+// arrays of n entries; in and out differ
+constexpr int kMaxScanJobs = 8;
+struct ScanJob {
+  const int64_t* in;
+  int64_t* out;
+};
+void exclusive_scans(const ScanJob* jobs, int k, int64_t n, DeviceAlloc& da, cudaStream_t s);
 
 // Tree build in two halves: the boxes (bounds, keys, sort, splits: all the
 // upward pass needs), then the active boxes and the interaction lists.

@@ -376,7 +376,7 @@ void light_curve(const double* y, int64_t m, double w, const double* smp, int64_
   exclusive_scan_i64(cnt.as<int64_t>(), off.as<int64_t>(), nce + 1, da, s);
   int64_t near = 0;
   const int64_t* addr[1] = {off.as<int64_t>() + nce};
-  read_i64(addr, 1, &near, da, s);
+  read_i64(addr, 1, &near, s);
   Scratch yp(&da, sizeof(Pos) * (size_t)std::max<int64_t>(near, 1));
   k_lc_ray_fill<<<grid_for(m, 256), 256, 0, s>>>(y2, m, cellof.as<int>(), off.as<int64_t>(),
                                                   cur.as<unsigned long long>(), G, yp.as<Pos>());

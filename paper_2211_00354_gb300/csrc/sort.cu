@@ -259,6 +259,8 @@ void radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, DeviceA
 }
 
 // ---- batched read-back of int64 values ------------------------------------
+// The values are stored straight into the thread's mapped host words: no copy
+// after the kernel, one wait.
 namespace {
 struct PickArgs {
   const int64_t* src[kMaxPick];
@@ -270,17 +272,88 @@ __global__ void k_pick_i64(PickArgs a, int64_t* __restrict__ out) {
 }
 }  // namespace
 
-void read_i64(const int64_t* const* addrs, int n, int64_t* host, DeviceAlloc& da, cudaStream_t s) {
+void read_i64(const int64_t* const* addrs, int n, int64_t* host, cudaStream_t s) {
   if (n <= 0) return;
   if (n > kMaxPick) fail(LENS_EINVAL, "internal: too many values in one read-back");
   PickArgs a{};
   for (int i = 0; i < n; ++i) a.src[i] = addrs[i];
   a.n = n;
-  Scratch out(&da, sizeof(int64_t) * (size_t)n);
-  k_pick_i64<<<1, kMaxPick, 0, s>>>(a, out.as<int64_t>());
+  const HostSlot slot = host_slot();
+  k_pick_i64<<<1, kMaxPick, 0, s>>>(a, slot.dev);
   LENS_LAUNCHED("k_pick_i64");
-  LENS_CUDA(cudaMemcpyAsync(host, out.p, sizeof(int64_t) * (size_t)n, cudaMemcpyDeviceToHost, s));
   LENS_CUDA(cudaStreamSynchronize(s));
+  for (int i = 0; i < n; ++i) host[i] = slot.host[i];
+}
+
+namespace {
+__global__ void k_copy_words(const int64_t* __restrict__ in, int n, int64_t* __restrict__ out) {
+  if ((int)threadIdx.x < n) out[threadIdx.x] = in[threadIdx.x];
+}
+}  // namespace
+
+void read_words(const int64_t* dev, int n, int64_t* host, cudaStream_t s) {
+  if (n < 1 || n > kMaxPick) fail(LENS_EINVAL, "internal: too many values in one read-back");
+  const HostSlot slot = host_slot();
+  k_copy_words<<<1, kMaxPick, 0, s>>>(dev, n, slot.dev);
+  LENS_LAUNCHED("k_copy_words");
+  LENS_CUDA(cudaStreamSynchronize(s));
+  for (int i = 0; i < n; ++i) host[i] = slot.host[i];
+}
+
+// ---- several scans of the same length ---------------------------------------
+// out[j][i] = sum_{q<i} in[j][q] for i = 0 .. n, so out[j][n] is the total.  Up to
+// kOneBlockScan entries a block per array does it (a few steps of 4096; the tree
+// of a small field needs nine scans, three to seven launches each otherwise).
+namespace {
+constexpr int kMultiThreads = 1024, kMultiItems = 4;
+constexpr int64_t kOneBlockScan = 32768;
+struct ScanJobs {
+  ScanJob job[kMaxScanJobs];
+};
+__global__ void __launch_bounds__(kMultiThreads) k_scan_multi(ScanJobs jobs, int64_t n) {
+  __shared__ int64_t sh[32];
+  const int64_t* in = jobs.job[blockIdx.x].in;
+  int64_t* out = jobs.job[blockIdx.x].out;
+  int64_t base = 0;
+  for (int64_t i0 = 0; i0 < n; i0 += kMultiThreads * kMultiItems) {
+    const int64_t i = i0 + (int64_t)threadIdx.x * kMultiItems;
+    int64_t v[kMultiItems], t = 0;
+#pragma unroll
+    for (int q = 0; q < kMultiItems; ++q) {
+      v[q] = i + q < n ? in[i + q] : 0;
+      t += v[q];
+    }
+    int64_t total;
+    int64_t x = base + block_excl_scan(t, sh, total);
+#pragma unroll
+    for (int q = 0; q < kMultiItems; ++q) {
+      if (i + q < n) out[i + q] = x;
+      x += v[q];
+    }
+    base += total;
+  }
+  if (threadIdx.x == 0) out[n] = base;
+}
+__global__ void k_scan_total(const int64_t* in, int64_t* out, int64_t n) {
+  out[n] = n ? out[n - 1] + in[n - 1] : 0;
+}
+}  // namespace
+
+void exclusive_scans(const ScanJob* jobs, int k, int64_t n, DeviceAlloc& da, cudaStream_t s) {
+  if (k < 1 || k > kMaxScanJobs) fail(LENS_EINVAL, "internal: number of scans");
+  if (n <= kOneBlockScan) {
+    ScanJobs J{};
+    for (int i = 0; i < k; ++i) J.job[i] = jobs[i];
+    k_scan_multi<<<k, kMultiThreads, 0, s>>>(J, n);
+    LENS_LAUNCHED("k_scan_multi");
+    return;
+  }
+  for (int i = 0; i < k; ++i) {
+    if (jobs[i].in == jobs[i].out) fail(LENS_EINVAL, "internal: scan in place");
+    exclusive_scan_i64(jobs[i].in, jobs[i].out, n, da, s);
+    k_scan_total<<<1, 1, 0, s>>>(jobs[i].in, jobs[i].out, n);
+    LENS_LAUNCHED("k_scan_total");
+  }
 }
 
 // out[i] = sum_{j<i} in[j]; returns nothing (caller reads out[n-1] + in[n-1]

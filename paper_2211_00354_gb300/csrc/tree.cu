@@ -24,6 +24,7 @@
 // are skipped in every list.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "cx.cuh"
@@ -99,6 +100,24 @@ k_bounds(const double* __restrict__ stars, const double* __restrict__ m, int64_t
     }
     part[blockIdx.x * kBoundsParts + t] = v;
   }
+}
+
+// The blocks' partial bounds into one, stored in mapped host memory (as float64
+// bits): one warp a part.
+__global__ void k_bounds_final(const double* __restrict__ part, int nb, int64_t* __restrict__ out) {
+  const int t = threadIdx.x >> 5, lane = threadIdx.x & 31;  // part t
+  const bool mx = t == 1 || t == 3 || t == 6;
+  double v = t == 4 ? 0.0 : mx ? -INFINITY : INFINITY;
+  for (int b = lane; b < nb; b += 32) {
+    const double x = part[b * kBoundsParts + t];
+    v = t == 4 ? v + x : mx ? fmax(v, x) : fmin(v, x);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, v, o);
+    v = t == 4 ? v + x : mx ? fmax(v, x) : fmin(v, x);
+  }
+  if (lane == 0) out[t] = __double_as_longlong(v);
 }
 
 __global__ void k_keys(const double* __restrict__ stars, int64_t n, double lo_x, double lo_y,
@@ -303,12 +322,18 @@ __global__ void k_active_flags(TreeView T, int64_t nb, double root_lo_x, double 
   fl[b] = (act && T.child[b] < 0) ? 1 : 0;
 }
 
-__global__ void k_compact(const int64_t* __restrict__ flag, const int64_t* __restrict__ pos,
-                          int64_t n, int* __restrict__ out, int* __restrict__ inv) {
+// the flagged boxes of both flag arrays in order, and each box's place or -1
+__global__ void k_compact(const int64_t* __restrict__ fa, const int64_t* __restrict__ pa,
+                          const int64_t* __restrict__ fl, const int64_t* __restrict__ pl, int64_t n,
+                          int* __restrict__ active, int* __restrict__ aidx,
+                          int* __restrict__ leaves, int* __restrict__ lidx) {
   const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (b >= n) return;
-  if (flag[b]) out[pos[b]] = (int)b;
-  if (inv) inv[b] = flag[b] ? (int)pos[b] : -1;
+  const bool a = fa[b], l = fl[b];
+  if (a) active[pa[b]] = (int)b;
+  if (l) leaves[pl[b]] = (int)b;
+  aidx[b] = a ? (int)pa[b] : -1;
+  lidx[b] = l ? (int)pl[b] : -1;
 }
 
 // box containing cell (level, ix, iy): the box at that level if it exists,
@@ -445,11 +470,6 @@ __global__ void k_lists(TreeView T, const int* __restrict__ active, int64_t nact
   }
 }
 
-__global__ void k_sentinels(int64_t* a, int64_t* b, int64_t* c, int64_t* d, int64_t va,
-                            int64_t vb, int64_t vc, int64_t vd) {
-  if (threadIdx.x == 0) { *a = va; *b = vb; *c = vc; *d = vd; }
-}
-
 }  // namespace
 
 void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaStream_t s) {
@@ -457,26 +477,24 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   const int depth = P.depth;
   // ---- 1. bounds + finiteness -------------------------------------------
   const int nbb = (int)std::min<int64_t>(1024, (n + 255) / 256);
-  std::vector<double> part(kBoundsParts * (size_t)nbb);
+  double q[kBoundsParts];
   {
     Scratch dpart(&P.da, sizeof(double) * kBoundsParts * nbb);
+    const HostSlot slot = host_slot();
     k_bounds<<<nbb, kBoundsThreads, 0, s>>>(stars, masses, n, dpart.as<double>());
     LENS_LAUNCHED("k_bounds");
+    k_bounds_final<<<1, 32 * kBoundsParts, 0, s>>>(dpart.as<double>(), nbb, slot.dev);
+    LENS_LAUNCHED("k_bounds_final");
     // the translation tables are formed on the host while the bounds run
     fmm_tables(P, s);
-    LENS_CUDA(cudaMemcpyAsync(part.data(), dpart.p, sizeof(double) * kBoundsParts * nbb,
-                              cudaMemcpyDeviceToHost, s));
     LENS_CUDA(cudaStreamSynchronize(s));
+    for (int k = 0; k < kBoundsParts; ++k) {
+      const int64_t w = slot.host[k];
+      std::memcpy(&q[k], &w, sizeof(double));
+    }
   }
-  double xmin = INFINITY, xmax = -INFINITY, ymin = INFINITY, ymax = -INFINITY, bad = 0;
-  double mmin = INFINITY, mmax = -INFINITY;
-  for (int b = 0; b < nbb; ++b) {
-    const double* q = &part[(size_t)kBoundsParts * b];
-    xmin = std::min(xmin, q[0]); xmax = std::max(xmax, q[1]);
-    ymin = std::min(ymin, q[2]); ymax = std::max(ymax, q[3]);
-    bad += q[4];
-    mmin = std::min(mmin, q[5]); mmax = std::max(mmax, q[6]);
-  }
+  double xmin = q[0], xmax = q[1], ymin = q[2], ymax = q[3];
+  const double bad = q[4], mmin = q[5], mmax = q[6];
   if (bad > 0) fail(LENS_EINVAL, "non-finite star position or mass");
   // all stars of one mass (a common microlensing field): the float32 near
   // field then sums 1/|d|^2-weighted offsets and scales by the mass once
@@ -515,22 +533,21 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   radix_sort_u64(P.skey, P.sidx, n, 2 * depth, P.da, s, lo_bit);
 
   // ---- 3. split nodes ---------------------------------------------------
-  Scratch dcnt(&P.da, sizeof(unsigned long long) * (kMaxDepth + 2) + sizeof(int) * 4);
+  // per-level split counts, then the flag of a box deeper than the sorted bits
+  constexpr int kCountWords = kMaxDepth + 3;
+  Scratch dcnt(&P.da, sizeof(unsigned long long) * kCountWords);
   unsigned long long* counts = dcnt.as<unsigned long long>();
   int* deep = reinterpret_cast<int*>(counts + kMaxDepth + 2);
   const unsigned nblk = grid_for(n, kSplitThreads);
   Scratch bcnt(&P.da, sizeof(int64_t) * kMaxDepth * (size_t)nblk);
-  unsigned long long hc[kMaxDepth + 2];
-  int hdeep[4];
+  int64_t hc[kCountWords];
   for (;;) {
     LENS_CUDA(cudaMemsetAsync(dcnt.p, 0, dcnt.bytes, s));
     k_splits<false><<<nblk, kSplitThreads, 0, s>>>(P.skey, n, depth, dcap, P.leaf, counts, deep,
                                                    bcnt.as<int64_t>(), nullptr, nullptr);
     LENS_LAUNCHED("k_splits<count>");
-    LENS_CUDA(cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
-    LENS_CUDA(cudaMemcpyAsync(hdeep, deep, sizeof(hdeep), cudaMemcpyDeviceToHost, s));
-    LENS_CUDA(cudaStreamSynchronize(s));
-    if (!hdeep[0]) break;
+    read_words(dcnt.as<int64_t>(), kCountWords, hc, s);
+    if (!hc[kMaxDepth + 2]) break;
     if (dcap == depth)
       fail(LENS_EDEPTH, "a box at the depth cap still holds more than leaf_size stars "
                         "(coincident stars?): raise leaf_size or max_depth");
@@ -546,7 +563,7 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   int maxl = -1;
   for (int l = 0; l < depth; ++l) {
     soff.off[l] = nsplit;
-    nsplit += (int64_t)hc[l];
+    nsplit += hc[l];
     if (hc[l]) maxl = l;
   }
   for (int l = depth; l <= kMaxDepth + 1; ++l) soff.off[l] = nsplit;
@@ -554,7 +571,7 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   P.level_off.assign(P.nlevels + 1, 0);
   P.level_off[0] = 0;
   P.level_off[1] = 1;
-  for (int l = 1; l < P.nlevels; ++l) P.level_off[l + 1] = P.level_off[l] + 4 * (int64_t)hc[l - 1];
+  for (int l = 1; l < P.nlevels; ++l) P.level_off[l + 1] = P.level_off[l] + 4 * hc[l - 1];
   P.nb = P.level_off[P.nlevels];
   if (P.nb > (int64_t)INT32_MAX) fail(LENS_ENOMEM, "tree too large");
   for (int l = 0; l <= kMaxDepth + 1; ++l)
@@ -577,8 +594,9 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   LENS_LAUNCHED("k_root");
   if (nsplit > 0) {
     Scratch dspl(&P.da, sizeof(uint64_t) * nsplit);
-    Scratch bpos(&P.da, sizeof(int64_t) * kMaxDepth * (size_t)nblk);
-    exclusive_scan_i64(bcnt.as<int64_t>(), bpos.as<int64_t>(), (int64_t)kMaxDepth * nblk, P.da, s);
+    Scratch bpos(&P.da, sizeof(int64_t) * (kMaxDepth * (size_t)nblk + 1));
+    const ScanJob job{bcnt.as<int64_t>(), bpos.as<int64_t>()};
+    exclusive_scans(&job, 1, (int64_t)kMaxDepth * nblk, P.da, s);
     k_splits<true><<<nblk, kSplitThreads, 0, s>>>(P.skey, n, depth, dcap, P.leaf, nullptr, nullptr,
                                                   nullptr, bpos.as<int64_t>(), dspl.as<uint64_t>());
     LENS_LAUNCHED("k_splits<write>");
@@ -600,50 +618,46 @@ void tree_build_lists(Plan& P, cudaStream_t s) {
   TreeView T{P.box_start, P.box_count, P.box_child, P.box_level, P.box_ix, P.box_iy,
              P.box_code, boff};
   Scratch fa(&P.da, sizeof(int64_t) * nb), fl(&P.da, sizeof(int64_t) * nb);
-  Scratch pa(&P.da, sizeof(int64_t) * nb), pl(&P.da, sizeof(int64_t) * nb);
+  Scratch pa(&P.da, sizeof(int64_t) * (nb + 1)), pl(&P.da, sizeof(int64_t) * (nb + 1));
   k_active_flags<<<grid_for(nb, 256), 256, 0, s>>>(
       T, nb, P.root_lo[0], P.root_lo[1], P.root_size, P.has_target ? 1 : 0, P.target[0],
       P.target[1], P.target[2], P.target[3], P.box_active, fa.as<int64_t>(), fl.as<int64_t>());
   LENS_LAUNCHED("k_active_flags");
-  exclusive_scan_i64(fa.as<int64_t>(), pa.as<int64_t>(), nb, P.da, s);
-  exclusive_scan_i64(fl.as<int64_t>(), pl.as<int64_t>(), nb, P.da, s);
+  {
+    const ScanJob jobs[2] = {{fa.as<int64_t>(), pa.as<int64_t>()}, {fl.as<int64_t>(), pl.as<int64_t>()}};
+    exclusive_scans(jobs, 2, nb, P.da, s);
+  }
   std::vector<int64_t> hpos(P.nlevels + 1);
-  int64_t lastf[2], lastp[2];
   {
     // level starts of the active list and the two totals, in one read-back
     std::vector<const int64_t*> addr;
     for (int l = 0; l < P.nlevels; ++l) addr.push_back(pa.as<int64_t>() + P.level_off[l]);
-    addr.push_back(fa.as<int64_t>() + nb - 1);
-    addr.push_back(pa.as<int64_t>() + nb - 1);
-    addr.push_back(fl.as<int64_t>() + nb - 1);
-    addr.push_back(pl.as<int64_t>() + nb - 1);
+    addr.push_back(pa.as<int64_t>() + nb);
+    addr.push_back(pl.as<int64_t>() + nb);
     std::vector<int64_t> v(addr.size());
-    read_i64(addr.data(), (int)addr.size(), v.data(), P.da, s);
+    read_i64(addr.data(), (int)addr.size(), v.data(), s);
     for (int l = 0; l < P.nlevels; ++l) hpos[l] = v[l];
-    lastf[0] = v[P.nlevels]; lastp[0] = v[P.nlevels + 1];
-    lastf[1] = v[P.nlevels + 2]; lastp[1] = v[P.nlevels + 3];
+    P.n_active = v[P.nlevels];
+    P.n_active_leaves = v[P.nlevels + 1];
   }
-  P.n_active = lastf[0] + lastp[0];
-  P.n_active_leaves = lastf[1] + lastp[1];
   hpos[P.nlevels] = P.n_active;
   P.active_level_off = hpos;
   P.active = P.dalloc_n<int>(P.n_active);
   P.active_leaves = P.dalloc_n<int>(P.n_active_leaves);
   P.box_aidx = P.dalloc_n<int>(nb);
-  k_compact<<<grid_for(nb, 256), 256, 0, s>>>(fa.as<int64_t>(), pa.as<int64_t>(), nb, P.active,
-                                               P.box_aidx);
-  LENS_LAUNCHED("k_compact");
   P.box_lidx = P.dalloc_n<int>(nb);
-  k_compact<<<grid_for(nb, 256), 256, 0, s>>>(fl.as<int64_t>(), pl.as<int64_t>(), nb,
+  k_compact<<<grid_for(nb, 256), 256, 0, s>>>(fa.as<int64_t>(), pa.as<int64_t>(), fl.as<int64_t>(),
+                                               pl.as<int64_t>(), nb, P.active, P.box_aidx,
                                                P.active_leaves, P.box_lidx);
   LENS_LAUNCHED("k_compact");
 
   // ---- 5. interaction lists ------------------------------------------
   const int64_t na = P.n_active;
-  Scratch cnt(&P.da, sizeof(int64_t) * 5 * (na + 1));
+  Scratch cnt(&P.da, sizeof(int64_t) * 4 * (na + 1));
   int64_t* c = cnt.as<int64_t>();
+  P.ustar_cnt = P.dalloc_n<int64_t>(na + 1);
   ListOut o{};
-  o.cV = c; o.cX = c + na; o.cU = c + 2 * na; o.cW = c + 3 * na; o.ustars = c + 4 * na;
+  o.cV = c; o.cX = c + na; o.cU = c + 2 * na; o.cW = c + 3 * na; o.ustars = P.ustar_cnt;
   Scratch nbr(&P.da, sizeof(int) * 18 * (size_t)std::max<int64_t>(na, 1));
   if (na > 0) {
     k_neighbours<<<grid_for(na * 18, 256), 256, 0, s>>>(T, P.active, na, nbr.as<int>());
@@ -653,36 +667,22 @@ void tree_build_lists(Plan& P, cudaStream_t s) {
   k_lists<false><<<grid_for(na, 128), 128, 0, s>>>(T, P.active, na, o);
   LENS_LAUNCHED("k_lists<count>");
   int64_t* offs[4];
-  int64_t tot[4];
-  for (int q = 0; q < 4; ++q) {
-    offs[q] = reinterpret_cast<int64_t*>(P.dalloc(sizeof(int64_t) * (na + 1)));
-    exclusive_scan_i64(c + q * na, offs[q], na, P.da, s);
-  }
-  // totals: last offset + last count; also total U stars
-  std::vector<int64_t> hl(10, 0);
-  P.ustar_cnt = P.dalloc_n<int64_t>(na + 1);
-  if (na > 0)
-    LENS_CUDA(cudaMemcpyAsync(P.ustar_cnt, c + 4 * na, sizeof(int64_t) * na,
-                              cudaMemcpyDeviceToDevice, s));
+  int64_t tot[5];
   Scratch usum(&P.da, sizeof(int64_t) * (na + 1));
-  if (na > 0) {
-    exclusive_scan_i64(c + 4 * na, usum.as<int64_t>(), na, P.da, s);
-    const int64_t* addr[10];
+  {
+    ScanJob jobs[5];
+    const int64_t* addr[5];
     for (int q = 0; q < 4; ++q) {
-      addr[2 * q] = offs[q] + na - 1;
-      addr[2 * q + 1] = c + q * na + na - 1;
+      offs[q] = reinterpret_cast<int64_t*>(P.dalloc(sizeof(int64_t) * (na + 1)));
+      jobs[q] = {c + q * na, offs[q]};
+      addr[q] = offs[q] + na;
     }
-    addr[8] = usum.as<int64_t>() + na - 1;
-    addr[9] = c + 4 * na + na - 1;
-    read_i64(addr, 10, hl.data(), P.da, s);
+    jobs[4] = {P.ustar_cnt, usum.as<int64_t>()};
+    addr[4] = usum.as<int64_t>() + na;
+    exclusive_scans(jobs, 5, na, P.da, s);
+    read_i64(addr, 5, tot, s);
   }
-  for (int q = 0; q < 4; ++q) tot[q] = hl[2 * q] + hl[2 * q + 1];
-  P.u_stars = hl[8] + hl[9];
-  // write the totals as the sentinel offsets[na] (kernel parameters: no host
-  // buffer has to outlive the call)
-  k_sentinels<<<1, 32, 0, s>>>(offs[0] + na, offs[1] + na, offs[2] + na, offs[3] + na, tot[0],
-                               tot[1], tot[2], tot[3]);
-  LENS_LAUNCHED("k_sentinels");
+  P.u_stars = tot[4];
   P.nV = tot[0]; P.nX = tot[1]; P.nU = tot[2]; P.nW = tot[3];
   P.V_list = P.dalloc_n<int>(tot[0]);
   P.X_list = P.dalloc_n<int>(tot[1]);
