@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
     const int64_t ridx = A.perm[A.ray_off[k] + r0 + t];
     const ff ox = ff_of(A.rays[2 * ridx] - cB.x), oy = ff_of(A.rays[2 * ridx + 1] - cB.y);
     sz[t] = make_float4(ox.hi, oy.hi, ox.lo, oy.lo);
-    sc[t] = make_float2((float)-A.gy[2 * ridx], (float)-A.gy[2 * ridx + 1]);
+    sc[t] = make_float2(-d2f(A.gy[2 * ridx]), -d2f(A.gy[2 * ridx + 1]));
   }
   __shared__ UStage su;
   for_u_stars(A, a, su, [&](int sj) {
@@ -288,15 +288,15 @@ __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
     }
     for (int64_t t = r0 + lane; t < r1; t += 32) {
       const int64_t ridx = A.perm[A.ray_off[k] + t];
-      const float2 c = make_float2((float)-A.gy[2 * ridx], (float)-A.gy[2 * ridx + 1]);
+      const float2 c = make_float2(-d2f(A.gy[2 * ridx]), -d2f(A.gy[2 * ridx + 1]));
       float2 pw, w;
       if (pass == 0) {
-        w = make_float2((float)((A.rays[2 * ridx] - cB.x) * irB),
-                        (float)((A.rays[2 * ridx + 1] - cB.y) * irB));
+        w = make_float2(d2f((A.rays[2 * ridx] - cB.x) * irB),
+                        d2f((A.rays[2 * ridx + 1] - cB.y) * irB));
         pw = c;
       } else {
-        const float2 inv = cinv(make_float2((float)(A.rays[2 * ridx] - cC.x),
-                                            (float)(A.rays[2 * ridx + 1] - cC.y)));
+        const float2 inv = cinv(make_float2(d2f(A.rays[2 * ridx] - cC.x),
+                                            d2f(A.rays[2 * ridx + 1] - cC.y)));
         w = make_float2(inv.x * (float)rC, inv.y * (float)rC);
         pw = cmul(c, inv);
       }

@@ -74,6 +74,26 @@ __device__ __forceinline__ float2 cinv(float2 z) {
   return make_float2(z.x * d, -z.y * d);
 }
 
+// Conversions on the integer pipe.  A float64 conversion holds the float64 pipe as
+// long as a float64 product does (~77 cycles a warp and sub-partition); the words
+// of a value in the normal range of both types are shifted and rounded in 2-8
+// integer instructions instead, with the same bits (round to nearest even), and
+// everything else (zero, subnormal, huge, infinite, NaN) takes the conversion.
+// A warp is sent that way by one such value, so zero, the common one, is kept out.
+__device__ __forceinline__ double f2d(float x) {
+  const unsigned v = __float_as_uint(x), m = v & 0x7fffffffu;
+  if (m == 0u) return __hiloint2double((int)v, 0);
+  if (m - 0x00800000u >= 0x7f000000u) return (double)x;
+  return __hiloint2double((int)((v & 0x80000000u) | ((m >> 3) + (896u << 20))), (int)(v << 29));
+}
+// exponents 2^-126 .. 2^126: the result is normal after rounding, too
+__device__ __forceinline__ float d2f(double x) {
+  const unsigned H = (unsigned)__double2hiint(x), L = (unsigned)__double2loint(x);
+  if (((H >> 20) & 0x7ffu) - 897u >= 253u) return (float)x;
+  const unsigned up = ((L & 0x1fffffffu) + 0x0fffffffu + ((L >> 29) & 1u)) >> 29;
+  return __uint_as_float((__funnelshift_l(L, H, 3) + up - (896u << 23)) | (H & 0x80000000u));
+}
+
 // Error-free sum of two floats (Knuth two-sum): s + e == a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;
@@ -89,7 +109,7 @@ struct fcomp {
     hi = s;
     lo += e;
   }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ double value() const { return f2d(hi) + f2d(lo); }
 };
 
 // Two compensated accumulators side by side (one per ray of a pair) on
@@ -163,11 +183,37 @@ namespace lens {
 struct ff {
   float hi, lo;
 };
+// hi = x rounded to float32, lo = the (exact) rest rounded: the 29 bits below hi,
+// as a signed integer, times their weight.  Exponents from 2^-74, so that the
+// rest is normal.
 __host__ __device__ __forceinline__ ff ff_of(double x) {
   ff r;
+#ifdef __CUDA_ARCH__
+  const unsigned H = (unsigned)__double2hiint(x), L = (unsigned)__double2loint(x);
+  const unsigned e = (H >> 20) & 0x7ffu;
+  if (e - 949u < 201u) {
+    const unsigned rem = L & 0x1fffffffu;
+    const unsigned up = (rem + 0x0fffffffu + ((L >> 29) & 1u)) >> 29;
+    r.hi = __uint_as_float((__funnelshift_l(L, H, 3) + up - (896u << 23)) | (H & 0x80000000u));
+    const int d = (int)rem - (int)(up << 29);
+    r.lo = (float)((int)H < 0 ? -d : d) * __uint_as_float((e - 948u) << 23);
+    return r;
+  }
+#endif
   r.hi = (float)x;
   r.lo = (float)(x - (double)r.hi);
   return r;
+}
+// floor(t) for 0 <= t < 2^32 from its words; false for anything else (negative,
+// infinite, NaN).  As floor and a conversion, off the float64 pipe.
+__device__ __forceinline__ bool floor_u32(double t, unsigned& q) {
+  const unsigned H = (unsigned)__double2hiint(t), L = (unsigned)__double2loint(t);
+  const unsigned e = H >> 20;  // a set sign makes it 2048 or more
+  q = 0;
+  if (e < 1023u) return true;
+  if (e > 1054u) return H == 0x80000000u && L == 0u;  // -0
+  q = (0x80000000u | (H << 11) | (L >> 21)) >> (1054u - e);
+  return true;
 }
 __device__ __forceinline__ ff ff_norm(float s, float e) {  // |s| >= |e|
   ff r;
@@ -199,7 +245,7 @@ __device__ __forceinline__ ff ff_mul(ff a, float b) {
   const float e = fmaf(a.hi, b, -p) + a.lo * b;
   return ff_norm(p, e);
 }
-__device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double ff_to_double(ff a) { return f2d(a.hi) + f2d(a.lo); }
 
 // The same float-float operations on two values side by side (one per ray of
 // a pair), on the two-lane float32 instructions; a - b is fma(b, -1, a), and

@@ -362,14 +362,14 @@ __global__ void k_ray_leaf(const double* __restrict__ rays, int64_t m, const int
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= m) return;
   const double x = rays[2 * r], y = rays[2 * r + 1];
-  const double qmax = (double)((1u << depth) - 1u);
-  const double fx = floor((x - lo_x) * scale), fy = floor((y - lo_y) * scale);
-  if (!(fx >= 0.0 && fx <= qmax && fy >= 0.0 && fy <= qmax)) {  // also catches NaN
+  const uint32_t qmax = (1u << depth) - 1u;
+  unsigned qx, qy;
+  if (!(floor_u32((x - lo_x) * scale, qx) && floor_u32((y - lo_y) * scale, qy) && qx <= qmax &&
+        qy <= qmax)) {  // also catches NaN
     *err = 1;  // host memory: a plain store, whoever comes first
     slot[r] = -1;
     return;
   }
-  const uint32_t qx = (uint32_t)fx, qy = (uint32_t)fy;
   int b = 0;
   for (int l = 0; l < depth; ++l) {
     const int c = child[b];

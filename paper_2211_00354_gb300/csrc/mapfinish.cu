@@ -70,7 +70,7 @@ k_map_finish(float* __restrict__ m32, float* __restrict__ D, int npx, int npy, i
             m[c] = 0.f;
             d[c] = 0.f;
           } else {
-            o[c] = (double)v.hi + (double)v.lo;
+            o[c] = ff_to_double(v);
           }
         }
       }
