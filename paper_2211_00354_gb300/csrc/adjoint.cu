@@ -29,6 +29,12 @@ namespace lens {
 namespace {
 
 constexpr int kAdjTile = 128;  // rays per tile
+// float32-bulk plans: twice that once the rays give the chip several blocks an SM all
+// the same (a star's offsets and sums are formed once a tile).  P2P^T and moments at 3e6
+// rays on 16 leaves 384 + 72 us (tiles of 128: 420 + 91), at 5e5 rays 69 + 18 (73 + 15),
+// at 1.3e5 26 + 15 (24 + 10): the line is where the two meet.
+constexpr int kAdjTile32 = 256;
+constexpr int64_t kAdjLarge = 1 << 19;
 constexpr int kAdjU = 64;      // U-list leaves staged at a time by k_adj_p2p32
 
 __device__ __forceinline__ void atomic_add2(double2* p, double2 v) {
@@ -38,34 +44,31 @@ __device__ __forceinline__ void atomic_add2(double2* p, double2 v) {
 
 struct AdjArgs {
   const double* rays; const double* gy;
-  const int* perm; const int64_t* ray_off; const int64_t* tile_off; int64_t nleaf;
+  const int* perm; const int64_t* ray_off; const int2* tile_leaf; int tile;
   const int* leaves; const int* aidx; const int* level; const int* ix; const int* iy;
   const int* start; const int* count; const int* child; const int* parent;
   const int64_t* U_off; const int* U_list; const int64_t* W_off; const int* W_list;
   const int64_t* V_off; const int* V_list; const int64_t* X_off; const int* X_list;
   const double2* spos; const double* smass;
   FmmTables tab;
-  double lo_x, lo_y, size;
+  double lo_x, lo_y, size, isize;  // isize = 1 / size
   int p;
   double2* Lh; double2* Mh;   // adjoints of L (by box) and M (by box)
   double2* Phi; double2* Psi; // per sorted star
   double* gkg;                // [2]
 };
 
-__device__ __forceinline__ int64_t leaf_of_tile(const int64_t* toff, int64_t nleaf, int64_t b) {
-  int64_t lo = 0, hi = nleaf;
-  while (hi - lo > 1) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (toff[mid] <= b) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
+// A box's half side, its inverse and its centre, without a division or a conversion
+// on the float64 pipe (a block of few rays formed them at ~40 operations there).
 __device__ __forceinline__ double box_r(const AdjArgs& A, int b) {
-  return A.size / (double)(2ull << A.level[b]);
+  return mul_pow2(A.size, -(A.level[b] + 1));
+}
+__device__ __forceinline__ double box_ir(const AdjArgs& A, int b) {
+  return mul_pow2(A.isize, A.level[b] + 1);
 }
 __device__ __forceinline__ double2 box_c(const AdjArgs& A, int b, double r) {
-  return make_double2(A.lo_x + (2.0 * A.ix[b] + 1.0) * r, A.lo_y + (2.0 * A.iy[b] + 1.0) * r);
+  return make_double2(fma(u2d(2u * (unsigned)A.ix[b] + 1u), r, A.lo_x),
+                      fma(u2d(2u * (unsigned)A.iy[b] + 1u), r, A.lo_y));
 }
 
 // One warp per (leaf, tile): L2P^T moments of the tile's rays and M2P^T for
@@ -74,18 +77,19 @@ __device__ __forceinline__ double2 box_c(const AdjArgs& A, int b, double r) {
 __global__ void __launch_bounds__(32) k_adj_leaf_moments(AdjArgs A) {
   extern __shared__ double2 acc[];  // [(p+1)][32]
   const int lane = threadIdx.x;
-  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
-  const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
+  const int2 kt = A.tile_leaf[blockIdx.x];
+  if (kt.x < 0) return;
+  const int64_t k = kt.x;
   const int B = A.leaves[k];
   const int a = A.aidx[B];
-  const int64_t tile = (int64_t)blockIdx.x - A.tile_off[k];
+  const int64_t tile = kt.y;
   const int64_t n = A.ray_off[k + 1] - A.ray_off[k];
   const int64_t r0 = tile * kAdjTile;
   const int64_t r1 = min64(n, r0 + kAdjTile);
   const int p = A.p;
   const double rB = box_r(A, B);
   const double2 cB = box_c(A, B, rB);
-  const double irB = 1.0 / rB;
+  const double irB = box_ir(A, B);
   // pass 0: L2P^T; pass e >= 1: M2P^T of W entry e-1
   const int64_t nW = A.W_off[a + 1] - A.W_off[a];
   for (int64_t pass = 0; pass <= nW; ++pass) {
@@ -133,12 +137,12 @@ __global__ void __launch_bounds__(32) k_adj_leaf_moments(AdjArgs A) {
 
 // The stars of a leaf's U list, flattened over the block's threads (a leaf's own
 // count is often below the block size): up to kAdjU leaves at a time, their first
-// star and inclusive star counts in shared memory.  f(sj) is called for every
-// star of the list, one thread each.
+// star and inclusive star counts in shared memory.  f(sj, h) is called for every
+// star of the list by S neighbouring lanes, h = 0 .. S - 1.
 struct UStage {
   int start[kAdjU], incl[kAdjU];
 };
-template <typename F>
+template <int S, typename F>
 __device__ __forceinline__ void for_u_stars(const AdjArgs& A, int a, UStage& su, F f) {
   const int64_t u0 = A.U_off[a], nu = A.U_off[a + 1] - u0;
   for (int64_t ub = 0; ub < nu; ub += kAdjU) {
@@ -154,14 +158,15 @@ __device__ __forceinline__ void for_u_stars(const AdjArgs& A, int a, UStage& su,
       for (int i = 1; i < nub; ++i) su.incl[i] += su.incl[i - 1];
     __syncthreads();
     const int tot = su.incl[nub - 1];
-    for (int q = threadIdx.x; q < tot; q += blockDim.x) {
+    for (int qs = threadIdx.x; qs < tot * S; qs += blockDim.x) {
+      const int q = qs / S;
       // the group's leaf holding flattened star q: the first with incl > q
       int lo = 0, hi = nub - 1;
       while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         if (su.incl[mid] > q) hi = mid; else lo = mid + 1;
       }
-      f(su.start[lo] + q - (lo ? su.incl[lo - 1] : 0));
+      f(su.start[lo] + q - (lo ? su.incl[lo - 1] : 0), qs % S);
     }
   }
 }
@@ -174,10 +179,11 @@ __device__ __forceinline__ void for_u_stars(const AdjArgs& A, int a, UStage& su,
 __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
   __shared__ double2 sz[kAdjTile], sc[kAdjTile];
   __shared__ UStage su;
-  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
-  const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
+  const int2 kt = A.tile_leaf[blockIdx.x];
+  if (kt.x < 0) return;
+  const int64_t k = kt.x;
   const int a = A.aidx[A.leaves[k]];
-  const int64_t tile = (int64_t)blockIdx.x - A.tile_off[k];
+  const int64_t tile = kt.y;
   const int64_t n = A.ray_off[k + 1] - A.ray_off[k];
   const int64_t r0 = tile * kAdjTile;
   const int nr = (int)min64(kAdjTile, n - r0);
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
     sz[t] = make_double2(A.rays[2 * ridx], A.rays[2 * ridx + 1]);
     sc[t] = make_double2(-A.gy[2 * ridx], -A.gy[2 * ridx + 1]);
   }
-  for_u_stars(A, a, su, [&](int sj) {
+  for_u_stars<1>(A, a, su, [&](int sj, int) {
     const double2 zj = A.spos[sj];
     double2 F = make_double2(0, 0), G = make_double2(0, 0);
 #pragma unroll 2
@@ -210,51 +216,101 @@ __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
 // (each pair's difference exact to float32 rounding however close a ray is
 // to a star), partial sums compensated; L2P^T / M2P^T moments with the
 // scaled offsets w rounded once to float32 (|w| <= ~1.5: no cancellation),
-// summed per lane in float32 and across lanes in float64.  The transposed
+// summed per lane in float32 and across lanes compensated.  The transposed
 // translations (L2L^T, M2L^T, P2L^T, M2M^T, P2M^T) stay float64.
 
-// P2P^T: block per (leaf, tile of rays), threads over the U-list stars; the
-// tile's rays staged as float-float offsets from the leaf centre with their
-// float32 charges.
+// P2P^T: block per (leaf, tile of rays), four lanes a star over the U-list stars, each
+// with every fourth pair of the tile's rays, staged as float-float offsets from
+// the leaf centre with their float32 charges; two rays an instruction (paired
+// float32), the four lanes' sums combined in float-float.  Bound by the FMA
+// pipe and issue: 12 products and differences and 28 operations of compensated
+// sums a pair of points.  A lane a star left a third of the lanes idle at ~70 stars a
+// list: 3e6 rays, p 24, leaves of 16: 530 -> 420 us,
+// tiles of 256 rays 384.
+constexpr int kStarLanes = 4;
+
+__device__ __forceinline__ ff lanes_sum(const fcomp2& a) {
+  ff u, v;
+  two_sum(a.hi.x, a.lo.x, u.hi, u.lo);
+  two_sum(a.hi.y, a.lo.y, v.hi, v.lo);
+  return ff_add(u, v);
+}
+__device__ __forceinline__ ff ff_shfl_xor(unsigned mask, ff a, int o) {
+  return ff{__shfl_xor_sync(mask, a.hi, o), __shfl_xor_sync(mask, a.lo, o)};
+}
+
 __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
-  __shared__ float4 sz[kAdjTile];  // x_hi, y_hi, x_lo, y_lo
-  __shared__ float2 sc[kAdjTile];
-  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
-  const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
+  // pairs of rays: x, x, -y, -y (high and low parts), charges, -c.y
+  __shared__ float4 szh[kAdjTile32 / 2], szl[kAdjTile32 / 2], sc[kAdjTile32 / 2];
+  __shared__ float2 snc[kAdjTile32 / 2];
+  const int2 kt = A.tile_leaf[blockIdx.x];
+  if (kt.x < 0) return;
+  const int64_t k = kt.x;
   const int B = A.leaves[k];
   const int a = A.aidx[B];
-  const int64_t tile = (int64_t)blockIdx.x - A.tile_off[k];
+  const int64_t tile = kt.y;
   const int64_t n = A.ray_off[k + 1] - A.ray_off[k];
-  const int64_t r0 = tile * kAdjTile;
-  const int nr = (int)min64(kAdjTile, n - r0);
+  const int64_t r0 = tile * A.tile;
+  const int nr = (int)min64(A.tile, n - r0);
+  const int np = (nr + 2 * kStarLanes - 1) / (2 * kStarLanes) * kStarLanes;  // pairs, whole rounds
   const double rB = box_r(A, B);
   const double2 cB = box_c(A, B, rB);
-  for (int t = threadIdx.x; t < nr; t += blockDim.x) {
-    const int64_t ridx = A.perm[A.ray_off[k] + r0 + t];
-    const ff ox = ff_of(A.rays[2 * ridx] - cB.x), oy = ff_of(A.rays[2 * ridx + 1] - cB.y);
-    sz[t] = make_float4(ox.hi, oy.hi, ox.lo, oy.lo);
-    sc[t] = make_float2(-d2f(A.gy[2 * ridx]), -d2f(A.gy[2 * ridx + 1]));
+  for (int t = threadIdx.x; t < 2 * np; t += blockDim.x) {
+    ff ox{1e18f, 0.f}, oy{1e18f, 0.f};  // beyond the tile: far, no charge
+    float c1 = 0.f, c2 = 0.f;
+    if (t < nr) {
+      const int64_t ridx = A.perm[A.ray_off[k] + r0 + t];
+      ox = ff_of(A.rays[2 * ridx] - cB.x);
+      oy = ff_of(A.rays[2 * ridx + 1] - cB.y);
+      c1 = -d2f(A.gy[2 * ridx]);
+      c2 = -d2f(A.gy[2 * ridx + 1]);
+    }
+    float* h = reinterpret_cast<float*>(szh + (t >> 1)) + (t & 1);
+    float* l = reinterpret_cast<float*>(szl + (t >> 1)) + (t & 1);
+    float* c = reinterpret_cast<float*>(sc + (t >> 1)) + (t & 1);
+    h[0] = ox.hi; h[2] = -oy.hi;
+    l[0] = ox.lo; l[2] = -oy.lo;
+    c[0] = c1; c[2] = c2;
+    reinterpret_cast<float*>(snc + (t >> 1))[t & 1] = -c2;
   }
   __shared__ UStage su;
-  for_u_stars(A, a, su, [&](int sj) {
+  for_u_stars<kStarLanes>(A, a, su, [&](int sj, int h) {
     const double2 zj = A.spos[sj];
     const ff sx = ff_of(zj.x - cB.x), sy = ff_of(zj.y - cB.y);
-    fcomp F1{0.f, 0.f}, F2{0.f, 0.f}, G1{0.f, 0.f}, G2{0.f, 0.f};
-    for (int t = 0; t < nr; ++t) {
-      const float4 z = sz[t];
-      const float2 c = sc[t];
+    const float2 xh = make_float2(-sx.hi, -sx.hi), xl = make_float2(-sx.lo, -sx.lo);
+    const float2 yh = make_float2(sy.hi, sy.hi), yl = make_float2(sy.lo, sy.lo);
+    const float2 tiny = make_float2(1e-30f, 1e-30f), m1 = make_float2(-1.f, -1.f);
+    const float2 zero = make_float2(0.f, 0.f);
+    fcomp2 F1{zero, zero}, F2{zero, zero}, G1{zero, zero}, G2{zero, zero};
+    for (int i = h; i < np; i += kStarLanes) {
+      const float4 zh = szh[i], zl = szl[i], c4 = sc[i];
+      const float2 cx = make_float2(c4.x, c4.y), cy = make_float2(c4.z, c4.w), ncy = snc[i];
       // d = z_r - z_j; 1/d = conj(d) / |d|^2 (a star exactly at the ray adds
       // nothing: d = 0 makes both terms 0 under the floor on |d|^2)
-      const float d1 = (z.x - sx.hi) + (z.z - sx.lo), d2 = (z.y - sy.hi) + (z.w - sy.lo);
-      const float w = frcp_fast(fmaf(d1, d1, fmaf(d2, d2, 1e-30f)));
-      const float i1 = d1 * w, i2 = -d2 * w;
-      const float c1 = c.x * i1 - c.y * i2, c2 = c.x * i2 + c.y * i1;  // c / d
+      const float2 d1 = __fadd2_rn(__fadd2_rn(make_float2(zh.x, zh.y), xh),
+                                   __fadd2_rn(make_float2(zl.x, zl.y), xl));
+      const float2 n2 = __fadd2_rn(__fadd2_rn(make_float2(zh.z, zh.w), yh),  // -d2
+                                   __fadd2_rn(make_float2(zl.z, zl.w), yl));
+      const float2 q = __ffma2_rn(d1, d1, __ffma2_rn(n2, n2, tiny));
+      const float2 w = make_float2(frcp_fast(q.x), frcp_fast(q.y));
+      const float2 i1 = __fmul2_rn(d1, w), i2 = __fmul2_rn(n2, w), mi2 = __fmul2_rn(i2, m1);
+      const float2 c1 = __ffma2_rn(cx, i1, __fmul2_rn(ncy, i2));  // c / d
+      const float2 c2 = __ffma2_rn(cx, i2, __fmul2_rn(cy, i1));
       F1.add(c1); F2.add(c2);
-      G1.add(c1 * i1 - c2 * i2); G2.add(c1 * i2 + c2 * i1);             // c / d^2
+      G1.add(__ffma2_rn(c1, i1, __fmul2_rn(c2, mi2)));            // c / d^2
+      G2.add(__ffma2_rn(c1, i2, __fmul2_rn(c2, i1)));
     }
-    const double mj = A.smass[sj];
-    atomic_add2(A.Phi + sj, make_double2(F1.value(), F2.value()));
-    atomic_add2(A.Psi + sj, make_double2(mj * G1.value(), mj * G2.value()));
+    // lane h ends with one of F1, G1, F2, G2 (its bits: G, second component)
+    const unsigned mask = 0xfu << (threadIdx.x & 28u);
+    const ff f1 = lanes_sum(F1), f2s = lanes_sum(F2), g1 = lanes_sum(G1), g2 = lanes_sum(G2);
+    const bool bg = h & 1, b2 = h & 2;
+    const ff k0 = ff_add(bg ? g1 : f1, ff_shfl_xor(mask, bg ? f1 : g1, 1));
+    const ff k1 = ff_add(bg ? g2 : f2s, ff_shfl_xor(mask, bg ? f2s : g2, 1));
+    const ff v = ff_add(b2 ? k1 : k0, ff_shfl_xor(mask, b2 ? k0 : k1, 2));
+    double2* dst = (bg ? A.Psi : A.Phi) + sj;
+    double x = ff_to_double(v);
+    if (bg) x *= A.smass[sj];
+    atomicAdd(b2 ? &dst->y : &dst->x, x);
   });
 }
 
@@ -263,18 +319,19 @@ __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
 __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
   extern __shared__ float2 acc32[];  // [(p+1)][33]: lane partials, padded
   const int lane = threadIdx.x;
-  if (blockIdx.x >= A.tile_off[A.nleaf]) return;
-  const int64_t k = leaf_of_tile(A.tile_off, A.nleaf, blockIdx.x);
+  const int2 kt = A.tile_leaf[blockIdx.x];
+  if (kt.x < 0) return;
+  const int64_t k = kt.x;
   const int B = A.leaves[k];
   const int a = A.aidx[B];
-  const int64_t tile = (int64_t)blockIdx.x - A.tile_off[k];
+  const int64_t tile = kt.y;
   const int64_t n = A.ray_off[k + 1] - A.ray_off[k];
-  const int64_t r0 = tile * kAdjTile;
-  const int64_t r1 = min64(n, r0 + kAdjTile);
+  const int64_t r0 = tile * A.tile;
+  const int64_t r1 = min64(n, r0 + A.tile);
   const int p = A.p;
   const double rB = box_r(A, B);
   const double2 cB = box_c(A, B, rB);
-  const double irB = 1.0 / rB;
+  const double irB = box_ir(A, B);
   const int64_t nW = A.W_off[a + 1] - A.W_off[a];
   for (int64_t pass = 0; pass <= nW; ++pass) {
     for (int l = 0; l <= p; ++l) acc32[l * 33 + lane] = make_float2(0.f, 0.f);
@@ -307,16 +364,19 @@ __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
     }
     __syncwarp();
     double2* dst = pass == 0 ? A.Lh + (int64_t)B * (p + 1) : A.Mh + (int64_t)C * (p + 1);
-    // lane l sums order l's 32 lane partials in float64 (a float64 shuffle
-    // tree would run the adds on every lane of every order)
+    // lane l sums order l's 32 lane partials, compensated (~48 bits): in
+    // float64 the additions and conversions were most of the kernel's time
+    // (3e6 rays, p 24: with the tile's box constants, 260 -> 91 us; tiles of 256,
+    // 72)
     for (int l = lane; l <= p; l += 32) {
-      double vx = 0.0, vy = 0.0;
+      fcomp vx{0.f, 0.f}, vy{0.f, 0.f};
       for (int q = 0; q < 32; ++q) {
         const float2 vf = acc32[l * 33 + q];
-        vx += vf.x;
-        vy += vf.y;
+        vx.add(vf.x);
+        vy.add(vf.y);
       }
-      if (vx != 0.0 || vy != 0.0) atomic_add2(dst + l, make_double2(vx, vy));
+      const double2 v = make_double2(vx.value(), vy.value());
+      if (v.x != 0.0 || v.y != 0.0) atomic_add2(dst + l, v);
     }
     __syncwarp();
   }
@@ -412,21 +472,62 @@ k_adj_m2l(AdjArgs A, const int* active, int64_t na) {
   }
 }
 
-// M2M^T for one level: warp per box of the level, from its parent's Mhat.
-__global__ void __launch_bounds__(128) k_adj_m2m(AdjArgs A, int64_t b0, int64_t b1) {
-  const int lane = threadIdx.x & 31;
-  const int64_t C = b0 + (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
-  if (C >= b1) return;
-  if (A.count[C] == 0) return;
-  const int P = A.parent[C];
-  const int q = (int)C - A.child[P];
-  const int P1 = A.p + 1;
-  const double2* T = A.tab.m2m + (int64_t)q * P1 * P1;
-  const double2* Mp = A.Mh + (int64_t)P * P1;
-  for (int kk = lane; kk <= A.p; kk += 32) {
-    double2 v = A.Mh[C * P1 + kk];
-    for (int l = kk; l <= A.p; ++l) v = cfma(T[l * P1 + kk], Mp[l], v);
-    A.Mh[C * P1 + kk] = v;
+// M2M^T for one level, the children in groups of four, one thread per (parent,
+// coefficient k).  The child offsets d_q = w i^m_q (w = (1+i)/2, m_q = 2, 3, 1, 0)
+// enter through powers of i alone, as in the M2M:
+//   Mhat_C,k += conj(w)^k sum_l i^(m (l-k)) C(l, k) w^l Mhat_P,l
+//            = conj(w)^k sum_r i^(m r) G_r[k],  G_r[k] the terms with l - k = r mod 4,
+// one real binomial sum and additions for four children.  Float64 pipe; with a
+// complex matrix per child, a warp a box and half of its lanes past the
+// triangle's edge: 1e5 stars, p 24: 172 -> 82 us.
+constexpr int kAdjM2mThreads = 128;
+
+__global__ void __launch_bounds__(kAdjM2mThreads)
+k_adj_m2m(AdjArgs A, int64_t c0, int64_t ngroups) {
+  extern __shared__ double2 Wp[];  // [parents per block][p+1], then the binomials
+  const int p = A.p, P1 = p + 1;
+  const int per = kAdjM2mThreads / P1;
+  const int t = threadIdx.x, pb = t / P1, k = t - pb * P1;
+  // C(l, k), k <= l, as [k][l - k]: row k from k (2 p + 3 - k) / 2
+  double* cb = reinterpret_cast<double*>(Wp + (int64_t)per * P1);
+  for (int i = t; i < P1 * P1; i += kAdjM2mThreads) {
+    const int kk = i / P1, l = i - kk * P1;
+    if (l >= kk) cb[kk * (2 * p + 3 - kk) / 2 + l - kk] = A.tab.binom[(int64_t)l * A.tab.ldb + kk];
+  }
+  const int64_t g = (int64_t)blockIdx.x * per + pb;
+  const bool on = pb < per && g < ngroups;
+  const int64_t c = c0 + 4 * g;  // first child of the group
+  double2 w = make_double2(0.0, 0.0);
+  if (on) {
+    w = A.tab.wpow[k];
+    Wp[pb * P1 + k] = cmul(w, A.Mh[(int64_t)A.parent[c] * P1 + k]);
+  }
+  __syncthreads();
+  if (!on) return;
+  const double* crow = cb + k * (2 * p + 3 - k) / 2;
+  const double2* Wk = Wp + pb * P1 + k;
+  double2 G[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) G[r] = make_double2(0.0, 0.0);
+  for (int t0 = 0; t0 <= p - k; t0 += 4) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (t0 + r <= p - k) {
+        G[r].x = fma(crow[t0 + r], Wk[t0 + r].x, G[r].x);
+        G[r].y = fma(crow[t0 + r], Wk[t0 + r].y, G[r].y);
+      }
+    }
+  }
+  const double2 s02 = G[0] + G[2], d02 = G[0] - G[2], s13 = G[1] + G[3], d13 = G[1] - G[3];
+  const double2 cw = make_double2(w.x, -w.y);
+  // sum_r i^(m r) G_r for m = 2, 3, 1, 0
+  const double2 f[4] = {s02 - s13, make_double2(d02.x + d13.y, d02.y - d13.x),
+                        make_double2(d02.x - d13.y, d02.y + d13.x), s02 + s13};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (A.count[c + q] == 0) continue;
+    double2* o = A.Mh + (c + q) * P1 + k;
+    *o = *o + cmul(cw, f[q]);
   }
 }
 
@@ -442,7 +543,7 @@ __global__ void __launch_bounds__(128) k_adj_p2m(AdjArgs A, int64_t nb) {
   const int p = A.p, P1 = p + 1;
   const double r = box_r(A, (int)b);
   const double2 c = box_c(A, (int)b, r);
-  const double ir = 1.0 / r;
+  const double ir = box_ir(A, (int)b);
   const double2* Mb = A.Mh + b * P1;
   const int s0 = A.start[b], s1 = s0 + A.count[b];
   for (int j = s0 + (int)(t % G); j < s1; j += G) {
@@ -499,7 +600,10 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
     return;
   }
   RayBuckets RB;
-  bucket_rays(P, rays, m, kAdjTile, RB, s);
+  const bool f32 = P.prec == LENS_FP32_BULK;
+  const int tile = f32 && m >= kAdjLarge ? kAdjTile32 : kAdjTile;
+  bucket_rays(P, rays, m, tile, RB, s);
+  Scratch tl = tile_leaves(P, RB.toff, P.n_active_leaves, RB.tiles_max, s);
   Scratch Lh(&P.da, sizeof(double2) * (size_t)P.nb * P1);
   Scratch Mh(&P.da, sizeof(double2) * (size_t)P.nb * P1);
   Scratch Phi(&P.da, sizeof(double2) * (size_t)P.n), Psi(&P.da, sizeof(double2) * (size_t)P.n);
@@ -509,19 +613,20 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
   LENS_CUDA(cudaMemsetAsync(Psi.p, 0, Psi.bytes, s));
   AdjArgs A{};
   A.rays = rays; A.gy = gy;
-  A.perm = RB.perm.as<int>(); A.ray_off = RB.off; A.tile_off = RB.toff;
-  A.nleaf = P.n_active_leaves;
+  A.perm = RB.perm.as<int>(); A.ray_off = RB.off;
+  A.tile_leaf = tl.as<int2>();
+  A.tile = tile;
   A.leaves = P.active_leaves; A.aidx = P.box_aidx; A.level = P.box_level; A.ix = P.box_ix;
   A.iy = P.box_iy; A.start = P.box_start; A.count = P.box_count; A.child = P.box_child;
   A.parent = P.box_parent;
   A.U_off = P.U_off; A.U_list = P.U_list; A.W_off = P.W_off; A.W_list = P.W_list;
   A.V_off = P.V_off; A.V_list = P.V_list; A.X_off = P.X_off; A.X_list = P.X_list;
   A.spos = P.spos; A.smass = P.smass; A.tab = P.tab;
-  A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.size = P.root_size; A.p = P.p;
+  A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.size = P.root_size; A.isize = 1.0 / P.root_size; A.p = P.p;
   A.Lh = Lh.as<double2>(); A.Mh = Mh.as<double2>();
   A.Phi = Phi.as<double2>(); A.Psi = Psi.as<double2>();
   const unsigned tiles = (unsigned)RB.tiles_max;
-  if (P.prec == LENS_FP32_BULK) {
+  if (f32) {
     const size_t smem = sizeof(float2) * (size_t)P1 * 33;
     k_adj_leaf_moments32<<<tiles, 32, smem, s>>>(A);
     LENS_LAUNCHED("k_adj_leaf_moments32");
@@ -549,9 +654,12 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
     LENS_LAUNCHED("k_adj_m2l");
   }
   // M2M^T, coarsest level first
+  const int per = kAdjM2mThreads / P1;
+  const size_t sm2 = sizeof(double2) * (size_t)per * P1 + sizeof(double) * (size_t)P1 * (P1 + 1) / 2;
   for (int l = 1; l < P.nlevels; ++l) {
-    const int64_t b0 = P.level_off[l], b1 = P.level_off[l + 1];
-    k_adj_m2m<<<grid_for((b1 - b0) * 32, 128), 128, 0, s>>>(A, b0, b1);
+    const int64_t b0 = P.level_off[l], ng = (P.level_off[l + 1] - b0) / 4;
+    if (ng <= 0) continue;
+    k_adj_m2m<<<grid_for(ng, per), kAdjM2mThreads, sm2, s>>>(A, b0, ng);
     LENS_LAUNCHED("k_adj_m2m");
   }
   if (P.leaf <= 8) k_adj_p2m<8><<<grid_for(P.nb * 8, 128), 128, 0, s>>>(A, P.nb);

@@ -94,6 +94,19 @@ __device__ __forceinline__ float d2f(double x) {
   return __uint_as_float((__funnelshift_l(L, H, 3) + up - (896u << 23)) | (H & 0x80000000u));
 }
 
+// The double of an integer > 0, and x 2^k for a normal x and result (else by a
+// product): the words again.
+__device__ __forceinline__ double u2d(unsigned v) {
+  const int lz = __clz((int)v);
+  const unsigned m = v << lz;
+  return __hiloint2double((int)(((1054u - lz) << 20) | ((m & 0x7fffffffu) >> 11)), (int)(m << 21));
+}
+__device__ __forceinline__ double mul_pow2(double x, int k) {
+  const int H = __double2hiint(x), e = ((H >> 20) & 0x7ff) + k;
+  if (e <= 0 || e >= 2047 || e - k == 0 || e - k == 2047) return ldexp(x, k);
+  return __hiloint2double(H + k * 0x100000, __double2loint(x));
+}
+
 // Error-free sum of two floats (Knuth two-sum): s + e == a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;

@@ -405,21 +405,11 @@ void fmm_tables(Plan& P, cudaStream_t s) {
     }
   };
   powers(0.5, 0.5, wpw.data());
-  std::vector<double2> m2m((size_t)4 * P1 * P1), l2l((size_t)4 * P1 * P1);
+  std::vector<double2> l2l((size_t)4 * P1 * P1);
   for (int q = 0; q < 4; ++q) {
     const double dre = ((q & 1) ? 0.5 : -0.5), dim = ((q >> 1) ? 0.5 : -0.5);
     const std::pair<double, double>* dq = dpow.data() + (size_t)q * P1;
     powers(dre, dim, dpow.data() + (size_t)q * P1);
-    for (int l = 0; l <= p; ++l)
-      for (int k = 0; k <= p; ++k) {
-        double2 v = make_double2(0.0, 0.0);
-        if (k <= l) {
-          const auto d = dq[l - k];
-          const double c = full(l, k) * std::ldexp(1.0, -k);
-          v = make_double2(c * d.first, c * d.second);
-        }
-        m2m[((size_t)q * P1 + l) * P1 + k] = v;
-      }
     for (int j = 0; j <= p; ++j)
       for (int l = 0; l <= p; ++l) {
         double2 v = make_double2(0.0, 0.0);
@@ -457,12 +447,12 @@ void fmm_tables(Plan& P, cudaStream_t s) {
   // one host block (kept in the plan until the copy has run: no wait here);
   // bin holds (2p+2)(p+2) doubles, an even count, so the complex tables
   // after it start on 16-byte boundaries
-  const size_t nd = bin.size() + 2 * (m2m.size() + l2l.size() + up.size() + wp.size());
+  const size_t nd = bin.size() + 2 * (l2l.size() + up.size() + wp.size());
   P.tab_host.assign(nd, 0.0);
   double* h = P.tab_host.data();
   std::memcpy(h, bin.data(), bin.size() * sizeof(double));
   size_t o = bin.size();
-  for (const auto* v : {&m2m, &l2l, &up, &wp}) {
+  for (const auto* v : {&l2l, &up, &wp}) {
     std::memcpy(h + o, v->data(), v->size() * sizeof(double2));
     o += 2 * v->size();
   }
@@ -470,7 +460,6 @@ void fmm_tables(Plan& P, cudaStream_t s) {
   LENS_CUDA(cudaMemcpyAsync(d, h, nd * sizeof(double), cudaMemcpyHostToDevice, s));
   o = bin.size();
   t.binom = d;
-  t.m2m = reinterpret_cast<double2*>(d + o); o += 2 * m2m.size();
   t.l2l = reinterpret_cast<double2*>(d + o); o += 2 * l2l.size();
   t.upow = reinterpret_cast<double2*>(d + o); o += 2 * up.size();
   t.wpow = reinterpret_cast<double2*>(d + o);

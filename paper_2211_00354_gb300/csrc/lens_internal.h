@@ -106,7 +106,6 @@ struct LeafGrid {
 struct FmmTables {
   int p = 0, ldb = 0;
   double* binom = nullptr;   // C(n, k), n < 2p+2, k < p+2: binom[n*ldb + k]
-  double2* m2m = nullptr;    // [4][p+1][p+1]: row l, col k (k <= l)
   double2* l2l = nullptr;    // [4][p+1][p+1]: row j, col l (l >= j)
   double2* upow = nullptr;   // [49][p+2]: u^k for offset (dx,dy) in [-3,3]^2
   double2* wpow = nullptr;   // [p+1]: ((1+i)/2)^k, exact in float64
