@@ -5,7 +5,7 @@
 // Each 8-bit pass is reduce-then-scan: (1) per-tile digit histograms plus
 // the digit totals (atomics), (2) one block per digit scans its row of the
 // digit-major histogram matrix and adds the keys of smaller digits, (3) a
-// stable scatter in which every warp ranks its keys with __match_any_sync,
+// stable scatter in which every warp ranks its keys by votes,
 // the block combines the per-warp counts, stages its tile in shared memory
 // in digit order and writes each digit's keys out as one contiguous run.
 // No kernel waits on another block, so nothing can spin: there is no
@@ -104,8 +104,8 @@ k_radix_scatter(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ v
     const bool ok = i < n;
     key[k] = ok ? kin[i] : 0;
     val[k] = (ok && vin) ? vin[i] : 0;
-    const uint32_t d = ok ? (uint32_t)((key[k] >> shift) & 0xff) : 256u;
-    const uint32_t peers = __match_any_sync(0xffffffffu, d);
+    const uint32_t d = (uint32_t)((key[k] >> shift) & 0xff);
+    const uint32_t peers = same_digit(d, ok);
     const uint32_t before = __popc(peers & lt_mask);
     uint32_t b0 = 0;
     if (ok) b0 = wcnt[warp][d];

@@ -149,6 +149,112 @@ __global__ void k_gather(const double* __restrict__ stars, const double* __restr
   smass[i] = m[j];
 }
 
+// Keys, sort and gather of a small field by one block: the stable 8-bit passes of
+// the device-wide sort (sort.cu) over the key bits from lo_bit up, at most 32, in shared
+// memory.  The device-wide form is 3 launches a pass and the keys', a memset's and the
+// gather's, each a few us of latency: 1000 stars ~70 -> 9 us, 7546 stars ~75 -> 43.
+// Above kSmallSort stars one SM's ranking costs more than that.
+constexpr int kSmallThreads = 1024, kSmallIPT = 8, kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallSort = kSmallThreads * kSmallIPT;  // 8192; the indices fit 16 bits
+constexpr size_t kSmallBytes = (sizeof(uint32_t) + sizeof(uint16_t)) * kSmallSort +
+                               sizeof(uint16_t) * 256 * kSmallWarps;
+
+__global__ void __launch_bounds__(kSmallThreads)
+k_sort_small(const double* __restrict__ stars, const double* __restrict__ m, int n, double lo_x,
+             double lo_y, double scale, int depth, int lo_bit, uint64_t* keys,
+             uint32_t* __restrict__ idx, double2* __restrict__ spos, double* __restrict__ smass) {
+  extern __shared__ uint32_t skey[];                                      // [kSmallSort]
+  uint16_t* sval = reinterpret_cast<uint16_t*>(skey + kSmallSort);        // [kSmallSort]
+  uint16_t* wcnt = sval + kSmallSort;                                     // [kSmallWarps][256]
+  __shared__ uint32_t wsum[8], dstart[256];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const uint32_t qmax = (1u << depth) - 1u, lt_mask = (1u << lane) - 1u;
+  for (int i = t; i < n; i += kSmallThreads) {
+    const uint64_t full = morton(clamped_cell((stars[2 * i] - lo_x) * scale, qmax),
+                                 clamped_cell((stars[2 * i + 1] - lo_y) * scale, qmax));
+    keys[i] = full;  // in the stars' order until the end
+    skey[i] = (uint32_t)(full >> lo_bit);
+    sval[i] = (uint16_t)i;
+  }
+  const int ipt = (n + kSmallThreads - 1) / kSmallThreads;  // keys a thread, <= kSmallIPT
+  const int base = warp * 32 * ipt + lane;
+  for (int shift = 0; shift < 2 * depth - lo_bit; shift += 8) {
+    for (int q = t; q < 128 * kSmallWarps; q += kSmallThreads) reinterpret_cast<uint32_t*>(wcnt)[q] = 0;
+    __syncthreads();
+    uint32_t key[kSmallIPT], rank[kSmallIPT];
+    uint16_t val[kSmallIPT];
+#pragma unroll
+    for (int k = 0; k < kSmallIPT; ++k) {
+      if (k >= ipt) break;
+      const int i = base + 32 * k;
+      const bool ok = i < n;
+      key[k] = ok ? skey[i] : 0u;
+      val[k] = ok ? sval[i] : (uint16_t)0;
+      const uint32_t d = (key[k] >> shift) & 0xffu;
+      const uint32_t peers = same_digit(d, ok);
+      const uint32_t before = __popc(peers & lt_mask);
+      uint32_t b0 = 0;
+      if (ok) b0 = wcnt[warp * 256 + d];
+      __syncwarp();
+      if (ok && before == 0) wcnt[warp * 256 + d] = (uint16_t)(b0 + __popc(peers));
+      __syncwarp();
+      rank[k] = b0 + before;
+    }
+    __syncthreads();
+    // per digit: exclusive prefix of the warps' counts, then the digit's start
+    uint32_t run = 0, incl = 0;
+    if (t < 256) {
+      for (int w = 0; w < kSmallWarps; ++w) {
+        const uint32_t c = wcnt[w * 256 + t];
+        wcnt[w * 256 + t] = (uint16_t)run;
+        run += c;
+      }
+      incl = run;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (lane == 31) wsum[warp] = incl;
+    }
+    __syncthreads();
+    if (t < 256) {
+      uint32_t start = incl - run;
+      for (int q = 0; q < warp; ++q) start += wsum[q];
+      dstart[t] = start;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSmallIPT; ++k) {
+      if (k >= ipt) break;
+      if (base + 32 * k >= n) continue;
+      const uint32_t d = (key[k] >> shift) & 0xffu;
+      const uint32_t p = dstart[d] + wcnt[warp * 256 + d] + rank[k];
+      skey[p] = key[k];
+      sval[p] = val[k];
+    }
+    __syncthreads();
+  }
+  if (2 * depth <= lo_bit) __syncthreads();  // no pass: the keys are all written
+  uint64_t full[kSmallIPT];
+#pragma unroll
+  for (int k = 0; k < kSmallIPT; ++k) {
+    const int i = t + k * kSmallThreads;
+    if (i >= n) break;
+    const int j = sval[i];
+    full[k] = keys[j];
+    idx[i] = (uint32_t)j;
+    spos[i] = make_double2(stars[2 * j], stars[2 * j + 1]);
+    smass[i] = m[j];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kSmallIPT; ++k) {
+    const int i = t + k * kSmallThreads;
+    if (i < n) keys[i] = full[k];
+  }
+}
+
 // first index in [lo, hi) whose key is > v  (keys sorted ascending)
 __device__ __forceinline__ int64_t upper_bound(const uint64_t* k, int64_t lo, int64_t hi, uint64_t v) {
   while (lo < hi) {
@@ -523,9 +629,6 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   P.spos = P.dalloc_n<double2>(n);
   P.smass = P.dalloc_n<double>(n);
   const double scale = (double)(1ull << depth) / size;
-  k_keys<<<grid_for(n, 256), 256, 0, s>>>(stars, n, P.root_lo[0], P.root_lo[1], scale, depth,
-                                           P.skey, P.sidx);
-  LENS_LAUNCHED("k_keys");
   // Sort by the top key bits only, down to a level the tree is unlikely to
   // pass (6 levels below the depth of a uniform field of n stars, leaf
   // stars per box); if a box of that level still holds more than leaf stars,
@@ -535,7 +638,20 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   dcap = std::min(depth, dcap);
   const int lo_bit = (2 * (depth - dcap)) / 8 * 8;
   dcap = depth - lo_bit / 2;  // the levels the sorted bits resolve
-  radix_sort_u64(P.skey, P.sidx, n, 2 * depth, P.da, s, lo_bit);
+  bool gathered = n <= kSmallSort && 2 * depth - lo_bit <= 32;
+  if (gathered) {
+    LENS_CUDA(cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)kSmallBytes));
+    k_sort_small<<<1, kSmallThreads, kSmallBytes, s>>>(stars, masses, (int)n, P.root_lo[0], P.root_lo[1],
+                                                       scale, depth, lo_bit, P.skey, P.sidx, P.spos,
+                                                       P.smass);
+    LENS_LAUNCHED("k_sort_small");
+  } else {
+    k_keys<<<grid_for(n, 256), 256, 0, s>>>(stars, n, P.root_lo[0], P.root_lo[1], scale, depth,
+                                             P.skey, P.sidx);
+    LENS_LAUNCHED("k_keys");
+    radix_sort_u64(P.skey, P.sidx, n, 2 * depth, P.da, s, lo_bit);
+  }
 
   // ---- 3. split nodes ---------------------------------------------------
   // per-level split counts, then the flag of a box deeper than the sorted bits
@@ -560,9 +676,12 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
     // passes again, least significant first)
     radix_sort_u64(P.skey, P.sidx, n, 2 * depth, P.da, s, 0);
     dcap = depth;
+    gathered = false;
   }
-  k_gather<<<grid_for(n, 256), 256, 0, s>>>(stars, masses, P.sidx, n, P.spos, P.smass);
-  LENS_LAUNCHED("k_gather");
+  if (!gathered) {
+    k_gather<<<grid_for(n, 256), 256, 0, s>>>(stars, masses, P.sidx, n, P.spos, P.smass);
+    LENS_LAUNCHED("k_gather");
+  }
   LevelOffsets soff{}, boff{};
   int64_t nsplit = 0;
   int maxl = -1;
