@@ -191,11 +191,16 @@ k_m2m(const int* __restrict__ parent, int64_t c0, int64_t ngroups, int p,
 // ---- downward pass ---------------------------------------------------------
 // The far-field part of each local expansion (M2L over the V list, P2L over
 // the X list) reads only multipole expansions and stars, so one launch forms
-// it for the active boxes of every level at once, one warp per box: the
-// float64 work of the coarse levels, a few boxes each, spreads over the whole
-// GPU instead of a handful of SMs per level.  L2L, the only level-to-level
-// dependence, then runs level by level from the top, one thread per
-// (box, coefficient).
+// it for the active boxes of every level at once, one warp per box (kFarWarps warps
+// for a small region): the float64 work of the coarse levels, a few boxes each,
+// spreads over the whole GPU instead of a handful of SMs per level.  L2L, the
+// only level-to-level dependence, then runs level by level from the top, one
+// thread per component of a (box, coefficient).
+//
+// Bound by the float64 pipe: an SM takes a warp's float64 instruction every 19
+// cycles, whatever lanes it has, and one warp issues them 64 cycles apart.  So real
+// and imaginary parts sit in lanes of their own wherever a sum runs over fewer
+// coefficients than lanes, and a region of few boxes gives each a whole block.
 struct DownArgs {
   const int* active;
   int64_t a0, a1;
@@ -210,41 +215,54 @@ struct DownArgs {
   double lo_x, lo_y, root_size;
   int p;
   int group;         // V entries per M2L pass
-  size_t smem_warp;  // shared bytes per warp (multiple of 16)
+  size_t smem_box;   // shared bytes per box (multiple of 16)
 };
 
 // V entries per M2L pass: 32, fewer for large p so that a warp's buffers
 // (2 G (p+1) complex values) stay within 24 KB.
 inline int downward_group(int p) { return std::max(1, std::min(32, 24576 / (32 * (p + 1)))); }
-// Shared bytes per warp: the larger of the P2L buffer ((p+1) x 32 complex +
-// 64 ints) and the M2L buffers (2 G (p+1) complex + G ints).
-inline size_t downward_smem_per_warp(int p) {
-  const size_t p2l = sizeof(double2) * (size_t)(p + 1) * 32 + 64 * sizeof(int);
+// Shared bytes per box: the larger of the P2L buffer ((p+1) x 33 complex +
+// 64 ints; the odd row keeps the columns' sums off one bank) and the M2L buffers (2 G (p+1) complex + G ints).
+constexpr int kP2lRow = 33;
+inline size_t downward_smem_per_box(int p) {
+  const size_t p2l = sizeof(double2) * (size_t)(p + 1) * kP2lRow + 64 * sizeof(int);
   const size_t g = (size_t)downward_group(p);
   const size_t m2l = sizeof(double2) * 2 * g * (size_t)(p + 1) + g * sizeof(int);
   return (std::max(p2l, m2l) + 15) / 16 * 16;
 }
 
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) k_far_local(DownArgs A) {
+// NW warps a box: 1 (kWarpsPerBlock boxes a block) or kFarWarps (one box a block, for up
+// to kFarFewBoxes active boxes, which as a warp each leave most of the pipes idle:
+// 33 boxes of p 24 72 -> 28 us, 329 of p 16 42 -> 24).  A box's sums are the same, term by term, for both.
+constexpr int kFarWarps = 8;
+constexpr int64_t kFarFewBoxes = 4 * 152;
+
+template <int NW>
+__global__ void __launch_bounds__(NW == 1 ? 32 * kWarpsPerBlock : 32 * NW) k_far_local(DownArgs A) {
   extern __shared__ double2 dsm[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t a = A.a0 + (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
+  constexpr int kT = 32 * NW;  // threads of a box
+  const int t0 = NW == 1 ? threadIdx.x & 31 : threadIdx.x;
+  const int lane = threadIdx.x & 31, wib = NW == 1 ? threadIdx.x >> 5 : 0;
+  const auto sync = [] { if (NW == 1) __syncwarp(); else __syncthreads(); };
+  const int64_t a = A.a0 + (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kT;
   if (a >= A.a1) return;
   const int p = A.p, P1 = p + 1;
   const int B = A.active[a];
   const int lv = A.level[B];
   const double r = A.root_size / (double)(2ull << lv);
   const double ir = 1.0 / r;
-  double2 acc[3];
+  // component c of coefficient l: item 2 l + c, thread t0 + kT s holds one
+  constexpr int kItems = (2 * (kMaxOrder + 1) + kT - 1) / kT;
+  double acc[kItems];
 #pragma unroll
-  for (int s = 0; s < 3; ++s) acc[s] = make_double2(0.0, 0.0);
+  for (int s = 0; s < kItems; ++s) acc[s] = 0.0;
   // M2L from V.  Up to G entries at a time, their (entry, coefficient) pairs
   // spread over the lanes (p + 1 = 17 coefficients would leave 15 of 32 lanes
   // idle with one entry per pass):
   //   H[e][k] = A_k u_e^k                       (pre-scale)
   //   T[e][l] = (-1)^l u_e^(l+1) / r * sum_k C(k+l, k) H[e][k]
   //   B_l    += sum_e T[e][l]
-  double2* buf = dsm + (int64_t)wib * (A.smem_warp / sizeof(double2));
+  double2* buf = dsm + (int64_t)wib * (A.smem_box / sizeof(double2));
   const int G = A.group;
   double2* H = buf;
   double2* T = buf + (int64_t)G * P1;
@@ -252,23 +270,23 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_far_local(DownArgs A) {
   const int bx = A.ix[B], by = A.iy[B];
   for (int64_t eb = A.V_off[a]; eb < A.V_off[a + 1]; eb += G) {
     const int ne = (int)min64(G, A.V_off[a + 1] - eb);
-    for (int e = lane; e < ne; e += 32) {
+    for (int e = t0; e < ne; e += kT) {
       const int C = A.V_list[eb + e];
       uo[e] = ((A.iy[C] - by + 3) * 7 + (A.ix[C] - bx + 3)) * (p + 2);
     }
-    __syncwarp();
+    sync();
     const int ntask = ne * P1;
-    for (int t = lane; t < ntask; t += 32) {
+    for (int t = t0; t < ntask; t += kT) {
       const int e = t / P1, k = t - e * P1;
       const int C = A.V_list[eb + e];
       H[t] = cmul(ld2(A.M + (int64_t)C * P1 + k), ld2(A.tab.upow + uo[e] + k));
     }
-    __syncwarp();
-    for (int t = lane; t < ntask; t += 32) {
+    sync();
+    for (int t = t0; t < ntask; t += kT) {
       const int e = t / P1, l = t - e * P1;
       const double2* He = H + e * P1;
-      double sx = 0.0, sy = 0.0;
-      for (int k = 0; k <= p; ++k) {
+      double sx = He[0].x, sy = He[0].y;  // C(l, 0) = 1
+      for (int k = 1; k <= p; ++k) {
         // C(k+l, k) = binom[(k+l)*ldb + k]
         const double c = __ldg(A.tab.binom + (int64_t)(k + l) * A.tab.ldb + k);
         const double2 v = He[k];
@@ -279,24 +297,25 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_far_local(DownArgs A) {
       if (l & 1) post = make_double2(-post.x, -post.y);
       T[t] = cmul(post, make_double2(sx * ir, sy * ir));
     }
-    __syncwarp();
+    sync();
+    const double* Td = reinterpret_cast<const double*>(T);
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      const int l = lane + 32 * s;
-      if (l > p) break;
-      double2 v = acc[s];
-      for (int e = 0; e < ne; ++e) v = v + T[e * P1 + l];
+    for (int s = 0; s < kItems; ++s) {
+      const int i = t0 + kT * s;
+      if (i >= 2 * P1) break;
+      double v = acc[s];
+      for (int e = 0; e < ne; ++e) v = v + Td[2 * e * P1 + i];
       acc[s] = v;
     }
-    __syncwarp();
+    sync();
   }
   // P2L from X.  The stars of the X boxes are taken 32 at a time across box
   // boundaries: lane j forms the series -m_j/(z_j-c) (r/(z_j-c))^l of its
-  // star by recurrence into shared memory, then lane l sums column l.  (One
+  // star by recurrence into shared memory, then a lane sums a column's component.  (One
   // star at a time with per-lane powers would idle most of the warp when the
   // X boxes hold a few stars each.)
   const double cx = A.lo_x + (2.0 * bx + 1.0) * r, cy = A.lo_y + (2.0 * by + 1.0) * r;
-  int* xs = reinterpret_cast<int*>(buf + (int64_t)P1 * 32);  // [32] inclusive counts, [32] starts
+  int* xs = reinterpret_cast<int*>(buf + (int64_t)P1 * kP2lRow);  // [32] inclusive counts, [32] starts
   for (int64_t eb = A.X_off[a]; eb < A.X_off[a + 1]; eb += 32) {
     const int ne = (int)min64(32, A.X_off[a + 1] - eb);
     int cnt = 0, st = 0;
@@ -312,13 +331,15 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_far_local(DownArgs A) {
       if (lane >= o) incl += v;
     }
     const int total = __shfl_sync(0xffffffffu, incl, 31);
-    __syncwarp();
-    xs[lane] = incl;
-    xs[32 + lane] = st;
-    __syncwarp();
+    sync();
+    if (t0 < 32) {
+      xs[lane] = incl;
+      xs[32 + lane] = st;
+    }
+    sync();
     for (int f0 = 0; f0 < total; f0 += 32) {
       const int f = f0 + lane;
-      if (f < total) {
+      if (t0 < 32 && f < total) {
         int e = 0;
         while (xs[e] <= f) ++e;  // first box whose inclusive count exceeds f
         const int j = xs[32 + e] + f - (e ? xs[e - 1] : 0);
@@ -328,51 +349,64 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock) k_far_local(DownArgs A) {
         const double2 q = make_double2(inv.x * r, inv.y * r);        // r/(z-c)
         double2 v = make_double2(-m * inv.x, -m * inv.y);            // -m/(z-c)
         for (int l = 0; l <= p; ++l) {
-          buf[l * 32 + lane] = v;
+          buf[l * kP2lRow + lane] = v;
           v = cmul(v, q);
         }
       }
-      __syncwarp();
+      sync();
       const int nv = min(32, total - f0);
+      const double* bd = reinterpret_cast<const double*>(buf);
 #pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const int l = lane + 32 * s;
-        if (l > p) break;
-        double2 v = acc[s];
-        for (int jj = 0; jj < nv; ++jj) v = v + buf[l * 32 + jj];
+      for (int s = 0; s < kItems; ++s) {
+        const int i = t0 + kT * s;
+        if (i >= 2 * P1) break;
+        const double* col = bd + 2 * (i >> 1) * kP2lRow + (i & 1);
+        double v = acc[s];
+        for (int jj = 0; jj < nv; ++jj) v = v + col[2 * jj];
         acc[s] = v;
       }
-      __syncwarp();
+      sync();
     }
   }
-  double2* out = A.L + (int64_t)B * P1;
+  double* out = reinterpret_cast<double*>(A.L + (int64_t)B * P1);
 #pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const int l = lane + 32 * s;
-    if (l <= p) out[l] = acc[s];
+  for (int s = 0; s < kItems; ++s) {
+    const int i = t0 + kT * s;
+    if (i < 2 * P1) out[i] = acc[s];
   }
 }
 
 // L2L of the active boxes of one level (>= 2; above it the parent's local
-// expansion is zero), one thread per (box, coefficient j):
+// expansion is zero), one thread per component of a (box, coefficient j):
 //   L_B[j] += sum_{l >= j} S_q[j][l] L_parent[l],  q = the box's quadrant.
-// The parent of an active box is active and its expansion is final.
-__global__ void k_l2l(const int* __restrict__ active, int64_t a0, int64_t a1,
+// The parent of an active box is active and its expansion is final.  Few boxes: two
+// products a term 64 cycles apart (a thread per complex coefficient, four):
+// 8.5 -> 7 us a level.  Small blocks, so that the warps of a level spread over the SMs.
+constexpr int kL2LThreads = 64;
+
+__global__ void __launch_bounds__(kL2LThreads)
+k_l2l(const int* __restrict__ active, int64_t a0, int64_t a1,
                       const int* __restrict__ parent, const int* __restrict__ child,
                       const double2* __restrict__ l2l, int p, double2* __restrict__ L) {
   const int P1 = p + 1;
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t a = a0 + t / P1;
+  const int64_t a = a0 + t / (2 * P1);
   if (a >= a1) return;
-  const int j = (int)(t - (a - a0) * P1);
+  const int i = (int)(t - (a - a0) * (2 * P1)), j = i >> 1, c = i & 1;
   const int B = active[a];
   const int par = parent[B];
   const int q = B - child[par];
   const double2* Lp = L + (int64_t)par * P1;
   const double2* S = l2l + ((int64_t)q * P1 + j) * P1;
-  double2 v = make_double2(0.0, 0.0);
-  for (int l = j; l <= p; ++l) v = cfma(ld2(S + l), ld2(Lp + l), v);
-  double2* o = L + (int64_t)B * P1 + j;
+  // component c of the sum, by cfma's products in its order: -z.y or z.x with the
+  // imaginary part of S, then z.x or z.y with the real one
+  double v = 0.0;
+  for (int l = j; l <= p; ++l) {
+    const double2 s2 = ld2(S + l), z = ld2(Lp + l);
+    const double w = c ? z.x : __hiloint2double(__double2hiint(z.y) ^ 0x80000000, __double2loint(z.y));
+    v = fma(s2.x, c ? z.y : z.x, fma(s2.y, w, v));
+  }
+  double* o = reinterpret_cast<double*>(L + (int64_t)B * P1 + j) + c;
   *o = *o + v;
 }
 
@@ -539,15 +573,18 @@ void fmm_downward(Plan& P, cudaStream_t s) {
   A.spos = P.spos; A.smass = P.smass; A.M = P.M; A.L = P.L; A.tab = t;
   A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.root_size = P.root_size; A.p = P.p;
   A.group = downward_group(P.p);
-  A.smem_warp = downward_smem_per_warp(P.p);
-  const size_t smem = A.smem_warp * kWarpsPerBlock;
+  A.smem_box = downward_smem_per_box(P.p);
+  const bool few = P.n_active <= kFarFewBoxes;
+  const size_t smem = A.smem_box * (few ? 1 : kWarpsPerBlock);
   if (smem > 48 * 1024)
-    LENS_CUDA(cudaFuncSetAttribute(k_far_local, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LENS_CUDA(cudaFuncSetAttribute(few ? k_far_local<kFarWarps> : k_far_local<1>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   A.a0 = 0;
   A.a1 = P.n_active;
   if (A.a1 > 0) {
     if (P.ev_far0) LENS_CUDA(cudaEventRecord(P.ev_far0, s));
-    k_far_local<<<grid_for(A.a1 * 32, 32 * kWarpsPerBlock), 32 * kWarpsPerBlock, smem, s>>>(A);
+    if (few) k_far_local<kFarWarps><<<(unsigned)A.a1, 32 * kFarWarps, smem, s>>>(A);
+    else k_far_local<1><<<grid_for(A.a1 * 32, 32 * kWarpsPerBlock), 32 * kWarpsPerBlock, smem, s>>>(A);
     LENS_LAUNCHED("k_far_local");
     if (P.ev_far1) LENS_CUDA(cudaEventRecord(P.ev_far1, s));
   }
@@ -555,8 +592,8 @@ void fmm_downward(Plan& P, cudaStream_t s) {
   for (int l = 2; l < P.nlevels; ++l) {
     const int64_t a0 = P.active_level_off[l], a1 = P.active_level_off[l + 1];
     if (a1 <= a0) continue;
-    k_l2l<<<grid_for((a1 - a0) * P1, 128), 128, 0, s>>>(P.active, a0, a1, P.box_parent,
-                                                       P.box_child, t.l2l, P.p, P.L);
+    k_l2l<<<grid_for((a1 - a0) * 2 * P1, kL2LThreads), kL2LThreads, 0, s>>>(
+        P.active, a0, a1, P.box_parent, P.box_child, t.l2l, P.p, P.L);
     LENS_LAUNCHED("k_l2l");
   }
 }

@@ -1,6 +1,6 @@
-"""The far field's translations (M2L by quarter-turn orbits, L2L from the parents)
-at expansion orders about the sizes of a warp and of a block's groups, on trees
-whose V lists are full, cut by the target region, and one-sided."""
+"""The far field's translations (M2L, P2L, L2L) at expansion orders about the sizes of
+a warp and of a block's groups, with a warp a box and a block a box (a small target
+region), on trees whose V lists are full, cut by the target region, and one-sided."""
 import numpy as np
 import pytest
 import torch
