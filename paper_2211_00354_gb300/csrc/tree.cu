@@ -481,103 +481,144 @@ struct ListOut {
   const int64_t* oV; const int64_t* oX; const int64_t* oU; const int64_t* oW;  // offsets (pass 2)
   int* V; int* X; int* U; int* W;
   int64_t* ustars;  // per active index: stars in U (pass 1)
-  const int* nbr;   // per active index: 18 neighbour boxes (k_neighbours)
+  int* nbr;         // per active index: 18 neighbour boxes (pass 1)
+  int2* uw;         // per active index and neighbour 9 .. 17: U and W entries (pass 1)
 };
 
-// The 18 neighbour lookups of each active box, one thread each: [0..8] the
-// boxes at level l-1 around its parent (V and X lists, levels >= 2), [9..17]
-// the boxes at level l around it (U and W lists, leaves), in the row-major
-// (dy, dx) order the list kernel walks them; -1 outside the root or unused.
-// A lookup is a binary search per level, so spreading them over threads
-// shortens the chains of dependent loads the list kernel would wait on.
-__global__ void k_neighbours(TreeView T, const int* __restrict__ active, int64_t nact,
-                             int* __restrict__ nbr) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= nact * 18) return;
-  const int64_t a = t / 18;
-  const int q = (int)(t - a * 18), q9 = q % 9;
-  const int dx = q9 % 3 - 1, dy = q9 / 3 - 1;
-  const int B = active[a];
-  const int l = T.level[B];
-  const long long bx = T.ix[B], by = T.iy[B];
-  int r = -1;
-  if (q < 9) {
-    if (l >= 2) r = find_box(T, l - 1, (bx >> 1) + dx, (by >> 1) + dy);
-  } else if (T.child[B] < 0) {
-    r = find_box(T, l, bx + dx, by + dy);
-  }
-  nbr[t] = r;
-}
+// The lists of each active box, a warp a box and a lane a neighbour, in two passes:
+// count, then write.  Lanes 0 .. 8 take the boxes at level l - 1 around the parent (V
+// and X, levels >= 2), lanes 9 .. 17 those at level l around the box (U and W,
+// leaves), in row-major (dy, dx) order, which is the order of the lists: a lane's
+// entries follow those of the lanes before it.  A neighbour that is coarser than asked
+// for covers several places; the first lane that finds it keeps it.  Bound by chains of
+// dependent loads (binary searches, then the boxes below a neighbour), which a thread
+// a box walked one neighbour after another: both passes and the lookups, 33 boxes
+// 48 -> 10 us, 2.4e4 boxes 128 -> 89; 1.1e5 boxes, enough to hide the chains, 155 -> 178.
+constexpr int kListThreads = 128;
 
 template <bool WRITE>
-__global__ void k_lists(TreeView T, const int* __restrict__ active, int64_t nact, ListOut o) {
-  const int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kListThreads)
+k_lists(TreeView T, const int* __restrict__ active, int64_t nact, ListOut o) {
+  const int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (a >= nact) return;
+  const int lane = threadIdx.x & 31;
   const int B = active[a];
   const int l = T.level[B];
-  int64_t nV = 0, nX = 0, nU = 0, nW = 0, us = 0;
-  int64_t pV = WRITE ? o.oV[a] : 0, pX = WRITE ? o.oX[a] : 0;
-  int64_t pU = WRITE ? o.oU[a] : 0, pW = WRITE ? o.oW[a] : 0;
-  if (l >= 2) {
-    int seen[9];
-    int nseen = 0;
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int Q = o.nbr[a * 18 + (dy + 1) * 3 + (dx + 1)];
-        if (Q < 0) continue;
-        if (T.level[Q] == l - 1 && T.child[Q] >= 0) {
-          for (int q = 0; q < 4; ++q) {
-            const int C = T.child[Q] + q;
-            if (T.count[C] == 0 || adjacent(T, C, B)) continue;
-            if (WRITE) o.V[pV++] = C;
-            ++nV;
-          }
-        } else {
-          bool dup = false;
-          for (int s = 0; s < nseen; ++s) dup |= (seen[s] == Q);
-          if (dup) continue;
-          seen[nseen++] = Q;
-          if (T.count[Q] == 0 || adjacent(T, Q, B)) continue;
-          if (WRITE) o.X[pX++] = Q;
-          ++nX;
-        }
-      }
+  const bool leaf = T.child[B] < 0;
+  const bool near = lane >= 9;  // U and W
+  const int q9 = near ? lane - 9 : lane, dx = q9 % 3 - 1, dy = q9 / 3 - 1;
+  const int bx = T.ix[B], by = T.iy[B];
+  int Q = -1;
+  if (WRITE) {
+    if (lane < 18) Q = o.nbr[a * 18 + lane];
+  } else if (lane < 18) {
+    if (!near) {
+      if (l >= 2) Q = find_box(T, l - 1, (bx >> 1) + dx, (by >> 1) + dy);
+    } else if (leaf) {
+      Q = find_box(T, l, (long long)bx + dx, (long long)by + dy);
+    }
+    o.nbr[a * 18 + lane] = Q;
   }
-  if (T.child[B] < 0) {
-    int seen[9];
-    int nseen = 0;
-    int stack[128];
-    for (int dy = -1; dy <= 1; ++dy)
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int C = o.nbr[a * 18 + 9 + (dy + 1) * 3 + (dx + 1)];
-        if (C < 0) continue;
-        if (T.level[C] < l) {
-          bool dup = false;
-          for (int s = 0; s < nseen; ++s) dup |= (seen[s] == C);
-          if (dup) continue;
-          seen[nseen++] = C;
-          if (T.count[C] > 0) { if (WRITE) o.U[pU++] = C; ++nU; us += T.count[C]; }
-          continue;
-        }
-        if (T.count[C] == 0) continue;
-        if (T.child[C] < 0) { if (WRITE) o.U[pU++] = C; ++nU; us += T.count[C]; continue; }
-        int sp = 0;
-        for (int q = 3; q >= 0; --q) stack[sp++] = T.child[C] + q;
-        while (sp > 0) {
-          const int Dn = stack[--sp];
-          if (T.count[Dn] == 0) continue;
-          if (adjacent(T, Dn, B)) {
-            if (T.child[Dn] < 0) { if (WRITE) o.U[pU++] = Dn; ++nU; us += T.count[Dn]; }
-            else if (sp + 4 <= 128) { for (int q = 3; q >= 0; --q) stack[sp++] = T.child[Dn] + q; }
-          } else {
-            if (WRITE) o.W[pW++] = Dn;
-            ++nW;
-          }
-        }
+  int nV = 0, nX = 0, nU = 0, nW = 0, us = 0;
+  unsigned vmask = 0;        // children of Q in V
+  bool descend = false;      // U and W entries below Q
+  const int Qc = Q >= 0 ? T.child[Q] : -1, Ql = Q >= 0 ? T.level[Q] : 0;
+  const bool split = !near && Ql == l - 1 && Qc >= 0;
+  // a coarser (or childless) neighbour found by an earlier lane of the same nine
+  bool dup = false;
+  if (__any_sync(0xffffffffu, Q >= 0 && !split && (!near || Ql < l))) {
+#pragma unroll
+    for (int j = 0; j < 17; ++j) {
+      const int e = __shfl_sync(0xffffffffu, Q, j);
+      dup |= j < lane && (j >= 9) == near && e == Q;
+    }
+  }
+  if (Q >= 0 && !near) {
+    if (split) {
+      // the children have B's level: not next to it when a coordinate is off by two
+      const int ox = 2 * ((bx >> 1) + dx) - bx, oy = 2 * ((by >> 1) + dy) - by;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int cx = ox + (q & 1), cy = oy + (q >> 1);
+        const bool far = cx < -1 || cx > 1 || cy < -1 || cy > 1;
+        if (far && T.count[Qc + q] != 0) vmask |= 1u << q;
       }
+      nV = __popc(vmask);
+    } else if (!dup && T.count[Q] != 0 && !adjacent(T, Q, B)) {
+      nX = 1;
+    }
+  } else if (Q >= 0) {
+    const int c = T.count[Q];
+    if (Ql < l) {
+      if (!dup && c > 0) { nU = 1; us = c; }
+    } else if (c > 0) {
+      if (Qc < 0) { nU = 1; us = c; } else descend = true;
+    }
+  }
+  // f(box, in U) for the boxes below Q in order: leaves next to B, and the largest
+  // boxes that are not
+  const auto walk = [&](auto f) {
+    int stack[128];
+    int sp = 0;
+    for (int q = 3; q >= 0; --q) stack[sp++] = Qc + q;
+    while (sp > 0) {
+      const int Dn = stack[--sp];
+      if (T.count[Dn] == 0) continue;
+      const int ch = T.child[Dn];
+      if (!adjacent(T, Dn, B)) f(Dn, false);
+      else if (ch < 0) f(Dn, true);
+      else if (sp + 4 <= 128) { for (int q = 3; q >= 0; --q) stack[sp++] = ch + q; }
+    }
+  };
+  if (descend) {
+    if (WRITE) {
+      const int2 n = o.uw[a * 9 + lane - 9];
+      nU = n.x;
+      nW = n.y;
+    } else {
+      walk([&](int Dn, bool u) { if (u) { ++nU; us += T.count[Dn]; } else { ++nW; } });
+      o.uw[a * 9 + lane - 9] = make_int2(nU, nW);
+    }
+  }
+  // places within the box's lists
+  const auto scan = [&](int v) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += y;
+    }
+    return v;
+  };
+  // (nV <= 4, and without a descent nU and nX <= 1: votes)
+  const unsigned le = 0xffffffffu >> (31 - lane);
+  const auto votes = [&](bool v) { return __popc(__ballot_sync(0xffffffffu, v) & le); };
+  const int iV = votes(nV & 1) + 2 * votes(nV & 2) + 4 * votes(nV & 4);
+  const int iX = votes(nX);
+  int iU = 0, iW = 0;
+  if (!leaf) {
+  } else if (__any_sync(0xffffffffu, descend)) {
+    iU = scan(nU);
+    iW = scan(nW);
+  } else {
+    iU = votes(nU);
   }
   if (!WRITE) {
-    o.cV[a] = nV; o.cX[a] = nX; o.cU[a] = nU; o.cW[a] = nW; o.ustars[a] = us;
+    const int64_t su = leaf ? __reduce_add_sync(0xffffffffu, us) : 0;
+    if (lane == 31) { o.cV[a] = iV; o.cX[a] = iX; o.cU[a] = iU; o.cW[a] = iW; o.ustars[a] = su; }
+    return;
+  }
+  if (nV) {
+    int64_t at = o.oV[a] + iV - nV;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (vmask >> q & 1u) o.V[at++] = Qc + q;
+  }
+  if (nX) o.X[o.oX[a] + iX - nX] = Q;
+  if (descend) {
+    int64_t pU = o.oU[a] + iU - nU, pW = o.oW[a] + iW - nW;
+    walk([&](int Dn, bool u) { if (u) o.U[pU++] = Dn; else o.W[pW++] = Dn; });
+  } else if (nU) {
+    o.U[o.oU[a] + iU - nU] = Q;
   }
 }
 
@@ -782,13 +823,10 @@ void tree_build_lists(Plan& P, cudaStream_t s) {
   P.ustar_cnt = P.dalloc_n<int64_t>(na + 1);
   ListOut o{};
   o.cV = c; o.cX = c + na; o.cU = c + 2 * na; o.cW = c + 3 * na; o.ustars = P.ustar_cnt;
-  Scratch nbr(&P.da, sizeof(int) * 18 * (size_t)std::max<int64_t>(na, 1));
-  if (na > 0) {
-    k_neighbours<<<grid_for(na * 18, 256), 256, 0, s>>>(T, P.active, na, nbr.as<int>());
-    LENS_LAUNCHED("k_neighbours");
-  }
-  o.nbr = nbr.as<int>();
-  k_lists<false><<<grid_for(na, 128), 128, 0, s>>>(T, P.active, na, o);
+  Scratch nbr(&P.da, (sizeof(int2) * 9 + sizeof(int) * 18) * (size_t)std::max<int64_t>(na, 1));
+  o.uw = nbr.as<int2>();
+  o.nbr = reinterpret_cast<int*>(o.uw + 9 * std::max<int64_t>(na, 1));
+  k_lists<false><<<grid_for(na * 32, kListThreads), kListThreads, 0, s>>>(T, P.active, na, o);
   LENS_LAUNCHED("k_lists<count>");
   int64_t* offs[4];
   int64_t tot[5];
@@ -814,7 +852,7 @@ void tree_build_lists(Plan& P, cudaStream_t s) {
   P.W_list = P.dalloc_n<int>(tot[3]);
   o.oV = offs[0]; o.oX = offs[1]; o.oU = offs[2]; o.oW = offs[3];
   o.V = P.V_list; o.X = P.X_list; o.U = P.U_list; o.W = P.W_list;
-  k_lists<true><<<grid_for(na, 128), 128, 0, s>>>(T, P.active, na, o);
+  k_lists<true><<<grid_for(na * 32, kListThreads), kListThreads, 0, s>>>(T, P.active, na, o);
   LENS_LAUNCHED("k_lists<write>");
   P.V_off = offs[0];
   P.X_off = offs[1];
