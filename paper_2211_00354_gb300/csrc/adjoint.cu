@@ -61,14 +61,13 @@ struct AdjArgs {
 // A box's half side, its inverse and its centre, without a division or a conversion
 // on the float64 pipe (a block of few rays formed them at ~40 operations there).
 __device__ __forceinline__ double box_r(const AdjArgs& A, int b) {
-  return mul_pow2(A.size, -(A.level[b] + 1));
+  return box_half(A.size, A.level[b]);
 }
 __device__ __forceinline__ double box_ir(const AdjArgs& A, int b) {
-  return mul_pow2(A.isize, A.level[b] + 1);
+  return box_inv_half(A.isize, A.level[b]);
 }
 __device__ __forceinline__ double2 box_c(const AdjArgs& A, int b, double r) {
-  return make_double2(fma(u2d(2u * (unsigned)A.ix[b] + 1u), r, A.lo_x),
-                      fma(u2d(2u * (unsigned)A.iy[b] + 1u), r, A.lo_y));
+  return make_double2(box_centre(A.lo_x, A.ix[b], r), box_centre(A.lo_y, A.iy[b], r));
 }
 
 // One warp per (leaf, tile): L2P^T moments of the tile's rays and M2P^T for

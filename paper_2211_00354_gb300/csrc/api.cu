@@ -289,6 +289,7 @@ lens_status lens_fmm_build(const double* stars_xy, const double* masses, int64_t
     } restore{P.da, P.da.stream};
     P.da.stream = P.fmm_stream;
     tree_build_lists(P, P.fmm_stream);
+    fmm_alloc_far(P);
   }
   LENS_CUDA(cudaEventRecord(P.ev_lists, P.fmm_stream));
   LENS_CUDA(cudaStreamWaitEvent(P.fmm_stream, P.ev_up, 0));

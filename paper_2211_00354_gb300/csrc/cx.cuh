@@ -107,6 +107,14 @@ __device__ __forceinline__ double mul_pow2(double x, int k) {
   return __hiloint2double(H + k * 0x100000, __double2loint(x));
 }
 
+// Half side and centre of the box (level, ix, iy) of a root of side `size` at lo, and
+// 1 / (half side) from 1 / size: divisions by powers of two, without the float64 pipe's.
+__device__ __forceinline__ double box_half(double size, int level) { return mul_pow2(size, -(level + 1)); }
+__device__ __forceinline__ double box_inv_half(double isize, int level) { return mul_pow2(isize, level + 1); }
+__device__ __forceinline__ double box_centre(double lo, int i, double half) {
+  return fma(u2d(2u * (unsigned)i + 1u), half, lo);
+}
+
 // Error-free sum of two floats (Knuth two-sum): s + e == a + b exactly.
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = a + b;

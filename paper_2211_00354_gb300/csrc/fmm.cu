@@ -68,6 +68,38 @@ __global__ void k_leaf_bins(const int* __restrict__ count, const int* __restrict
   if (PASS == 1 && key > 0) list[offs[key] + base + __popc(peers & ((1u << lane) - 1u))] = (int)b;
 }
 
+// All of it by one block, for a small tree: the two passes, the offsets and two
+// memsets are five short operations (321 boxes: ~18 us with their gaps -> 3).
+constexpr int kBinThreads = 1024, kBinSmallBoxes = 8192, kBinSmallLeaf = 64;
+
+__global__ void __launch_bounds__(kBinThreads)
+k_leaf_bins_small(const int* __restrict__ count, const int* __restrict__ child, int nb, int p,
+                  int leaf_size, int* __restrict__ offs, int* __restrict__ list, double2* __restrict__ M) {
+  __shared__ int bins[kBinSmallLeaf + 1];
+  for (int k = threadIdx.x; k <= kBinSmallLeaf; k += kBinThreads) bins[k] = 0;
+  __syncthreads();
+  for (int b = threadIdx.x; b < nb; b += kBinThreads) {
+    if (child[b] >= 0) continue;
+    const int nst = count[b];
+    if (nst > 0) {
+      atomicAdd(&bins[min(nst, leaf_size)], 1);
+    } else {
+      double2* out = M + b * (int64_t)(p + 1);
+      for (int k = 0; k <= p; ++k) out[k] = make_double2(0.0, 0.0);
+    }
+  }
+  __syncthreads();
+  // bins[k]: the first place of count k, largest counts first
+  if (threadIdx.x == 0) {
+    int acc = 0;
+    for (int k = leaf_size; k >= 1; --k) { const int c = bins[k]; bins[k] = acc; acc += c; }
+    offs[0] = acc;  // leaves in the list
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < nb; b += kBinThreads)
+    if (child[b] < 0 && count[b] > 0) list[atomicAdd(&bins[min(count[b], leaf_size)], 1)] = b;
+}
+
 // offs[k] for counts k = leaf_size .. 1 (descending), offs[0] = total
 __global__ void k_bin_offsets(const int* __restrict__ bins, int leaf_size, int* __restrict__ offs) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
@@ -212,7 +244,7 @@ struct DownArgs {
   const double2* M;
   double2* L;
   FmmTables tab;
-  double lo_x, lo_y, root_size;
+  double lo_x, lo_y, root_size, inv_size;
   int p;
   int group;         // V entries per M2L pass
   size_t smem_box;   // shared bytes per box (multiple of 16)
@@ -233,7 +265,7 @@ inline size_t downward_smem_per_box(int p) {
 
 // NW warps a box: 1 (kWarpsPerBlock boxes a block) or kFarWarps (one box a block, for up
 // to kFarFewBoxes active boxes, which as a warp each leave most of the pipes idle:
-// 33 boxes of p 24 72 -> 28 us, 329 of p 16 42 -> 24).  A box's sums are the same, term by term, for both.
+// 33 boxes of p 24 72 -> 17 us, 329 of p 16 42 -> 22).  A box's sums are the same, term by term, for both.
 constexpr int kFarWarps = 8;
 constexpr int64_t kFarFewBoxes = 4 * 152;
 
@@ -249,8 +281,7 @@ __global__ void __launch_bounds__(NW == 1 ? 32 * kWarpsPerBlock : 32 * NW) k_far
   const int p = A.p, P1 = p + 1;
   const int B = A.active[a];
   const int lv = A.level[B];
-  const double r = A.root_size / (double)(2ull << lv);
-  const double ir = 1.0 / r;
+  const double r = box_half(A.root_size, lv), ir = box_inv_half(A.inv_size, lv);
   // component c of coefficient l: item 2 l + c, thread t0 + kT s holds one
   constexpr int kItems = (2 * (kMaxOrder + 1) + kT - 1) / kT;
   double acc[kItems];
@@ -314,7 +345,7 @@ __global__ void __launch_bounds__(NW == 1 ? 32 * kWarpsPerBlock : 32 * NW) k_far
   // star by recurrence into shared memory, then a lane sums a column's component.  (One
   // star at a time with per-lane powers would idle most of the warp when the
   // X boxes hold a few stars each.)
-  const double cx = A.lo_x + (2.0 * bx + 1.0) * r, cy = A.lo_y + (2.0 * by + 1.0) * r;
+  const double cx = box_centre(A.lo_x, bx, r), cy = box_centre(A.lo_y, by, r);
   int* xs = reinterpret_cast<int*>(buf + (int64_t)P1 * kP2lRow);  // [32] inclusive counts, [32] starts
   for (int64_t eb = A.X_off[a]; eb < A.X_off[a + 1]; eb += 32) {
     const int ne = (int)min64(32, A.X_off[a + 1] - eb);
@@ -368,7 +399,8 @@ __global__ void __launch_bounds__(NW == 1 ? 32 * kWarpsPerBlock : 32 * NW) k_far
       sync();
     }
   }
-  double* out = reinterpret_cast<double*>(A.L + (int64_t)B * P1);
+  // by box, or by active index for the chain
+  double* out = reinterpret_cast<double*>(A.L + (NW == 1 ? (int64_t)B : a) * P1);
 #pragma unroll
   for (int s = 0; s < kItems; ++s) {
     const int i = t0 + kT * s;
@@ -408,6 +440,54 @@ k_l2l(const int* __restrict__ active, int64_t a0, int64_t a1,
   }
   double* o = reinterpret_cast<double*>(L + (int64_t)B * P1 + j) + c;
   *o = *o + v;
+}
+
+// For a small region (kFarFewBoxes): a block per active box forms the local expansions of
+// its ancestors from level 1 down and then its own, the same operations in the same order as
+// level by level, from the far-field parts F (by active index) into L; one launch, each
+// level's few boxes repeated by those below them, instead of one per level (33 boxes of p 24 on
+// 4 levels 41 us with the launches' gaps -> 17, 324 boxes of p 16 on 14 levels 90 -> 35).
+__global__ void k_l2l_chain(const int* __restrict__ active, const int* __restrict__ parent,
+                            const int* __restrict__ aidx, const int* __restrict__ level,
+                            const int* __restrict__ ix, const int* __restrict__ iy,
+                            const double2* __restrict__ l2l, int p, const double2* __restrict__ F,
+                            double2* __restrict__ L) {
+  __shared__ int anc[kMaxDepth + 2];        // active index of the ancestor of each level
+  __shared__ double2 cur[2][kMaxOrder + 1];
+  const int P1 = p + 1, i = threadIdx.x, j = i >> 1, c = i & 1;
+  const int B = active[blockIdx.x], lv = level[B], bx = ix[B], by = iy[B];
+  if (i == 0) {
+    int b = B;
+    for (int l = lv; l >= 0; --l) { anc[l] = aidx[b]; if (l) b = parent[b]; }
+  }
+  __syncthreads();
+  const bool on = i < 2 * P1;
+  const auto far = [&](int l) {
+    return on ? reinterpret_cast<const double*>(F + (int64_t)anc[l] * P1)[i] : 0.0;
+  };
+  int l = min(lv, 1);  // the expansions of levels 0 and 1 are their far parts
+  double x = far(l);
+  for (;;) {
+    const double next = l < lv ? far(l + 1) : 0.0;
+    double2* now = cur[l & 1];
+    if (on) reinterpret_cast<double*>(now)[i] = x;
+    if (l == lv) break;
+    __syncthreads();
+    ++l;
+    if (on) {
+      const int s = lv - l, q = ((bx >> s) & 1) | (((by >> s) & 1) << 1);
+      const double2* S = l2l + ((int64_t)q * P1 + j) * P1;
+      double v = 0.0;
+#pragma unroll 4
+      for (int k = j; k <= p; ++k) {
+        const double2 s2 = ld2(S + k), z = now[k];
+        const double w = c ? z.x : __hiloint2double(__double2hiint(z.y) ^ 0x80000000, __double2loint(z.y));
+        v = fma(s2.x, c ? z.y : z.x, fma(s2.y, w, v));
+      }
+      x = next + v;
+    }
+  }
+  if (on) reinterpret_cast<double*>(L + (int64_t)B * P1)[i] = x;
 }
 
 }  // namespace
@@ -507,6 +587,11 @@ void fmm_alloc(Plan& P) {
   if (!P.p2m_bins) P.p2m_bins = P.dalloc_n<int>(2 * ((size_t)P.leaf + 1));
 }
 
+void fmm_alloc_far(Plan& P) {
+  if (P.n_active > 0 && P.n_active <= kFarFewBoxes)
+    P.L_far = P.dalloc_n<double2>((size_t)P.n_active * (P.p + 1));
+}
+
 void fmm_p2m(Plan& P, cudaStream_t s) {
   const int p = P.p, P1 = p + 1;
   if (!P.M || !P.p2m_list || !P.p2m_bins) fail(LENS_ECUDA, "internal: expansion buffers not allocated");
@@ -516,16 +601,21 @@ void fmm_p2m(Plan& P, cudaStream_t s) {
   int* cnt = P.p2m_bins;
   int* offs = cnt + (L + 1);
   int* list = P.p2m_list;
-  LENS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(L + 1), s));
-  k_leaf_bins<0><<<grid_for(P.nb, 256), 256, 0, s>>>(P.box_count, P.box_child, P.nb, p, L, cnt, offs,
-                                                      list, P.M);
-  LENS_LAUNCHED("k_leaf_bins<count>");
-  k_bin_offsets<<<1, 32, 0, s>>>(cnt, L, offs);
-  LENS_LAUNCHED("k_bin_offsets");
-  LENS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(L + 1), s));
-  k_leaf_bins<1><<<grid_for(P.nb, 256), 256, 0, s>>>(P.box_count, P.box_child, P.nb, p, L, cnt, offs,
-                                                      list, P.M);
-  LENS_LAUNCHED("k_leaf_bins<place>");
+  if (P.nb <= kBinSmallBoxes && L <= kBinSmallLeaf) {
+    k_leaf_bins_small<<<1, kBinThreads, 0, s>>>(P.box_count, P.box_child, (int)P.nb, p, L, offs, list, P.M);
+    LENS_LAUNCHED("k_leaf_bins_small");
+  } else {
+    LENS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(L + 1), s));
+    k_leaf_bins<0><<<grid_for(P.nb, 256), 256, 0, s>>>(P.box_count, P.box_child, P.nb, p, L, cnt, offs,
+                                                        list, P.M);
+    LENS_LAUNCHED("k_leaf_bins<count>");
+    k_bin_offsets<<<1, 32, 0, s>>>(cnt, L, offs);
+    LENS_LAUNCHED("k_bin_offsets");
+    LENS_CUDA(cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)(L + 1), s));
+    k_leaf_bins<1><<<grid_for(P.nb, 256), 256, 0, s>>>(P.box_count, P.box_child, P.nb, p, L, cnt, offs,
+                                                        list, P.M);
+    LENS_LAUNCHED("k_leaf_bins<place>");
+  }
   const int tpb = 32;
   if (P.prec == LENS_FP32_BULK) {
     const size_t smem = sizeof(float2) * (size_t)P1 * tpb;
@@ -571,10 +661,12 @@ void fmm_downward(Plan& P, cudaStream_t s) {
   A.ix = P.box_ix; A.iy = P.box_iy; A.start = P.box_start; A.count = P.box_count;
   A.V_off = P.V_off; A.V_list = P.V_list; A.X_off = P.X_off; A.X_list = P.X_list;
   A.spos = P.spos; A.smass = P.smass; A.M = P.M; A.L = P.L; A.tab = t;
-  A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.root_size = P.root_size; A.p = P.p;
+  A.lo_x = P.root_lo[0]; A.lo_y = P.root_lo[1]; A.root_size = P.root_size;
+  A.inv_size = 1.0 / P.root_size; A.p = P.p;
   A.group = downward_group(P.p);
   A.smem_box = downward_smem_per_box(P.p);
-  const bool few = P.n_active <= kFarFewBoxes;
+  const bool few = P.L_far != nullptr;
+  if (few) A.L = P.L_far;
   const size_t smem = A.smem_box * (few ? 1 : kWarpsPerBlock);
   if (smem > 48 * 1024)
     LENS_CUDA(cudaFuncSetAttribute(few ? k_far_local<kFarWarps> : k_far_local<1>,
@@ -589,6 +681,12 @@ void fmm_downward(Plan& P, cudaStream_t s) {
     if (P.ev_far1) LENS_CUDA(cudaEventRecord(P.ev_far1, s));
   }
   const int P1 = P.p + 1;
+  if (few) {
+    k_l2l_chain<<<(unsigned)P.n_active, (2 * P1 + 31) / 32 * 32, 0, s>>>(
+        P.active, P.box_parent, P.box_aidx, P.box_level, P.box_ix, P.box_iy, t.l2l, P.p, P.L_far, P.L);
+    LENS_LAUNCHED("k_l2l_chain");
+    return;
+  }
   for (int l = 2; l < P.nlevels; ++l) {
     const int64_t a0 = P.active_level_off[l], a1 = P.active_level_off[l + 1];
     if (a1 <= a0) continue;

@@ -167,6 +167,7 @@ struct Plan {
   // expansions: (p+1) complex coefficients per box, scaled (see fmm.cu)
   double2* M = nullptr;
   double2* L = nullptr;
+  double2* L_far = nullptr;  // far-field parts by active index (small regions)
   int* p2m_list = nullptr;  // non-empty leaves sorted by star count (nb slots)
   int* p2m_bins = nullptr;  // 2 (leaf_size + 1): counts and offsets per star count
   FmmTables tab;
@@ -268,6 +269,8 @@ void fmm_tables(Plan& P, cudaStream_t s);
 // expansion buffers (M, L, P2M leaf order), allocated on the caller's stream
 // before the expansions are handed to the plan's own stream
 void fmm_alloc(Plan& P);
+// the far-field parts of a small region, allocated on the stream that forms them
+void fmm_alloc_far(Plan& P);
 void fmm_p2m(Plan& P, cudaStream_t s);
 void fmm_m2m(Plan& P, cudaStream_t s);
 void fmm_downward(Plan& P, cudaStream_t s);
