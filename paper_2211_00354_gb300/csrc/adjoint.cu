@@ -31,8 +31,8 @@ namespace {
 constexpr int kAdjTile = 128;  // rays per tile
 // float32-bulk plans: twice that once the rays give the chip several blocks an SM all
 // the same (a star's offsets and sums are formed once a tile).  P2P^T and moments at 3e6
-// rays on 16 leaves 384 + 72 us (tiles of 128: 420 + 91), at 5e5 rays 69 + 18 (73 + 15),
-// at 1.3e5 26 + 15 (24 + 10): the line is where the two meet.
+// rays on 16 leaves 384 + 72 us (tiles of 128: 420 + 91; plain sums), at 5e5 rays 69 + 18
+// (73 + 15), at 1.3e5 26 + 15 (24 + 10): the line is where the two meet.
 constexpr int kAdjTile32 = 256;
 constexpr int64_t kAdjLarge = 1 << 19;
 constexpr int kAdjU = 64;      // U-list leaves staged at a time by k_adj_p2p32
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
 // (each pair's difference exact to float32 rounding however close a ray is
 // to a star), partial sums compensated; L2P^T / M2P^T moments with the
 // scaled offsets w rounded once to float32 (|w| <= ~1.5: no cancellation),
-// summed per lane in float32 and across lanes compensated.  The transposed
+// summed per lane and across lanes compensated.  The transposed
 // translations (L2L^T, M2L^T, P2L^T, M2M^T, P2M^T) stay float64.
 
 // P2P^T: block per (leaf, tile of rays), four lanes a star over the U-list stars, each
@@ -313,10 +313,27 @@ __global__ void __launch_bounds__(128) k_adj_p2p32(AdjArgs A) {
   });
 }
 
+// a b, each component's fused product fixed: the same bits wherever it is inlined
+__device__ __forceinline__ float2 cmul_fixed(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+
 // L2P^T and M2P^T moments in float32: one warp per (leaf, tile), as
-// k_adj_leaf_moments.
+// k_adj_leaf_moments.  A lane takes four rays at a time (a trip to shared memory per
+// order and four rays) and compensates every sum: the terms of a tile cancel, so
+// roundings of plain partial sums were most of the gradient's own spread
+// (3e6 rays, p 24: 72 us with plain sums, 113 so).
+constexpr int kMomRays = 4;
+// a + b + c + d, the sum's head and its errors
+__device__ __forceinline__ ff sum4(float a, float b, float c, float d) {
+  float s, t, e, f, g, r;
+  two_sum(a, b, s, e);
+  two_sum(c, d, t, f);
+  two_sum(s, t, r, g);
+  return ff{r, g + (e + f)};
+}
 __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
-  extern __shared__ float2 acc32[];  // [(p+1)][33]: lane partials, padded
+  extern __shared__ float4 acc32[];  // [(p+1)][33]: lane partials (x, y, and their errors), padded
   const int lane = threadIdx.x;
   const int2 kt = A.tile_leaf[blockIdx.x];
   if (kt.x < 0) return;
@@ -333,7 +350,7 @@ __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
   const double irB = box_ir(A, B);
   const int64_t nW = A.W_off[a + 1] - A.W_off[a];
   for (int64_t pass = 0; pass <= nW; ++pass) {
-    for (int l = 0; l <= p; ++l) acc32[l * 33 + lane] = make_float2(0.f, 0.f);
+    for (int l = 0; l <= p; ++l) acc32[l * 33 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
     int C = -1;
     double rC = 0;
     double2 cC = make_double2(0, 0);
@@ -342,37 +359,51 @@ __global__ void __launch_bounds__(32) k_adj_leaf_moments32(AdjArgs A) {
       rC = box_r(A, C);
       cC = box_c(A, C, rC);
     }
-    for (int64_t t = r0 + lane; t < r1; t += 32) {
-      const int64_t ridx = A.perm[A.ray_off[k] + t];
-      const float2 c = make_float2(-d2f(A.gy[2 * ridx]), -d2f(A.gy[2 * ridx + 1]));
-      float2 pw, w;
-      if (pass == 0) {
-        w = make_float2(d2f((A.rays[2 * ridx] - cB.x) * irB),
-                        d2f((A.rays[2 * ridx + 1] - cB.y) * irB));
-        pw = c;
-      } else {
-        const float2 inv = cinv(make_float2(d2f(A.rays[2 * ridx] - cC.x),
-                                            d2f(A.rays[2 * ridx + 1] - cC.y)));
-        w = make_float2(inv.x * (float)rC, inv.y * (float)rC);
-        pw = cmul(c, inv);
+    for (int64_t t = r0 + lane; t < r1; t += 32 * kMomRays) {
+      float2 pw[kMomRays], w[kMomRays];
+#pragma unroll
+      for (int q = 0; q < kMomRays; ++q) {
+        pw[q] = w[q] = make_float2(0.f, 0.f);
+        if (t + 32 * q >= r1) continue;
+        const int64_t ridx = A.perm[A.ray_off[k] + t + 32 * q];
+        const float2 c = make_float2(-d2f(A.gy[2 * ridx]), -d2f(A.gy[2 * ridx + 1]));
+        if (pass == 0) {
+          w[q] = make_float2(d2f((A.rays[2 * ridx] - cB.x) * irB),
+                             d2f((A.rays[2 * ridx + 1] - cB.y) * irB));
+          pw[q] = c;
+        } else {
+          const float2 inv = cinv(make_float2(d2f(A.rays[2 * ridx] - cC.x),
+                                              d2f(A.rays[2 * ridx + 1] - cC.y)));
+          w[q] = make_float2(inv.x * (float)rC, inv.y * (float)rC);
+          pw[q] = cmul(c, inv);
+        }
       }
       for (int l = 0; l <= p; ++l) {
-        acc32[l * 33 + lane] = acc32[l * 33 + lane] + pw;
-        pw = cmul(pw, w);
+        float4 a4 = acc32[l * 33 + lane];
+        const ff x = sum4(pw[0].x, pw[1].x, pw[2].x, pw[3].x), y = sum4(pw[0].y, pw[1].y, pw[2].y, pw[3].y);
+        float e1, e2;
+        two_sum(a4.x, x.hi, a4.x, e1);
+        two_sum(a4.y, y.hi, a4.y, e2);
+        a4.z += e1 + x.lo;
+        a4.w += e2 + y.lo;
+        acc32[l * 33 + lane] = a4;
+#pragma unroll
+        for (int q = 0; q < kMomRays; ++q) pw[q] = cmul_fixed(pw[q], w[q]);
       }
     }
     __syncwarp();
     double2* dst = pass == 0 ? A.Lh + (int64_t)B * (p + 1) : A.Mh + (int64_t)C * (p + 1);
     // lane l sums order l's 32 lane partials, compensated (~48 bits): in
     // float64 the additions and conversions were most of the kernel's time
-    // (3e6 rays, p 24: with the tile's box constants, 260 -> 91 us; tiles of 256,
-    // 72)
+    // (3e6 rays, p 24: with the tile's box constants, 260 -> 91 us)
     for (int l = lane; l <= p; l += 32) {
       fcomp vx{0.f, 0.f}, vy{0.f, 0.f};
       for (int q = 0; q < 32; ++q) {
-        const float2 vf = acc32[l * 33 + q];
+        const float4 vf = acc32[l * 33 + q];
         vx.add(vf.x);
         vy.add(vf.y);
+        vx.lo += vf.z;
+        vy.lo += vf.w;
       }
       const double2 v = make_double2(vx.value(), vy.value());
       if (v.x != 0.0 || v.y != 0.0) atomic_add2(dst + l, v);
@@ -626,7 +657,7 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
   A.Phi = Phi.as<double2>(); A.Psi = Psi.as<double2>();
   const unsigned tiles = (unsigned)RB.tiles_max;
   if (f32) {
-    const size_t smem = sizeof(float2) * (size_t)P1 * 33;
+    const size_t smem = sizeof(float4) * (size_t)P1 * 33;
     k_adj_leaf_moments32<<<tiles, 32, smem, s>>>(A);
     LENS_LAUNCHED("k_adj_leaf_moments32");
     k_adj_p2p32<<<tiles, 128, 0, s>>>(A);
