@@ -160,63 +160,111 @@ __global__ void k_p2m(const double2* __restrict__ spos, const double* __restrict
 //                                              additions only),
 // one REAL binomial matrix on four complex vectors instead of four complex
 // matrices: about a third of the float64 operations of the direct form.
-// w^k and conj(w)^k are exact, so the rounding is that of the direct form.
-// Thread (parent, k) forms the four H_r[k] = conj(w)^k G_r[k], then thread
-// (parent, l) sums row l: many short float64 chains instead of one long one
-// per parent, so the pipe is fed from many warps.  A level's parents are
-// walked through their children: the boxes of level l+1 are the groups of
-// four children of the level-l splits, so group g (boxes c0+4g .. c0+4g+3)
-// has one parent and no thread lands on a leaf.
-constexpr int kM2MThreads = 128;
+// w^k and conj(w)^k are exact, so the rounding is that of the direct form: 2^-ceil(k/2)
+// times one of the eight units 1, 1 +- i, ...  The powers of two go into the
+// binomials (a product's rounding does not depend on them); a unit costs one addition
+// a component for odd k and none for even k.  Thread (parent, k) forms the four
+// H_r[k] = unit conj(w)^k G_r[k]; then the components of rows l and p - l, p + 2 terms
+// together, are one thread's: lanes of a warp end at the same time, where a row a
+// thread left half of the triangle idle.  An SM takes a warp's float64 instruction
+// every 19 cycles, so their number is what it costs: 38 -> 24 a parent at p 16 (5.3e5
+// boxes 431 -> 310 us).  A level's parents are walked through their children:
+// the boxes of level l+1 are the groups of four children of the level-l splits, so
+// group g (boxes c0+4g .. c0+4g+3) has one parent and no thread lands on a leaf.
+constexpr int kM2MMaxThreads = 256;
 
-__global__ void __launch_bounds__(kM2MThreads)
-k_m2m(const int* __restrict__ parent, int64_t c0, int64_t ngroups, int p,
-      const double* __restrict__ binom, int ldb, const double2* __restrict__ wpow,
-      double2* __restrict__ M) {
+__device__ __forceinline__ double flip(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? 0x80000000 : 0), __double2loint(x));
+}
+// component c (0 real, 1 imaginary) of z times the unit of (1 + i)^k (k mod 8: 1, 1+i, i,
+// -1+i, -1, -1-i, -i, 1-i), mine = z's component c, other = its other one
+__device__ __forceinline__ double unit_component(int k, int c, double mine, double other) {
+  // odd k: x - y and x + y up to signs; even k: x and y
+  const int q = (k >> 1) & 3;  // quarter turns
+  // i^q times v: component c is +-v of component c ^ (q & 1)
+  double v0 = mine, v1 = other;  // components c and 1 - c of z (1 + i)^(k & 1)
+  if (k & 1) {
+    // (1+i)(x + iy) = (x - y) + i (x + y)
+    const double sum = mine + other, dif = c ? other - mine : mine - other;  // x + y, x - y
+    v0 = c ? sum : dif;
+    v1 = c ? dif : sum;
+  }
+  // q = 1: (x, y) -> (-y, x); 2: (-x, -y); 3: (y, -x)
+  const double r = (q & 1) ? v1 : v0;
+  return flip(r, c ? q >= 2 : (q == 1 || q == 2));
+}
+
+// parents: per a block, their threads rounded up to whole warps
+__global__ void __launch_bounds__(kM2MMaxThreads)
+k_m2m(const int* __restrict__ parent, int64_t c0, int64_t ngroups, int p, int per,
+      const double* __restrict__ binom, int ldb, double2* __restrict__ M) {
   extern __shared__ double2 H[];  // [parents per block][4][p+1], then the binomials
-  const int P1 = p + 1;
-  const int per = kM2MThreads / P1;  // parents per block (>= 1 for p <= 64)
-  const int t = threadIdx.x, pb = t / P1, k = t - pb * P1;
+  const int P1 = p + 1, T = blockDim.x, t = threadIdx.x;
   // rows 0..p of the binomial table, triangular (row l from l (l+1) / 2), in
   // shared memory: the row sums below then wait on no global load (a small
-  // level has too few blocks to keep the table in L1)
+  // level has too few blocks to keep the table in L1); times 2^-(ceil(l/2) + ceil(k/2))
   double* cb_tab = reinterpret_cast<double*>(H + (int64_t)per * 4 * P1);
-  for (int i = t; i < P1 * (P1 + 1) / 2; i += kM2MThreads) {
+  for (int i = t; i < P1 * (P1 + 1) / 2; i += T) {
     // i = l (l+1)/2 + kk, 0 <= kk <= l
     int l = (int)((sqrtf(8.f * (float)i + 1.f) - 1.f) * 0.5f);
     while (l * (l + 1) / 2 > i) --l;
     while ((l + 1) * (l + 2) / 2 <= i) ++l;
-    cb_tab[i] = binom[(int64_t)l * ldb + (i - l * (l + 1) / 2)];
+    const int kk = i - l * (l + 1) / 2;
+    cb_tab[i] = mul_pow2(binom[(int64_t)l * ldb + kk], -((l + 1) / 2 + (kk + 1) / 2));
   }
-  const int64_t g = (int64_t)blockIdx.x * per + pb;
-  const bool on = pb < per && g < ngroups;
-  const int64_t c = c0 + 4 * g;     // first child of the group
-  const int64_t b = on ? parent[c] : 0;
-  double2* Hp = H + (int64_t)pb * 4 * P1;
-  if (on) {
-    const double2* A = M + c * P1;  // children c .. c+3 are contiguous
+  const int64_t g0 = (int64_t)blockIdx.x * per;
+  const int ng = (int)min64(per, ngroups - g0);  // parents of this block
+  for (int i = t; i < ng * P1; i += T) {
+    const int pb = i / P1, k = i - pb * P1;
+    const double2* A = M + (c0 + 4 * (g0 + pb)) * P1;  // four children, contiguous
     const double2 B0 = ld2(A + 3 * P1 + k), B1 = ld2(A + 2 * P1 + k);
     const double2 B2 = ld2(A + k), B3 = ld2(A + P1 + k);
     const double2 s02 = B0 + B2, d02 = B0 - B2, s13 = B1 + B3, d13 = B1 - B3;
-    double2 w = ld2(wpow + k);
-    w.y = -w.y;
-    Hp[0 * P1 + k] = cmul(w, s02 + s13);
-    Hp[1 * P1 + k] = cmul(w, make_double2(d02.x - d13.y, d02.y + d13.x));
-    Hp[2 * P1 + k] = cmul(w, s02 - s13);
-    Hp[3 * P1 + k] = cmul(w, make_double2(d02.x + d13.y, d02.y - d13.x));
+    const double2 X[4] = {s02 + s13, make_double2(d02.x - d13.y, d02.y + d13.x), s02 - s13,
+                          make_double2(d02.x + d13.y, d02.y - d13.x)};
+    double2* h = H + (int64_t)pb * 4 * P1 + k;
+    const int kc = (8 - (k & 7)) & 7;  // conj: the unit of (1 - i)^k is that of (1 + i)^(8 - k)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      // (1 - i)^k has the parity of k; one addition a component for odd k
+      h[r * P1] = make_double2(unit_component(kc, 0, X[r].x, X[r].y), unit_component(kc, 1, X[r].y, X[r].x));
+    }
   }
   __syncthreads();
-  if (on) {
-    const int l = k;
-    double sx = 0.0, sy = 0.0;
-    const double* crow = cb_tab + l * (l + 1) / 2;
-    for (int kk = 0; kk <= l; ++kk) {
-      const double cb = crow[kk];
-      const double2 h = Hp[((l - kk) & 3) * P1 + kk];
-      sx = fma(cb, h.x, sx);
-      sy = fma(cb, h.y, sy);
+  const int nt = 2 * ((P1 + 1) / 2);  // threads a parent: pairs of rows times two components
+  for (int i0 = 0; i0 < per * nt; i0 += T) {
+    const int i = i0 + t, pb = i / nt, j = i - pb * nt, c = j & 1;
+    const bool on = pb < ng && i < per * nt;
+    const int la = j >> 1, lb = p - la;  // la <= lb
+    double va = 0.0, vb = 0.0;
+    if (on) {
+      const double* h = reinterpret_cast<const double*>(H + (int64_t)pb * 4 * P1) + c;
+      // one loop over both rows, so that the lanes' loops are of one length
+      const double* cr = cb_tab + la * (la + 1) / 2;
+      const int steps = lb != la ? p + 2 : la + 1;
+      int l = la, k = 0;
+      double acc = 0.0;
+      for (int q = 0; q < steps; ++q) {
+        acc = fma(cr[k], h[2 * (((l - k) & 3) * P1 + k)], acc);
+        ++k;
+        if (q == la) {
+          va = acc;
+          acc = 0.0;
+          l = lb;
+          cr = cb_tab + lb * (lb + 1) / 2;
+          k = 0;
+        }
+      }
+      vb = acc;
     }
-    M[b * (int64_t)P1 + l] = cmul(ld2(wpow + l), make_double2(sx, sy));
+    // the other component is the neighbouring lane's (T and nt are even)
+    const double oa = __shfl_xor_sync(0xffffffffu, va, 1), ob = __shfl_xor_sync(0xffffffffu, vb, 1);
+    if (on) {
+      const int64_t b = parent[c0 + 4 * (g0 + pb)];
+      double* out = reinterpret_cast<double*>(M + b * P1) + c;
+      out[2 * la] = unit_component(la, c, va, oa);
+      if (lb != la) out[2 * lb] = unit_component(lb, c, vb, ob);
+    }
   }
 }
 
@@ -408,6 +456,24 @@ __global__ void __launch_bounds__(NW == 1 ? 32 * kWarpsPerBlock : 32 * NW) k_far
   }
 }
 
+// Component c of sum_{l >= j} S[j][l] z_l, row and z from l = j on, n terms, in order,
+// each by cfma's products (-z.y or z.x with the imaginary part of S, then z.x or z.y with
+// the real one).  S goes with the (l - j)-th power of (+-1 +- i) / 2: its imaginary part is
+// 0 for l - j = 0 mod 4 and its real part for l - j = 2 mod 4, and a product with 0 is
+// left out (1.1e5 boxes of p 12 303 -> 277 us).
+__device__ __forceinline__ double l2l_component(const double2* __restrict__ S, const double2* z, int n, int c) {
+  double v = 0.0;
+  const auto re = [&](int t) { return c ? z[t].y : z[t].x; };
+  const auto im = [&](int t) { return c ? z[t].x : flip(z[t].y, true); };
+  for (int t = 0; t < n; t += 4) {
+    v = fma(ld2(S + t).x, re(t), v);
+    if (t + 1 < n) { const double2 s = ld2(S + t + 1); v = fma(s.x, re(t + 1), fma(s.y, im(t + 1), v)); }
+    if (t + 2 < n) v = fma(ld2(S + t + 2).y, im(t + 2), v);
+    if (t + 3 < n) { const double2 s = ld2(S + t + 3); v = fma(s.x, re(t + 3), fma(s.y, im(t + 3), v)); }
+  }
+  return v;
+}
+
 // L2L of the active boxes of one level (>= 2; above it the parent's local
 // expansion is zero), one thread per component of a (box, coefficient j):
 //   L_B[j] += sum_{l >= j} S_q[j][l] L_parent[l],  q = the box's quadrant.
@@ -428,16 +494,7 @@ k_l2l(const int* __restrict__ active, int64_t a0, int64_t a1,
   const int B = active[a];
   const int par = parent[B];
   const int q = B - child[par];
-  const double2* Lp = L + (int64_t)par * P1;
-  const double2* S = l2l + ((int64_t)q * P1 + j) * P1;
-  // component c of the sum, by cfma's products in its order: -z.y or z.x with the
-  // imaginary part of S, then z.x or z.y with the real one
-  double v = 0.0;
-  for (int l = j; l <= p; ++l) {
-    const double2 s2 = ld2(S + l), z = ld2(Lp + l);
-    const double w = c ? z.x : __hiloint2double(__double2hiint(z.y) ^ 0x80000000, __double2loint(z.y));
-    v = fma(s2.x, c ? z.y : z.x, fma(s2.y, w, v));
-  }
+  const double v = l2l_component(l2l + ((int64_t)q * P1 + j) * P1 + j, L + (int64_t)par * P1 + j, P1 - j, c);
   double* o = reinterpret_cast<double*>(L + (int64_t)B * P1 + j) + c;
   *o = *o + v;
 }
@@ -476,15 +533,7 @@ __global__ void k_l2l_chain(const int* __restrict__ active, const int* __restric
     ++l;
     if (on) {
       const int s = lv - l, q = ((bx >> s) & 1) | (((by >> s) & 1) << 1);
-      const double2* S = l2l + ((int64_t)q * P1 + j) * P1;
-      double v = 0.0;
-#pragma unroll 4
-      for (int k = j; k <= p; ++k) {
-        const double2 s2 = ld2(S + k), z = now[k];
-        const double w = c ? z.x : __hiloint2double(__double2hiint(z.y) ^ 0x80000000, __double2loint(z.y));
-        v = fma(s2.x, c ? z.y : z.x, fma(s2.y, w, v));
-      }
-      x = next + v;
+      x = next + l2l_component(l2l + ((int64_t)q * P1 + j) * P1 + j, now + j, P1 - j, c);
     }
   }
   if (on) reinterpret_cast<double*>(L + (int64_t)B * P1)[i] = x;
@@ -640,14 +689,21 @@ void fmm_p2m(Plan& P, cudaStream_t s) {
 void fmm_m2m(Plan& P, cudaStream_t s) {
   const FmmTables& t = P.tab;
   const int P1 = P.p + 1;
-  const int per = kM2MThreads / P1;
+  // parents a block: the fewest that fill whole warps best
+  const int nt = 2 * ((P1 + 1) / 2);
+  int per = 1, threads = (nt + 31) / 32 * 32;
+  for (int q = 2; q * nt <= kM2MMaxThreads; ++q) {
+    const int th = (q * nt + 31) / 32 * 32;
+    if (th <= kM2MMaxThreads && (int64_t)q * threads > (int64_t)per * th) { per = q; threads = th; }
+  }
   const size_t smem = sizeof(double2) * 4 * (size_t)P1 * per + sizeof(double) * P1 * (P1 + 1) / 2;
+  if (smem > 48 * 1024)
+    LENS_CUDA(cudaFuncSetAttribute(k_m2m, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   for (int l = P.nlevels - 2; l >= 0; --l) {
     // level l+1 holds the children of the level-l splits, four per split
     const int64_t c0 = P.level_off[l + 1], ng = (P.level_off[l + 2] - c0) / 4;
     if (ng <= 0) continue;
-    k_m2m<<<grid_for(ng, per), kM2MThreads, smem, s>>>(P.box_parent, c0, ng, P.p, t.binom,
-                                                       t.ldb, t.wpow, P.M);
+    k_m2m<<<grid_for(ng, per), threads, smem, s>>>(P.box_parent, c0, ng, P.p, per, t.binom, t.ldb, P.M);
     LENS_LAUNCHED("k_m2m");
   }
 }
