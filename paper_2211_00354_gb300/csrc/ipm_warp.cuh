@@ -392,6 +392,149 @@ __device__ __noinline__ void ext_cell_call(const IpmArgs& A, const PixCorner* q4
   ext_cell_body<false>(A, q, cut_x, cut_y, lane, led);
 }
 
+// Ill-conditioned cells, those of boxes up to kExtPixels, a lane a cell: the area,
+// slopes and their divisions once per cell, its pixels spread over the lanes as in
+// ext_cell, the cut ones taken 32 at a time from whichever cells.  (By the whole warp, a
+// cell's ~400 operations of preparation ran on all lanes alike and its few pixels
+// left two thirds of them idle.)
+constexpr int kExtPixels = 4096, kExtSide = 255;  // (a side fits 8 bits)
+
+struct ExtCells {
+  ff u[4][32], v[4][32], sl[4][32];  // corners local to the box, slopes
+  float2 inv[32];                    // 1 / A_P, high and low
+  int4 box[32];                      // ix0, iy0, cx0, cy0
+  int wd[32];                        // width of the clipped box
+  int who[32], cut[64];
+};
+// sum of the fractions put into the map (they cancel in folded cells) and cells counted
+struct ExtSum {
+  fcomp fin{0.f, 0.f};
+  int cells = 0;
+};
+
+// lane: its cell's corners where it has one; true for a cell left to ext_cell
+__device__ __forceinline__ bool ext_round(const IpmArgs& A, ExtCells& sh, int lane, bool has,
+                                          const PixCorner (&q4)[4], Ledger& led, ExtSum& sum) {
+  const int npx = A.ip.npx;
+  int npix = 0;
+  bool large = false;
+  if (has) {
+    const int ix0 = min4(q4[0].iu, q4[1].iu, q4[2].iu, q4[3].iu);
+    const int ix1 = max4(q4[0].iu, q4[1].iu, q4[2].iu, q4[3].iu);
+    const int iy0 = min4(q4[0].iv, q4[1].iv, q4[2].iv, q4[3].iv);
+    const int iy1 = max4(q4[0].iv, q4[1].iv, q4[2].iv, q4[3].iv);
+    const int cx0 = max(ix0, 0), cx1 = min(ix1, npx - 1);
+    const int cy0 = max(iy0, 0), cy1 = min(iy1, A.ip.npy - 1);
+    const int wd = cx1 - cx0 + 1, ht = cy1 - cy0 + 1;
+    large = wd > kExtSide || ht > kExtSide || wd * ht > kExtPixels;
+    if (!large) {
+      ff u[4], v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // integer part (< 2^24 in the box) + fraction: exact as a two-sum
+        two_sum((float)(q4[k].iu - ix0), q4[k].fu, u[k].hi, u[k].lo);
+        two_sum((float)(q4[k].iv - iy0), q4[k].fv, v[k].hi, v[k].lo);
+      }
+      const ff A_P = ff_half(ff_sub(ff_mul(ff_sub(u[2], u[0]), ff_sub(v[3], v[1])),
+                                    ff_mul(ff_sub(u[3], u[1]), ff_sub(v[2], v[0]))));
+      if (!(fabsf(A_P.hi) > A.thr_degen)) {
+        led.ndeg += 1;
+      } else {
+        led.nff += 1;
+        sum.cells += 1;
+        npix = wd * ht;
+        const ff inv = ff_div(ff{1.f, 0.f}, A_P);
+        sh.inv[lane] = make_float2(inv.hi, inv.lo);
+        sh.box[lane] = make_int4(ix0, iy0, cx0, cy0);
+        sh.wd[lane] = wd;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const ff ey = ff_sub(v[(k + 1) & 3], v[k]);
+          sh.sl[k][lane] = ey.hi != 0.f ? ff_div(ff_sub(u[(k + 1) & 3], u[k]), ey) : ff{0.f, 0.f};
+          sh.u[k][lane] = u[k];
+          sh.v[k][lane] = v[k];
+        }
+      }
+    }
+  }
+  WarpTasks T;
+  T.begin(npix, sh.who, lane);
+  int ncut = 0;  // warp-uniform: entries waiting in sh.cut
+  for (int f0 = 0; f0 < T.total; f0 += 32) {
+    int off;
+    const int L = T.owner(f0, sh.who, lane, off);
+    bool cut = false;
+    int code = 0;
+    if (f0 + lane < T.total) {
+      const int4 bx = sh.box[L];
+      const int wd = sh.wd[L], r = off / wd, c = off - r * wd;
+      const int ox = bx.z - bx.x + c, oy = bx.w - bx.y + r;
+      float fx[4], fy[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { fx[k] = sh.u[k][L].hi; fy[k] = sh.v[k][L].hi; }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        cut |= seg_meets_pixel(fx[e], fy[e], fx[(e + 1) & 3], fy[(e + 1) & 3], (float)ox, (float)oy);
+      code = L << 16 | r << 8 | c;  // r, c < kExtSide
+      if (!cut) {
+        const int wn = winding4(fx, fy, (float)ox + 0.5f, (float)oy + 0.5f);
+        const float fr = (float)wn * sh.inv[L].x;
+        if (fr != 0.0f) {
+          atomicAdd(&A.map[(int64_t)(bx.w + r) * npx + bx.z + c], A.scale_f * fr);
+          sum.fin.add(fr);
+          led.nupd += 1;
+        }
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, cut);
+    if (cut) sh.cut[ncut + __popc(m & ((1u << lane) - 1u))] = code;  // < 64: ncut < 32 here
+    ncut += __popc(m);
+    const bool last = f0 + 32 >= T.total;
+    while (ncut >= 32 || (last && ncut > 0)) {
+      __syncwarp();
+      const int take = min(ncut, 32), rest = ncut - take;
+      if (lane < take) {
+        const int e = sh.cut[lane], C = e >> 16, r = (e >> 8) & 0xff, c = e & 0xff;
+        const int4 bx = sh.box[C];
+        ff u[4], v[4], sl[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { u[k] = sh.u[k][C]; v[k] = sh.v[k][C]; sl[k] = sh.sl[k][C]; }
+        const float2 iv = sh.inv[C];
+        const float fr =
+            ff_mul(pixel_area_ff(u, v, sl, bx.z - bx.x + c, bx.w - bx.y + r), ff{iv.x, iv.y}).hi;
+        if (fr != 0.0f) {
+          atomicAdd(&A.map[(int64_t)(bx.w + r) * npx + bx.z + c], A.scale_f * fr);
+          sum.fin.add(fr);
+          led.nupd += 1;
+        }
+      }
+      // move the rest (at most 31) to the front
+      const int k = lane < rest ? sh.cut[take + lane] : 0;
+      __syncwarp();
+      if (lane < rest) sh.cut[lane] = k;
+      ncut = rest;
+    }
+    __syncwarp();
+  }
+  __syncwarp();  // the cells' staging is read before the next round's
+  return large;
+}
+// the sums of the warp into the ledger
+__device__ __forceinline__ void ext_close(const ExtSum& sum, int lane, Ledger& led) {
+  ff f;
+  two_sum(sum.fin.hi, sum.fin.lo, f.hi, f.lo);
+  int n = sum.cells;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    f = ff_add(f, ff{__shfl_xor_sync(0xffffffffu, f.hi, o), __shfl_xor_sync(0xffffffffu, f.lo, o)});
+    n += __shfl_xor_sync(0xffffffffu, n, o);
+  }
+  if (lane == 0) {
+    led.fin += f.hi;
+    led.fout += ff_add(ff{(float)n, 0.f}, ff_neg(f)).hi;
+  }
+}
+
 // One round of 32 cells (lane = cell; `has`: the lane holds a cell, `c` its
 // id for the queues, q4 its corners c00, c10, c11, c01 in pixel coordinates):
 //  A. lane = cell: pixel box, ledger of cells that are dropped or outside,
