@@ -37,6 +37,12 @@ constexpr int kIpmThreads = 256;
 // warps (308 us of a 200^2-pixel window's map) and the 7.8e3 chunks of a 500^2
 // grid to 976.
 constexpr int kMaxGrab = 8;
+// Cells per chunk: 32, fewer (down to kMinLanes lanes with a cell) while that leaves fewer
+// than kChunksPerWarp chunks for a resident warp.  Most of a round's work is pixels and rows,
+// spread over all lanes whoever holds the cells, so short rounds cost little and a
+// refinement level or a small grid reaches all the warps: 2.9e4 sub-cells of a window map
+// 79 -> 29 us (2 chunks a warp the same, 4: a 500^2 grid 35 -> 46 us).
+constexpr int kMinLanes = 4, kChunksPerWarp = 1;
 constexpr int kBlocksPerSm = 4;
 
 constexpr int kWarps = kIpmThreads / 32;
@@ -55,10 +61,11 @@ template <bool QUADS, bool LIST = false>
 __global__ void __launch_bounds__(kIpmThreads, kBlocksPerSm) k_ipm_cells(IpmArgs A) {
   __shared__ WarpCells sh[kWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t nchunks = (A.ncells + 31) >> 5;
+  const int lanes = A.lanes;
+  const int64_t nchunks = (A.ncells + lanes - 1) / lanes;
   const int64_t W = A.nx + 1;
   Ledger led;
-  // Chunks of 32 cells are handed out by a counter (qcount[1]), so the
+  // Chunks of A.lanes cells are handed out by a counter (qcount[1]), so the
   // warps of a block finish together however the large cells fall; one
   // fetch takes A.grab chunks.
   unsigned* next = reinterpret_cast<unsigned*>(A.qcount) + 1;
@@ -69,8 +76,8 @@ __global__ void __launch_bounds__(kIpmThreads, kBlocksPerSm) k_ipm_cells(IpmArgs
   for (int64_t ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * grab; ch < nchunks;) {
     // the following grab is fetched while this one is processed
     if (lane == 0 && left == grab) g_u = atomicAdd(next, 1u);
-    const int64_t idx = ch * 32 + lane;
-    const bool has = idx < A.ncells;
+    const int64_t idx = ch * lanes + lane;
+    const bool has = lane < lanes && idx < A.ncells;
     int64_t c = idx;
     PixCorner q4[4];
     if (has) {
@@ -180,14 +187,17 @@ void ipm_launch(IpmArgs& A, bool quads, int* qcount, cudaStream_t s,
   int dev = 0, sms = 152;
   LENS_CUDA(cudaGetDevice(&dev));
   LENS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t chunk_blocks = (A.ncells + kIpmThreads - 1) / kIpmThreads;
+  A.lanes = 32;
+  const int64_t warps = (int64_t)sms * kBlocksPerSm * kWarps;
+  while (A.lanes > kMinLanes && A.ncells / A.lanes < kChunksPerWarp * warps) A.lanes /= 2;
+  const int64_t chunk_blocks = (A.ncells + A.lanes * kWarps - 1) / (A.lanes * kWarps);
   const unsigned g = (unsigned)std::min<int64_t>(chunk_blocks, (int64_t)sms * 8);
   int L = 0;
   while ((1ll << L) < A.nx) ++L;
   A.div_s = 30 + L;
   A.div_m = A.nx > 0 ? (uint32_t)((1ull << A.div_s) / (uint64_t)A.nx + 1) : 0;
   A.grab = (int)std::max<int64_t>(
-      1, std::min<int64_t>(kMaxGrab, (A.ncells >> 5) / ((int64_t)sms * kBlocksPerSm * kWarps * 8)));
+      1, std::min<int64_t>(kMaxGrab, A.ncells / A.lanes / (warps * 8)));
   if (quads) k_ipm_cells<true><<<g, kIpmThreads, 0, s>>>(A);
   else if (A.cell_list) k_ipm_cells<false, true><<<g, kIpmThreads, 0, s>>>(A);
   else k_ipm_cells<false><<<g, kIpmThreads, 0, s>>>(A);
