@@ -55,7 +55,7 @@ __device__ __forceinline__ int64_t cell_row(const IpmArgs& A, uint32_t c) {
   return (int64_t)(((uint64_t)c * A.div_m) >> A.div_s);
 }
 
-// One warp per round of 32 cells of a grid chunk (or of a cell list, or of
+// One warp per round of up to 32 cells of a grid chunk (or of a cell list, or of
 // sub-cells given as four corners each), rounds handed out by a counter.
 template <bool QUADS, bool LIST = false>
 __global__ void __launch_bounds__(kIpmThreads, kBlocksPerSm) k_ipm_cells(IpmArgs A) {
