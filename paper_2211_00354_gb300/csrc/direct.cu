@@ -89,10 +89,13 @@ k_direct_f32(const float4* __restrict__ shl, const float* __restrict__ sm, int64
     int64_t r = base + threadIdx.x + (int64_t)k * kThreads;
     if (r >= m) continue;
     const double x1 = rays[2 * r], x2 = rays[2 * r + 1];
-    y[2 * r] = fma(a, x1, -ax[k].value());
-    y[2 * r + 1] = fma(b, x2, -ay[k].value());
+    // plain conversions: once a ray they cost nothing, and branches here keep the
+    // compiler from unrolling the loop over the stars (2e4 x 2e4 pairs 1.14 -> 1.92 ms)
+    const auto value = [](const fcomp& c) { return (double)c.hi + (double)c.lo; };
+    y[2 * r] = fma(a, x1, -value(ax[k]));
+    y[2 * r + 1] = fma(b, x2, -value(ay[k]));
     if (JAC) {
-      const double d11 = j11[k].value(), d12 = j12[k].value();
+      const double d11 = value(j11[k]), d12 = value(j12[k]);
       jac[4 * r + 0] = a - d11;
       jac[4 * r + 1] = -d12;
       jac[4 * r + 2] = -d12;
