@@ -316,6 +316,10 @@ __global__ void k_track(const double* __restrict__ map, int npx, int npy, double
 // (401 x 333 pixels, R = 240: 9168 us against 306).
 constexpr size_t kRingBytes = (size_t)384 << 20, kRingMax = (size_t)512 << 20;
 constexpr int kRingMinRows = 32;  // output rows a launch
+// a few terms a pixel of a small map are less than a second launch: one pass there (64^2
+// px, R 1: 35 us against 38; R 12: 50 against 43; 1000^2 px, R 1: 76 against 56)
+constexpr int kOnePassR = 4;
+constexpr int64_t kOnePassPixels = 1 << 16;
 constexpr int kTwoPassMaxR = 256;  // (R + 1)^2 in-map weights are formed on the host
 
 bool source_two_pass(const double* map, RowPass A, double dfull, double* out, DeviceAlloc& da,
@@ -391,7 +395,7 @@ void map_source(const double* map, int npx, int npy, double sigma_px, double tru
   const int steps = (R + kRowStep - 1) / kRowStep * kRowStep + 1;
   // one host block: g, G, r(dy) (float64 slots), then the float-float tables of
   // the two-pass form on a 16-byte boundary, its ints and its in-map weights
-  const bool two = R <= kTwoPassMaxR;
+  const bool two = R <= kTwoPassMaxR && (R > kOnePassR || (int64_t)npx * npy > kOnePassPixels);
   const size_t nf = (3 * n1 + 1) / 2 * 2, ni = (size_t)steps + n1;
   const size_t nq0 = nf + 2 * (size_t)steps + (ni + 1) / 2;
   std::vector<double> tab(nq0 + (two ? n1 * n1 : 0), 0.0);
