@@ -175,7 +175,8 @@ lens_status lens_fmm_build(const double* stars_xy, const double* masses,
  * grid): L2P + P2P (+ M2P for the adaptive W lists), then y.
  *   rays_xy: dev m x 2; y_out: dev m x 2; jac_out: dev m x 4 (row-major
  *   dy/dx) or NULL.  Rays must lie in the plan's target region (EDOMAIN
- *   otherwise; reported after a stream synchronisation).  m = 0 is a no-op. */
+ *   otherwise; reported after a stream synchronisation, the outputs not
+ *   written).  m = 0 is a no-op. */
 lens_status lens_deflect(lens_plan* plan, const double* rays_xy, int64_t m,
                          double* y_out, double* jac_out, void* stream);
 
@@ -188,7 +189,7 @@ lens_status lens_deflect(lens_plan* plan, const double* rays_xy, int64_t m,
  * float64 throughout whatever the plan's precision (a float32-bulk plan's
  * multipoles carry float32 P2M sums).  A star exactly at a ray contributes
  * nothing.  psi_out: dev m.  Synchronises `stream`.  LENS_EDOMAIN for a
- * ray outside the target region or not finite. */
+ * ray outside the target region or not finite (psi_out not written). */
 lens_status lens_potential(lens_plan* plan, const double* rays_xy, int64_t m,
                            double* psi_out, void* stream);
 
@@ -324,7 +325,9 @@ lens_status lens_ipm_map_ex(lens_plan* plan, const lens_grid* grid,
  *   grad_xy: dev n x 2 = dL/dx_i (caller's star order),
  *   grad_m:  dev n     = dL/dm_i,
  *   grad_kg: dev 2     = dL/dkappa_s, dL/dgamma.
- * Any output pointer may be NULL. */
+ * Any output pointer may be NULL.  EDOMAIN for a ray outside the target region
+ * or not finite: reported after a stream synchronisation, grad_xy and grad_m
+ * not written, grad_kg zero. */
 lens_status lens_deflect_adjoint(lens_plan* plan, const double* rays_xy,
                                  int64_t m, const double* grad_y,
                                  double* grad_xy, double* grad_m,

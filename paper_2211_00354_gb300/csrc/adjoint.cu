@@ -590,7 +590,9 @@ __global__ void __launch_bounds__(128) k_adj_p2m(AdjArgs A, int64_t nb) {
   }
 }
 
-__global__ void k_adj_kg(const double* rays, const double* gy, int64_t m, double* gkg) {
+__global__ void k_adj_kg(const double* rays, const double* gy, int64_t m, const int64_t* bad,
+                         double* gkg) {
+  if (*bad) return;  // the call is refused
   __shared__ double sh[2][256];
   double sk = 0, sg = 0;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < m;
@@ -609,9 +611,9 @@ __global__ void k_adj_kg(const double* rays, const double* gy, int64_t m, double
 }
 
 __global__ void k_adj_out(const double2* Phi, const double2* Psi, const uint32_t* sidx, int64_t n,
-                          double* gxy, double* gm) {
+                          const int64_t* bad, double* gxy, double* gm) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || *bad) return;
   const int64_t j = sidx[i];
   if (gm) gm[j] = Phi[i].x;
   if (gxy) { gxy[2 * j] = Psi[i].x; gxy[2 * j + 1] = -Psi[i].y; }
@@ -633,7 +635,7 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
   const bool f32 = P.prec == LENS_FP32_BULK;
   const int tile = f32 && m >= kAdjLarge ? kAdjTile32 : kAdjTile;
   bucket_rays(P, rays, m, tile, RB, s);
-  Scratch tl = tile_leaves(P, RB.toff, P.n_active_leaves, RB.tiles_max, s);
+  Scratch tl = tile_leaves(P, RB.toff, P.n_active_leaves, RB.tiles_max, s, RB.bad);
   Scratch Lh(&P.da, sizeof(double2) * (size_t)P.nb * P1);
   Scratch Mh(&P.da, sizeof(double2) * (size_t)P.nb * P1);
   Scratch Phi(&P.da, sizeof(double2) * (size_t)P.n), Psi(&P.da, sizeof(double2) * (size_t)P.n);
@@ -697,15 +699,15 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
   else k_adj_p2m<32><<<grid_for(P.nb * 32, 128), 128, 0, s>>>(A, P.nb);
   LENS_LAUNCHED("k_adj_p2m");
   if (gkg) {
-    k_adj_kg<<<grid_for(m, 256, 1024), 256, 0, s>>>(rays, gy, m, gkg);
+    k_adj_kg<<<grid_for(m, 256, 1024), 256, 0, s>>>(rays, gy, m, RB.bad, gkg);
     LENS_LAUNCHED("k_adj_kg");
   }
   if (gxy || gm) {
     k_adj_out<<<grid_for(P.n, 256), 256, 0, s>>>(Phi.as<double2>(), Psi.as<double2>(), P.sidx, P.n,
-                                                 gxy, gm);
+                                                 RB.bad, gxy, gm);
     LENS_LAUNCHED("k_adj_out");
   }
-  check_rays(RB);
+  check_rays(RB, s);
 }
 
 }  // namespace lens

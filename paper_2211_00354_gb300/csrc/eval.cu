@@ -364,7 +364,8 @@ constexpr int kBucketThreads = 256;
 __global__ void __launch_bounds__(kBucketThreads)
 k_ray_leaf(const double* __restrict__ rays, int64_t m, const int* __restrict__ child,
            const int* __restrict__ lidx, double lo_x, double lo_y, double scale, int depth,
-           int* __restrict__ slot, int64_t* __restrict__ counts, int64_t* __restrict__ err) {
+           int* __restrict__ slot, int64_t* __restrict__ counts, int64_t* __restrict__ bad,
+           int64_t* __restrict__ err) {
   __shared__ int s_lead;
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   int li = -1;
@@ -384,7 +385,8 @@ k_ray_leaf(const double* __restrict__ rays, int64_t m, const int* __restrict__ c
     }
     if (li < 0) {
       li = -1;
-      *err = 1;  // host memory: a plain store, whoever comes first
+      *bad = 1;  // plain stores, whoever comes first; err is host memory
+      *err = 1;
     }
     slot[r] = li;
   }
@@ -494,10 +496,10 @@ k_ray_offsets(const int64_t* __restrict__ cnt, int64_t n, int tile, int64_t* __r
 // bisection with toff[lo] <= t < toff[hi] held throughout; a leaf of no
 // tiles shares its offset with the next and is passed over.
 __global__ void k_tile_leaf(const int64_t* __restrict__ toff, int64_t nl, int64_t total,
-                            int2* __restrict__ out) {
+                            const int64_t* __restrict__ bad, int2* __restrict__ out) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= total) return;
-  if (t >= toff[nl]) { out[t] = make_int2(-1, 0); return; }
+  if (t >= toff[nl] || (bad && *bad)) { out[t] = make_int2(-1, 0); return; }
   int64_t lo = 0, hi = nl;
   while (hi - lo > 1) {
     const int64_t mid = (lo + hi) >> 1;
@@ -508,10 +510,11 @@ __global__ void k_tile_leaf(const int64_t* __restrict__ toff, int64_t nl, int64_
 
 }  // namespace
 
-Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s) {
+Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s,
+                    const int64_t* bad) {
   if (total > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
   Scratch tl(&P.da, sizeof(int2) * (size_t)std::max<int64_t>(total, 1));
-  k_tile_leaf<<<grid_for(total, 256), 256, 0, s>>>(toff, nl, total, tl.as<int2>());
+  k_tile_leaf<<<grid_for(total, 256), 256, 0, s>>>(toff, nl, total, bad, tl.as<int2>());
   LENS_LAUNCHED("k_tile_leaf");
   return tl;
 }
@@ -649,23 +652,24 @@ void evaluate_grid_pix(Plan& P, const GridRows& g, PixCorner* out, const IpmPara
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s) {
   const int64_t nl = P.n_active_leaves;
   if (nl == 0) fail(LENS_EDOMAIN, "plan has no active leaves");
-  // counts and cursors (zeroed together), then the offsets
+  // counts, cursors and the flag (zeroed together), then the offsets
   const size_t n = (size_t)nl + 1;
-  B.mem = Scratch(&P.da, sizeof(int64_t) * 4 * n);
+  B.mem = Scratch(&P.da, sizeof(int64_t) * (4 * n + 1));
   B.slot = Scratch(&P.da, sizeof(int) * m);
   B.perm = Scratch(&P.da, sizeof(int) * m);
   int64_t* cnt = B.mem.as<int64_t>();
   int64_t* cur = cnt + n;
-  int64_t* off = cur + n;
+  int64_t* bad = cur + n;
+  int64_t* off = bad + 1;
   int64_t* toff = off + n;
   B.flag = host_slot();
   B.flag.host[0] = 0;
   LENS_CUDA(cudaEventCreateWithFlags(&B.leaves_known, cudaEventDisableTiming));
-  LENS_CUDA(cudaMemsetAsync(B.mem.p, 0, sizeof(int64_t) * 2 * n, s));
+  LENS_CUDA(cudaMemsetAsync(B.mem.p, 0, sizeof(int64_t) * (2 * n + 1), s));
   const double scale = (double)(1ull << P.depth) / P.root_size;
   k_ray_leaf<<<grid_for(m, kBucketThreads), kBucketThreads, 0, s>>>(rays, m, P.box_child, P.box_lidx, P.root_lo[0],
                                               P.root_lo[1], scale, P.depth, B.slot.as<int>(), cnt,
-                                              B.flag.dev);
+                                              bad, B.flag.dev);
   LENS_LAUNCHED("k_ray_leaf");
   LENS_CUDA(cudaEventRecord(B.leaves_known, s));
   if (nl <= kOneBlockLeaves) {
@@ -681,13 +685,17 @@ void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B
   LENS_LAUNCHED("k_ray_scatter");
   B.off = off;
   B.toff = toff;
+  B.bad = bad;
   B.tiles_max = m / tile + std::min(nl, m);
   if (B.tiles_max > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
 }
 
-void check_rays(const RayBuckets& B) {
+void check_rays(const RayBuckets& B, cudaStream_t s) {
   LENS_CUDA(cudaEventSynchronize(B.leaves_known));
-  if (B.flag.host[0]) fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
+  if (!B.flag.host[0]) return;
+  // what was launched returns at once; the caller may free its buffers on the error
+  LENS_CUDA(cudaStreamSynchronize(s));
+  fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
 }
 
 void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* jac, cudaStream_t s) {
@@ -696,7 +704,7 @@ void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* ja
   const int rpt = f64 ? kRptD : eval32_rays_per_thread(jac != nullptr);
   RayBuckets B;
   bucket_rays(P, rays, m, (f64 ? kEvalThreads : kEval32Threads) * rpt, B, s);
-  Scratch tl = tile_leaves(P, B.toff, P.n_active_leaves, B.tiles_max, s);
+  Scratch tl = tile_leaves(P, B.toff, P.n_active_leaves, B.tiles_max, s, B.bad);
   if (f64) {
     wait_expansions(P, s);
     EvalArgs A = base_args(P);
@@ -707,7 +715,7 @@ void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* ja
   } else {
     eval32_rays(P, rays, B.off, B.perm.as<int>(), tl.as<int2>(), B.tiles_max, y, jac, s);
   }
-  check_rays(B);
+  check_rays(B, s);
 }
 
 }  // namespace lens

@@ -289,11 +289,14 @@ void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* ja
 // is read back: a launch over tiles covers tiles_max and its blocks past
 // toff[nl] return, and check_rays(), called once the work is launched, waits until
 // every ray has its leaf (not for the work) and fails if one lies outside the
-// target region.
+// target region.  Then *bad is nonzero and the work does nothing: no tile has a
+// leaf, the kernels that write outputs without tiles look at it, and the call
+// fails with its stream idle and the outputs as they were.
 struct RayBuckets {
   Scratch mem, perm, slot;
   const int64_t* off = nullptr;
   const int64_t* toff = nullptr;
+  const int64_t* bad = nullptr;
   int64_t tiles_max = 0;
   HostSlot flag{};
   cudaEvent_t leaves_known = nullptr;  // every ray has its leaf (or raised the flag)
@@ -303,10 +306,12 @@ struct RayBuckets {
   ~RayBuckets() { if (leaves_known) cudaEventDestroy(leaves_known); }
 };
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s);
-void check_rays(const RayBuckets& B);
+void check_rays(const RayBuckets& B, cudaStream_t s);
 // (leaf, tile within the leaf) of each of `total` tiles (toff: exclusive scan of
-// the leaves' tile counts, toff[nl] their sum; a tile past it gets leaf -1)
-Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s);
+// the leaves' tile counts, toff[nl] their sum; a tile past it gets leaf -1, and every
+// tile where bad is given and *bad is not 0)
+Scratch tile_leaves(Plan& P, const int64_t* toff, int64_t nl, int64_t total, cudaStream_t s,
+                    const int64_t* bad = nullptr);
 
 struct IpmParams {
   double u0, v0, inv_du, inv_dv;  // source-plane window origin, inverse pixel size

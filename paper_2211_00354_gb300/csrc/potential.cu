@@ -207,14 +207,14 @@ __device__ __forceinline__ double pot_m2p(double a0, int p, double2 t, double rC
 // Thread per ray, rays in leaf order (slot[r]: its leaf).
 template <bool UM>
 __global__ void __launch_bounds__(128)
-k_pot_rays(PotArgs A, const double* __restrict__ rays, const int64_t* __restrict__ n_in,
+k_pot_rays(PotArgs A, const double* __restrict__ rays, int64_t m, const int64_t* __restrict__ bad,
            const int* __restrict__ slot,
            const int* __restrict__ perm, const LeafPot* __restrict__ lp,
            const double2* __restrict__ Bi, int wmax, double* __restrict__ psi) {
   __shared__ double inv[kPotInv];
   fill_inv(inv, A.p + 2);
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= *n_in) return;  // the rays that lie in a leaf
+  if (t >= m || *bad) return;  // all rays lie in a leaf, or the call is refused
   const int64_t r = perm[t];
   const double x = rays[2 * r], y = rays[2 * r + 1];
   const int k0 = slot[r];
@@ -288,15 +288,15 @@ void evaluate_potential(Plan& P, const double* rays, int64_t m, double* psi, cud
   // masses, ~35 with a logarithm each
   const int wmax = (6 * P.p + 45) / (P.equal_mass ? 5 : 35);
   if (P.equal_mass)
-    k_pot_rays<true><<<grid_for(m, 128), 128, 0, s>>>(A, rays, RB.off + nl, RB.slot.as<int>(),
+    k_pot_rays<true><<<grid_for(m, 128), 128, 0, s>>>(A, rays, m, RB.bad, RB.slot.as<int>(),
                                                       RB.perm.as<int>(), lp.as<LeafPot>(),
                                                       Bi.as<double2>(), wmax, psi);
   else
-    k_pot_rays<false><<<grid_for(m, 128), 128, 0, s>>>(A, rays, RB.off + nl, RB.slot.as<int>(),
+    k_pot_rays<false><<<grid_for(m, 128), 128, 0, s>>>(A, rays, m, RB.bad, RB.slot.as<int>(),
                                                        RB.perm.as<int>(), lp.as<LeafPot>(),
                                                        Bi.as<double2>(), wmax, psi);
   LENS_LAUNCHED("k_pot_rays");
-  check_rays(RB);
+  check_rays(RB, s);
   LENS_CUDA(cudaStreamSynchronize(s));
 }
 
