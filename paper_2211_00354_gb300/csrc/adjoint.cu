@@ -707,7 +707,7 @@ void adjoint(Plan& P, const double* rays, int64_t m, const double* gy, double* g
                                                  RB.bad, gxy, gm);
     LENS_LAUNCHED("k_adj_out");
   }
-  check_rays(RB, s);
+  check_rays(RB);
 }
 
 }  // namespace lens

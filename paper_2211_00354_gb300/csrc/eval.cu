@@ -663,6 +663,7 @@ void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B
   int64_t* off = bad + 1;
   int64_t* toff = off + n;
   B.flag = host_slot();
+  B.wait.begin(s);
   B.flag.host[0] = 0;
   LENS_CUDA(cudaEventCreateWithFlags(&B.leaves_known, cudaEventDisableTiming));
   LENS_CUDA(cudaMemsetAsync(B.mem.p, 0, sizeof(int64_t) * (2 * n + 1), s));
@@ -690,12 +691,11 @@ void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B
   if (B.tiles_max > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
 }
 
-void check_rays(const RayBuckets& B, cudaStream_t s) {
+void check_rays(RayBuckets& B) {
   LENS_CUDA(cudaEventSynchronize(B.leaves_known));
-  if (!B.flag.host[0]) return;
-  // what was launched returns at once; the caller may free its buffers on the error
-  LENS_CUDA(cudaStreamSynchronize(s));
-  fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
+  // (B.wait then waits for what was launched: the caller may free its buffers on the error)
+  if (B.flag.host[0]) fail(LENS_EDOMAIN, "a ray lies outside the plan's target region (or is not finite)");
+  B.wait.done();
 }
 
 void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* jac, cudaStream_t s) {
@@ -715,7 +715,7 @@ void evaluate_rays(Plan& P, const double* rays, int64_t m, double* y, double* ja
   } else {
     eval32_rays(P, rays, B.off, B.perm.as<int>(), tl.as<int2>(), B.tiles_max, y, jac, s);
   }
-  check_rays(B, s);
+  check_rays(B);
 }
 
 }  // namespace lens

@@ -69,13 +69,30 @@ struct Scratch {
 // read-back of a size or a flag is then one kernel's store and one wait instead
 // of a copy on top.  One block per host thread (kept until the thread ends),
 // handed out in turn; a slot is read before kHostSlots later ones are taken,
-// since every call that takes one waits for it before it returns.
+// since every call that takes one waits for it before it returns, by a SlotWait
+// where it ends with an error.
 constexpr int kHostSlots = 64, kHostSlotWords = 80;
 struct HostSlot {
   volatile int64_t* host;  // kHostSlotWords words
   int64_t* dev;
 };
 HostSlot host_slot();
+// Between taking a slot and its read: waits for the stream whose kernels store into the
+// slot when the scope is left before done().
+class SlotWait {
+ public:
+  SlotWait() = default;
+  explicit SlotWait(cudaStream_t s) : s_(s), pending_(true) {}
+  SlotWait(const SlotWait&) = delete;
+  SlotWait& operator=(const SlotWait&) = delete;
+  ~SlotWait() { if (pending_) cudaStreamSynchronize(s_); }
+  void begin(cudaStream_t s) { s_ = s; pending_ = true; }
+  void done() { pending_ = false; }
+
+ private:
+  cudaStream_t s_ = nullptr;
+  bool pending_ = false;
+};
 
 constexpr int kMaxDepth = 28;   // quadtree levels below the root (56-bit keys)
 constexpr int kMaxOrder = 64;   // expansion order cap
@@ -299,6 +316,7 @@ struct RayBuckets {
   const int64_t* bad = nullptr;
   int64_t tiles_max = 0;
   HostSlot flag{};
+  SlotWait wait;                       // until check_rays has found the flag down
   cudaEvent_t leaves_known = nullptr;  // every ray has its leaf (or raised the flag)
   RayBuckets() = default;
   RayBuckets(const RayBuckets&) = delete;
@@ -306,7 +324,7 @@ struct RayBuckets {
   ~RayBuckets() { if (leaves_known) cudaEventDestroy(leaves_known); }
 };
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s);
-void check_rays(const RayBuckets& B, cudaStream_t s);
+void check_rays(RayBuckets& B);
 // (leaf, tile within the leaf) of each of `total` tiles (toff: exclusive scan of
 // the leaves' tile counts, toff[nl] their sum; a tile past it gets leaf -1, and every
 // tile where bad is given and *bad is not 0)

@@ -296,7 +296,7 @@ void evaluate_potential(Plan& P, const double* rays, int64_t m, double* psi, cud
                                                        RB.perm.as<int>(), lp.as<LeafPot>(),
                                                        Bi.as<double2>(), wmax, psi);
   LENS_LAUNCHED("k_pot_rays");
-  check_rays(RB, s);
+  check_rays(RB);
   LENS_CUDA(cudaStreamSynchronize(s));
 }
 

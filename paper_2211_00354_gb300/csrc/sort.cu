@@ -279,9 +279,11 @@ void read_i64(const int64_t* const* addrs, int n, int64_t* host, cudaStream_t s)
   for (int i = 0; i < n; ++i) a.src[i] = addrs[i];
   a.n = n;
   const HostSlot slot = host_slot();
+  SlotWait wait(s);
   k_pick_i64<<<1, kMaxPick, 0, s>>>(a, slot.dev);
   LENS_LAUNCHED("k_pick_i64");
   LENS_CUDA(cudaStreamSynchronize(s));
+  wait.done();
   for (int i = 0; i < n; ++i) host[i] = slot.host[i];
 }
 
@@ -294,9 +296,11 @@ __global__ void k_copy_words(const int64_t* __restrict__ in, int n, int64_t* __r
 void read_words(const int64_t* dev, int n, int64_t* host, cudaStream_t s) {
   if (n < 1 || n > kMaxPick) fail(LENS_EINVAL, "internal: too many values in one read-back");
   const HostSlot slot = host_slot();
+  SlotWait wait(s);
   k_copy_words<<<1, kMaxPick, 0, s>>>(dev, n, slot.dev);
   LENS_LAUNCHED("k_copy_words");
   LENS_CUDA(cudaStreamSynchronize(s));
+  wait.done();
   for (int i = 0; i < n; ++i) host[i] = slot.host[i];
 }
 

@@ -633,6 +633,7 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
   {
     Scratch dpart(&P.da, sizeof(double) * kBoundsParts * nbb);
     const HostSlot slot = host_slot();
+    SlotWait wait(s);
     k_bounds<<<nbb, kBoundsThreads, 0, s>>>(stars, masses, n, dpart.as<double>());
     LENS_LAUNCHED("k_bounds");
     k_bounds_final<<<1, 32 * kBoundsParts, 0, s>>>(dpart.as<double>(), nbb, slot.dev);
@@ -640,6 +641,7 @@ void tree_build_boxes(Plan& P, const double* stars, const double* masses, cudaSt
     // the translation tables are formed on the host while the bounds run
     fmm_tables(P, s);
     LENS_CUDA(cudaStreamSynchronize(s));
+    wait.done();
     for (int k = 0; k < kBoundsParts; ++k) {
       const int64_t w = slot.host[k];
       std::memcpy(&q[k], &w, sizeof(double));
