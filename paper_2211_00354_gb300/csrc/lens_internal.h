@@ -67,8 +67,8 @@ struct Scratch {
 
 // A few words of host memory that kernels write through the mapped pointer: the
 // read-back of a size or a flag is then one kernel's store and one wait instead
-// of a copy on top.  One block per host thread (kept until the thread ends),
-// handed out in turn; a slot is read before kHostSlots later ones are taken,
+// of a copy on top.  One block per host thread (passed on to a later thread when it
+// ends), handed out in turn; a slot is read before kHostSlots later ones are taken,
 // since every call that takes one waits for it before it returns, by a SlotWait
 // where it ends with an error.
 constexpr int kHostSlots = 64, kHostSlotWords = 80;
