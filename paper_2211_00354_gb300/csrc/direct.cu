@@ -127,7 +127,10 @@ k_direct_f64(const double* __restrict__ stars, const double* __restrict__ sm, in
     for (int q = 0; q < cnt; ++q) {
       const double d1 = x1 - t_pos[q].x, d2 = x2 - t_pos[q].y;
       const double r2 = d1 * d1 + d2 * d2;
-      const double inv = rcp_or_zero(r2);
+      double inv;
+      if (rcp_in_range(r2)) inv = rcp_newton(r2);
+      else if (r2 == 0.0) continue;  // a star exactly on the ray, whatever its mass
+      else inv = 1.0 / r2;           // a NaN coordinate makes both components NaN
       const double w = t_m[q] * inv;
       px = fma(w, d1, px);
       py = fma(w, d2, py);
