@@ -197,7 +197,11 @@ __global__ void __launch_bounds__(128) k_adj_p2p(AdjArgs A) {
 #pragma unroll 2
     for (int t = 0; t < nr; ++t) {
       const double2 d = make_double2(sz[t].x - zj.x, sz[t].y - zj.y);
-      const double w = rcp_or_zero(d.x * d.x + d.y * d.y);  // 0: self-interaction skipped
+      const double r2 = d.x * d.x + d.y * d.y;
+      double w;
+      if (rcp_in_range(r2)) w = rcp_newton(r2);
+      else if (r2 == 0.0) continue;  // self-interaction, whatever the charge
+      else w = 1.0 / r2;
       const double2 inv = make_double2(d.x * w, -d.y * w);
       const double2 ci = cmul(sc[t], inv);
       F = F + ci;
