@@ -67,6 +67,7 @@ struct E32Args {
   // ray source
   const double* rays; const int64_t* ray_off; const int* perm;
   double* y; double* jac;
+  bool y16;  // y starts on a 16-byte boundary (the caller's buffer need not)
   PixCorner* pix; ff iduf, idvf;
 };
 
@@ -759,10 +760,18 @@ __global__ void __launch_bounds__(kT, 7) k_eval_quads(E32Args A) {
       if (okc[0]) A.pix[o] = pc[0];
       if (okc[1]) A.pix[o + half] = pc[1];
     } else {
-      double2* y = reinterpret_cast<double2*>(A.y);
       const double K1 = lp->K1, K2 = lp->K2;
-      if (okc[0]) y[o] = make_double2(K1 + ff_to_double(ff{T1.hi.x, T1.lo.x}), K2 + ff_to_double(ff{T2.hi.x, T2.lo.x}));
-      if (okc[1]) y[o + half] = make_double2(K1 + ff_to_double(ff{T1.hi.y, T1.lo.y}), K2 + ff_to_double(ff{T2.hi.y, T2.lo.y}));
+      const auto put = [&](int64_t i, ff t1, ff t2) {
+        const double2 v = make_double2(K1 + ff_to_double(t1), K2 + ff_to_double(t2));
+        if (A.y16) {
+          reinterpret_cast<double2*>(A.y)[i] = v;
+        } else {
+          A.y[2 * i] = v.x;
+          A.y[2 * i + 1] = v.y;
+        }
+      };
+      if (okc[0]) put(o, ff{T1.hi.x, T1.lo.x}, ff{T2.hi.x, T2.lo.x});
+      if (okc[1]) put(o + half, ff{T1.hi.y, T1.lo.y}, ff{T2.hi.y, T2.lo.y});
     }
   }
 }
@@ -1270,6 +1279,7 @@ void eval32_grid(Plan& P, const GridRows& g, const int64_t* rect, const int2* ti
   A.gnx1 = g.nx + 1;
   A.grow0 = g.row0;
   A.y = y; A.jac = jac; A.pix = pix;
+  A.y16 = reinterpret_cast<uintptr_t>(y) % 16 == 0;
   if (px) { A.iduf = ff_of(ip->inv_du); A.idvf = ff_of(ip->inv_dv); }
   wait_expansions(P, s);
   leaf_grid(px ? 3 : 1);
