@@ -687,7 +687,7 @@ void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B
   B.off = off;
   B.toff = toff;
   B.bad = bad;
-  B.tiles_max = m / tile + std::min(nl, m);
+  B.tiles_max = ray_tiles_max(m, nl, tile);
   if (B.tiles_max > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many ray tiles in one call");
 }
 

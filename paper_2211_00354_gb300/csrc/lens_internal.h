@@ -323,6 +323,11 @@ struct RayBuckets {
   RayBuckets& operator=(const RayBuckets&) = delete;
   ~RayBuckets() { if (leaves_known) cudaEventDestroy(leaves_known); }
 };
+// Tiles of m rays over nl leaves, at most: a leaf of c rays has (c + tile - 1) / tile, and
+// at most min(nl, m) leaves have any.
+constexpr int64_t ray_tiles_max(int64_t m, int64_t nl, int tile) {
+  return (m + (int64_t)(tile - 1) * (nl < m ? nl : m)) / tile;
+}
 void bucket_rays(Plan& P, const double* rays, int64_t m, int tile, RayBuckets& B, cudaStream_t s);
 void check_rays(RayBuckets& B);
 // (leaf, tile within the leaf) of each of `total` tiles (toff: exclusive scan of
