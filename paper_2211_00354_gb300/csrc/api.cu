@@ -1,7 +1,7 @@
 // api.cu -- the extern "C" boundary of liblens.so (declared in include/lens.h)
 // plus the host plumbing: status codes, thread-local error text, device
 // allocation through the caller's allocator, host-side fault injection
-// (LENS_FAULT=alloc@K | launch@K), and the chunk driver of lens_ipm_map
+// (LENS_FAULT=alloc@K | launch@K | memory@BYTES), and the chunk driver of lens_ipm_map
 // (Sec. 2.4: split the image plane into chunks, deflect each chunk with the
 // FMM, apportion its cells with IPM, accumulate one map).
 #include <algorithm>
@@ -13,6 +13,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "lens_internal.h"
@@ -27,17 +28,30 @@ std::atomic<long long> g_alloc_count{0}, g_launch_count{0};
 
 struct FaultSpec {
   long long alloc_at = -1, launch_at = -1;
+  long long memory = -1;  // bytes that the library's pool can give out (-1: the device's)
   FaultSpec() {
     const char* e = std::getenv("LENS_FAULT");
     if (!e) return;
     long long k = 0;
     if (std::sscanf(e, "alloc@%lld", &k) == 1) alloc_at = k;
     else if (std::sscanf(e, "launch@%lld", &k) == 1) launch_at = k;
+    else if (std::sscanf(e, "memory@%lld", &k) == 1) memory = k;
   }
 };
 const FaultSpec& fault_spec() {
   static FaultSpec f;
   return f;
+}
+
+// The library's pool as a device of few bytes (LENS_FAULT=memory@BYTES)
+struct SmallDevice {
+  std::mutex mu;
+  std::unordered_map<void*, size_t> size;
+  size_t used = 0;
+};
+SmallDevice& small_device() {
+  static SmallDevice* d = new SmallDevice();
+  return *d;
 }
 }  // namespace
 
@@ -162,19 +176,37 @@ void* DeviceAlloc::alloc(size_t bytes) {
     p = a.alloc(bytes, (void*)stream, a.ctx);
     if (!p) fail(LENS_ENOMEM, "allocator returned NULL for " + std::to_string(bytes) + " bytes");
   } else {
+    const bool small = fault_spec().memory >= 0;
+    SmallDevice& d = small_device();
+    std::unique_lock<std::mutex> lock(d.mu, std::defer_lock);
+    if (small) {
+      lock.lock();
+      if (d.used + bytes > (size_t)fault_spec().memory)
+        fail(LENS_ENOMEM, "no " + std::to_string(bytes) + " bytes left (LENS_FAULT)");
+    }
     cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, library_pool(), stream);
     if (e != cudaSuccess) {
       cudaGetLastError();
       fail(LENS_ENOMEM, "cudaMallocFromPoolAsync(" + std::to_string(bytes) + "): " + cudaGetErrorString(e));
     }
+    if (small) d.used += d.size[p] = bytes;
   }
   return p;
 }
 
 void DeviceAlloc::release(void* p) {
   if (!p) return;
-  if (custom) a.free(p, (void*)stream, a.ctx);
-  else cudaFreeAsync(p, stream);
+  if (custom) {
+    a.free(p, (void*)stream, a.ctx);
+    return;
+  }
+  if (fault_spec().memory >= 0) {
+    SmallDevice& d = small_device();
+    std::lock_guard<std::mutex> lock(d.mu);
+    d.used -= d.size[p];
+    d.size.erase(p);
+  }
+  cudaFreeAsync(p, stream);
 }
 
 }  // namespace lens

@@ -514,6 +514,8 @@ struct RayParts {
 // the gradient of few rays takes them as they come: the counting, its scan and read-back
 // cost more than the order saves (300 samples: 100 rays 259 -> 204 us, 5000 rays the same)
 constexpr int64_t kFewRays = 1 << 12;
+// rays at a time where the memory for the order is not to be had (2 MB of positions)
+constexpr int64_t kRayStep = 1 << 16;
 
 RayGrid ray_grid(const SampleGrid& G, int sub) {
   const double icell = 1.0 / G.cell;
@@ -523,9 +525,8 @@ RayGrid ray_grid(const SampleGrid& G, int sub) {
                  (float)(sub * icell), sub};
 }
 
-void bucket_near_rays(const double* y, int64_t m, const SampleGrid& G, bool numbers, DeviceAlloc& da,
-                      cudaStream_t s, RayParts& B) {
-  int sub = kMaxSub;
+void bucket_near_rays(const double* y, int64_t m, const SampleGrid& G, int sub, bool numbers,
+                      DeviceAlloc& da, cudaStream_t s, RayParts& B) {
   const int64_t nce = (int64_t)(G.nx + 2) * (G.ny + 2);
   while (sub > 1 && nce * sub * sub > (1 << 22)) sub /= 2;
   const int64_t np = nce * sub * sub;
@@ -562,7 +563,13 @@ void light_curve(const double* y, int64_t m, double w, const double* smp, int64_
   build_sample_grid(smp, ns, sigma, trunc, da, s, H);
   const SampleGrid& G = H.G;
   RayParts B;
-  bucket_near_rays(y, m, G, false, da, s, B);
+  try {
+    bucket_near_rays(y, m, G, kMaxSub, false, da, s, B);
+  } catch (const Error& e) {
+    if (e.status != LENS_ENOMEM) throw;
+    B = RayParts{};  // whole cells: a sixteenth of the counters
+    bucket_near_rays(y, m, G, 1, false, da, s, B);
+  }
   if (ns > (int64_t)INT32_MAX) fail(LENS_EINVAL, "too many light-curve samples");
   static const ExpTab kExp = make_exp_tab();
   k_lc_fwd<<<(unsigned)ns, kLcThreads, 0, s>>>(smp, ns, G, B.R, B.off.as<int64_t>(), B.yp.as<Pos>(), kExp,
@@ -595,22 +602,34 @@ void light_curve_grad(const double* y, int64_t m, double w, const double* smp, i
                                                       coef.as<float2>());
   LENS_LAUNCHED("k_lc_sample_coef");
   static const ExpTab kExp = make_exp_tab();
-  RayParts B;
-  if (m <= kFewRays) {
-    B.R = ray_grid(H.G, 1);
-    B.near = m;
-    B.yp = Scratch(&da, sizeof(Pos) * (size_t)m);
-    k_lc_ray_pos<<<grid_for(m, 256), 256, 0, s>>>(y, m, H.G, B.R, B.yp.as<Pos>());
-    LENS_LAUNCHED("k_lc_ray_pos");
-  } else {
-    bucket_near_rays(y, m, H.G, true, da, s, B);
-    LENS_CUDA(cudaMemsetAsync(gy, 0, sizeof(double) * 2 * m, s));
-  }
-  if (B.near > 0) {
-    k_lc_grad<<<grid_for(B.near, kGradThreads), kGradThreads, 0, s>>>(
-        B.yp.as<Pos>(), B.num.as<int64_t>(), B.near, H.G, so.as<float4>(), coef.as<float2>(), kExp,
-        ff_of(-inv2s2), ff_of(trunc * trunc * sigma * sigma), (float)(trunc * sigma), gy);
+  const auto grad = [&](const Pos* yp, const int64_t* num, int64_t n, double* out) {
+    if (n == 0) return;
+    k_lc_grad<<<grid_for(n, kGradThreads), kGradThreads, 0, s>>>(
+        yp, num, n, H.G, so.as<float4>(), coef.as<float2>(), kExp, ff_of(-inv2s2),
+        ff_of(trunc * trunc * sigma * sigma), (float)(trunc * sigma), out);
     LENS_LAUNCHED("k_lc_grad");
+  };
+  bool ordered = m > kFewRays;
+  RayParts B;
+  try {
+    if (ordered) bucket_near_rays(y, m, H.G, kMaxSub, true, da, s, B);
+  } catch (const Error& e) {
+    if (e.status != LENS_ENOMEM) throw;
+    ordered = false;
+    B = RayParts{};
+  }
+  if (ordered) {
+    LENS_CUDA(cudaMemsetAsync(gy, 0, sizeof(double) * 2 * m, s));
+    grad(B.yp.as<Pos>(), B.num.as<int64_t>(), B.near, gy);
+  } else {
+    const int64_t step = std::min(m, kRayStep);
+    Scratch yp(&da, sizeof(Pos) * (size_t)step);
+    for (int64_t i = 0; i < m; i += step) {
+      const int64_t n = std::min(step, m - i);
+      k_lc_ray_pos<<<grid_for(n, 256), 256, 0, s>>>(y + 2 * i, n, H.G, ray_grid(H.G, 1), yp.as<Pos>());
+      LENS_LAUNCHED("k_lc_ray_pos");
+      grad(yp.as<Pos>(), nullptr, n, gy + 2 * i);
+    }
   }
   LENS_CUDA(cudaStreamSynchronize(s));
 }
