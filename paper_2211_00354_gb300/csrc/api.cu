@@ -168,6 +168,15 @@ HostSlot host_slot() {
   return HostSlot{b.host + k, b.dev + k};
 }
 
+size_t free_memory() {
+  size_t fr = 0, tot = 0;
+  LENS_CUDA(cudaMemGetInfo(&fr, &tot));
+  if (fault_spec().memory < 0) return fr;
+  SmallDevice& d = small_device();
+  std::lock_guard<std::mutex> lock(d.mu);
+  return std::min(fr, (size_t)fault_spec().memory - d.used);
+}
+
 void* DeviceAlloc::alloc(size_t bytes) {
   fault_point_alloc();
   if (bytes == 0) bytes = 16;
@@ -256,6 +265,167 @@ void check_grid(const Plan& P, const lens_grid* g) {
     lo1 = P.root_lo[1]; hi1 = P.root_lo[1] + P.root_size;
     if (!(g->x0 >= lo0 && x1 < hi0 && g->y0 >= lo1 && y1 < hi1))
       fail(LENS_EDOMAIN, "grid extends beyond the plan's root box");
+  }
+}
+
+// One pass of lens_ipm_map_ex over the grid in chunks of `rows` rows: deflection, IPM,
+// refinement, the map and its ledger.  Throws with the map undefined; nothing of it
+// outlives the call.
+void map_pass(Plan& P, const lens_grid& grid, const IpmParams& ip, int64_t rows, int64_t flush_cells,
+              int refine_levels, bool fused, double* map_out, lens_ipm_stats* stats, cudaStream_t s) {
+  const int64_t nx = grid.nx, ny = grid.ny;
+  const int npx = ip.npx, npy = ip.npy;
+  Scratch corners(&P.da, sizeof(PixCorner) * (size_t)(rows + 1) * (size_t)(nx + 1));
+  Scratch queue(&P.da, sizeof(int) * (size_t)rows * (size_t)nx + sizeof(int) * 4);
+  Scratch sdev(&P.da, sizeof(double) * 16);
+  // the map accumulates in float32 (increments are O(1) and a pixel receives
+  // ~mu n_0 of them; float32 keeps ~1e-6 relative) and is written out in
+  // float64 once at the end, so no float64 conversion runs per increment
+  Scratch map32(&P.da, sizeof(float) * (size_t)npx * (size_t)npy);
+  // whole-pixel runs of large cells enter as +v / -v at the ends of the run
+  // in a per-row difference array, prefix-summed into the map at the end
+  Scratch rowdiff(&P.da, sizeof(float) * ((size_t)npx + 1) * (size_t)npy);
+  int* qcount = queue.as<int>() + (size_t)rows * (size_t)nx;
+  // refinement: the grid cells of a chunk over the cap, then per level
+  Scratch rq0(&P.da, refine_levels > 0 ? sizeof(int) * ((size_t)rows * (size_t)nx + 2) : 0);
+  int* rq0count = refine_levels > 0 ? rq0.as<int>() + (size_t)rows * (size_t)nx : nullptr;
+  int64_t refined = 0;
+  LENS_CUDA(cudaMemsetAsync(map32.p, 0, map32.bytes, s));
+  LENS_CUDA(cudaMemsetAsync(rowdiff.p, 0, rowdiff.bytes, s));
+  LENS_CUDA(cudaMemsetAsync(sdev.p, 0, sdev.bytes, s));
+  P.ev_clear();
+  P.timing = true;
+  P.work = sdev.as<double>() + 12;
+  struct Reset {
+    Plan& P;
+    ~Reset() { P.timing = false; P.work = nullptr; P.ev_clear(); }
+  } reset{P};
+  struct Events : std::vector<cudaEvent_t> {
+    ~Events() { for (auto e : *this) cudaEventDestroy(e); }
+  } ev;
+  auto mark = [&]() {
+    cudaEvent_t e;
+    LENS_CUDA(cudaEventCreate(&e));
+    ev.push_back(e);
+    LENS_CUDA(cudaEventRecord(e, s));
+  };
+  int64_t chunks = 0, pending = 0;
+  bool flushed = false;
+  const long long l0 = launch_count();
+  for (int64_t r0 = 0; r0 < ny; r0 += rows) {
+    const int64_t nr = std::min<int64_t>(rows, ny - r0);
+    if (pending > 0 && pending + nr * nx > flush_cells) {
+      ipm_finish_map(map32.as<float>(), rowdiff.as<float>(), npx, npy, map_out, flushed, true, s);
+      flushed = true;
+      pending = 0;
+    }
+    GridRows g{grid.x0, grid.y0, grid.h, nx, ny, r0, nr + 1};
+    if (rq0count) LENS_CUDA(cudaMemsetAsync(rq0count, 0, sizeof(int), s));
+    if (fused) {
+      // deflection and IPM in one kernel; only leaf-boundary corners reach
+      // `corners`, for the seam cells mapped after it
+      mark();
+      evaluate_grid_fused(P, g, corners.as<PixCorner>(), ip, map32.as<float>(), rowdiff.as<float>(),
+                          sdev.as<double>(), queue.as<int>(), qcount, rq0.as<int>(), rq0count, s);
+      mark();
+    } else {
+      mark();
+      evaluate_grid_pix(P, g, corners.as<PixCorner>(), ip, s);
+      mark();
+      ipm_accumulate(corners.as<PixCorner>(), nx, nr, ip, map32.as<float>(), rowdiff.as<float>(),
+                     sdev.as<double>(), queue.as<int>(), qcount, rq0.as<int>(), rq0count, s,
+                     &P.ev_ipm);
+    }
+    pending += nr * nx;
+    ++chunks;
+    if (refine_levels > 0) {
+      // split the cells over the cap 2 x 2, level by level; the sub-cell
+      // corner rays are not part of the grid's ray count
+      double* work = P.work;
+      P.work = nullptr;
+      int np = 0;
+      LENS_CUDA(cudaMemcpyAsync(&np, rq0count, sizeof(int), cudaMemcpyDeviceToHost, s));
+      LENS_CUDA(cudaStreamSynchronize(s));
+      Scratch parents_keep, org_keep;
+      const int* parents = rq0.as<int>();
+      const double2* org_in = nullptr;
+      double hc = grid.h;
+      for (int level = 1; level <= refine_levels && np > 0; ++level) {
+        const bool more = level < refine_levels;
+        Scratch org_out(&P.da, sizeof(double2) * 4 * (size_t)np);
+        Scratch rq(&P.da, more ? sizeof(int) * (4 * (size_t)np + 2) : 0);
+        int* rqc = more ? rq.as<int>() + 4 * (size_t)np : nullptr;
+        if (rqc) LENS_CUDA(cudaMemsetAsync(rqc, 0, sizeof(int), s));
+        ipm_refine(P, parents, np, org_in, grid.x0, grid.y0, r0, nx, hc, level, ip,
+                   map32.as<float>(), rowdiff.as<float>(), sdev.as<double>(),
+                   more ? rq.as<int>() : nullptr, rqc, org_out.as<double2>(), s, &P.ev_ipm);
+        refined += np;
+        pending += 4 * (int64_t)np;
+        int next = 0;
+        if (more) {
+          LENS_CUDA(cudaMemcpyAsync(&next, rqc, sizeof(int), cudaMemcpyDeviceToHost, s));
+          LENS_CUDA(cudaStreamSynchronize(s));
+        }
+        // this level's queue and corners feed the next one
+        parents_keep = std::move(rq);
+        org_keep = std::move(org_out);
+        parents = parents_keep.as<int>();
+        org_in = org_keep.as<double2>();
+        np = next;
+        hc *= 0.5;
+      }
+      P.work = work;
+    }
+  }
+  ipm_finish_map(map32.as<float>(), rowdiff.as<float>(), npx, npy, map_out, flushed, false, s);
+  mark();
+  double hs[16];
+  int64_t hw[16];
+  read_words(sdev.as<int64_t>(), 16, hw, s);
+  std::memcpy(hs, hw, sizeof(hs));
+  double msd = 0, msi = 0;
+  for (size_t k = 0; k + 1 < ev.size(); ++k) {
+    float ms = 0;
+    cudaEventElapsedTime(&ms, ev[k], ev[k + 1]);
+    if (k % 2 == 0) msd += ms; else msi += ms;
+  }
+  // every corner of every chunk must have been owned by exactly one leaf
+  double expect_rays = 0;
+  for (int64_t r0 = 0; r0 < ny; r0 += rows)
+    expect_rays += (double)(std::min<int64_t>(rows, ny - r0) + 1) * (double)(nx + 1);
+  if (hs[12] != expect_rays)
+    fail(LENS_ECUDA, "internal: leaves covered " + std::to_string(hs[12]) + " of " +
+                         std::to_string(expect_rays) + " grid rays");
+  double mse = 0, msk = 0;
+  for (auto& e : P.ev_eval) { float ms = 0; cudaEventElapsedTime(&ms, e.first, e.second); mse += ms; }
+  for (auto& e : P.ev_ipm) { float ms = 0; cudaEventElapsedTime(&ms, e.first, e.second); msk += ms; }
+  double msf = 0;
+  for (auto& e : P.ev_fused) { float ms = 0; cudaEventElapsedTime(&ms, e.first, e.second); msf += ms; }
+  if (stats) {
+    stats->cells = (double)nx * (double)ny;
+    stats->area_total = stats->cells * ip.a_cell;
+    stats->area_in_map = ip.a_cell * hs[2];
+    stats->area_outside = ip.a_cell * hs[3];
+    stats->area_dropped = ip.a_cell * hs[6];
+    stats->area_degenerate = ip.a_cell * hs[7];
+    stats->cells_dropped = hs[4];
+    stats->cells_degenerate = hs[5];
+    stats->chunks = chunks;
+    stats->ms_deflect = msd;
+    stats->ms_ipm = msi;
+    stats->rays = hs[12];
+    stats->p2p_pairs = hs[13];
+    stats->m2p_evals = hs[14];
+    stats->ipm_updates = hs[8];
+    stats->cells_queued = hs[9];
+    stats->cells_ext = hs[10];
+    stats->ms_eval_kernel = mse;
+    stats->ms_ipm_kernel = msk;
+    stats->launches = launch_count() - l0;
+    stats->cells_refined = (double)refined;
+    stats->fused = fused ? 1 : 0;
+    stats->ms_fused_kernel = msf;
+    stats->rays_evaluated = fused ? hs[15] : hs[12];
   }
 }
 }  // namespace
@@ -528,14 +698,13 @@ lens_status lens_ipm_map_ex(lens_plan* plan, const lens_grid* grid, const lens_b
     return std::min<int64_t>(std::max<int64_t>(1, max_cells / nx), ny);
   };
   const auto rows_from_memory = [&]() {
-    size_t fr = 0, tot = 0;
-    LENS_CUDA(cudaMemGetInfo(&fr, &tot));
+    const size_t fr = free_memory();
     // 16 B per corner + 4 B queue slot per cell, within a quarter of free memory
     return rows_for((int64_t)std::min<double>((double)fr / 4.0 / 20.0, (double)(1ll << 30)));
   };
   // A grid (or the part of it between flushes) of at most kSmallCells cells, 84 MB,
   // is taken at once: the query of the free memory costs the host as much as
-  // a few launches, and is made only if the buffers are then not to be had.
+  // a few launches, and is made only if the memory is then not to be had.
   constexpr int64_t kSmallCells = 1 << 22;
   const bool unasked = max_cells_per_chunk == 0 && std::min(flush_cells, nx * ny) <= kSmallCells;
   int64_t rows = max_cells_per_chunk ? rows_for(max_cells_per_chunk)
@@ -552,166 +721,13 @@ lens_status lens_ipm_map_ex(lens_plan* plan, const lens_grid* grid, const lens_b
   ip.scale = ip.a_cell / ip.s_star;
   ip.npx = npx; ip.npy = npy; ip.cap = bbox_cap_px;
 
-  Scratch corners, queue;
-  for (bool again = unasked;; again = false) {
-    try {
-      corners = Scratch(&P.da, sizeof(PixCorner) * (size_t)(rows + 1) * (size_t)(nx + 1));
-      queue = Scratch(&P.da, sizeof(int) * (size_t)rows * (size_t)nx + sizeof(int) * 4);
-      break;
-    } catch (const Error& e) {
-      if (!again || e.status != LENS_ENOMEM) throw;
-      corners.reset();
-      rows = rows_from_memory();
-    }
-  }
-  Scratch sdev(&P.da, sizeof(double) * 16);
-  // the map accumulates in float32 (increments are O(1) and a pixel receives
-  // ~mu n_0 of them; float32 keeps ~1e-6 relative) and is written out in
-  // float64 once at the end, so no float64 conversion runs per increment
-  Scratch map32(&P.da, sizeof(float) * (size_t)npx * (size_t)npy);
-  // whole-pixel runs of large cells enter as +v / -v at the ends of the run
-  // in a per-row difference array, prefix-summed into the map at the end
-  Scratch rowdiff(&P.da, sizeof(float) * ((size_t)npx + 1) * (size_t)npy);
-  int* qcount = queue.as<int>() + (size_t)rows * (size_t)nx;
-  // refinement: the grid cells of a chunk over the cap, then per level
-  Scratch rq0(&P.da, refine_levels > 0 ? sizeof(int) * ((size_t)rows * (size_t)nx + 2) : 0);
-  int* rq0count = refine_levels > 0 ? rq0.as<int>() + (size_t)rows * (size_t)nx : nullptr;
-  int64_t refined = 0;
-  LENS_CUDA(cudaMemsetAsync(map32.p, 0, map32.bytes, s));
-  LENS_CUDA(cudaMemsetAsync(rowdiff.p, 0, rowdiff.bytes, s));
-  LENS_CUDA(cudaMemsetAsync(sdev.p, 0, sdev.bytes, s));
-  P.ev_clear();
-  P.timing = true;
-  P.work = sdev.as<double>() + 12;
-  struct Reset {
-    Plan& P;
-    ~Reset() { P.timing = false; P.work = nullptr; P.ev_clear(); }
-  } reset{P};
-  std::vector<cudaEvent_t> ev;
-  auto mark = [&]() {
-    cudaEvent_t e;
-    LENS_CUDA(cudaEventCreate(&e));
-    LENS_CUDA(cudaEventRecord(e, s));
-    ev.push_back(e);
-  };
-  int64_t chunks = 0, pending = 0;
-  bool flushed = false;
-  const long long l0 = launch_count();
-  for (int64_t r0 = 0; r0 < ny; r0 += rows) {
-    const int64_t nr = std::min<int64_t>(rows, ny - r0);
-    if (pending > 0 && pending + nr * nx > flush_cells) {
-      ipm_finish_map(map32.as<float>(), rowdiff.as<float>(), npx, npy, map_out, flushed, true, s);
-      flushed = true;
-      pending = 0;
-    }
-    GridRows g{grid->x0, grid->y0, grid->h, nx, ny, r0, nr + 1};
-    if (rq0count) LENS_CUDA(cudaMemsetAsync(rq0count, 0, sizeof(int), s));
-    if (fused) {
-      // deflection and IPM in one kernel; only leaf-boundary corners reach
-      // `corners`, for the seam cells mapped after it
-      mark();
-      evaluate_grid_fused(P, g, corners.as<PixCorner>(), ip, map32.as<float>(), rowdiff.as<float>(),
-                          sdev.as<double>(), queue.as<int>(), qcount, rq0.as<int>(), rq0count, s);
-      mark();
-    } else {
-      mark();
-      evaluate_grid_pix(P, g, corners.as<PixCorner>(), ip, s);
-      mark();
-      ipm_accumulate(corners.as<PixCorner>(), nx, nr, ip, map32.as<float>(), rowdiff.as<float>(),
-                     sdev.as<double>(), queue.as<int>(), qcount, rq0.as<int>(), rq0count, s,
-                     &P.ev_ipm);
-    }
-    pending += nr * nx;
-    ++chunks;
-    if (refine_levels > 0) {
-      // split the cells over the cap 2 x 2, level by level; the sub-cell
-      // corner rays are not part of the grid's ray count
-      double* work = P.work;
-      P.work = nullptr;
-      int np = 0;
-      LENS_CUDA(cudaMemcpyAsync(&np, rq0count, sizeof(int), cudaMemcpyDeviceToHost, s));
-      LENS_CUDA(cudaStreamSynchronize(s));
-      Scratch parents_keep, org_keep;
-      const int* parents = rq0.as<int>();
-      const double2* org_in = nullptr;
-      double hc = grid->h;
-      for (int level = 1; level <= refine_levels && np > 0; ++level) {
-        const bool more = level < refine_levels;
-        Scratch org_out(&P.da, sizeof(double2) * 4 * (size_t)np);
-        Scratch rq(&P.da, more ? sizeof(int) * (4 * (size_t)np + 2) : 0);
-        int* rqc = more ? rq.as<int>() + 4 * (size_t)np : nullptr;
-        if (rqc) LENS_CUDA(cudaMemsetAsync(rqc, 0, sizeof(int), s));
-        ipm_refine(P, parents, np, org_in, grid->x0, grid->y0, r0, nx, hc, level, ip,
-                   map32.as<float>(), rowdiff.as<float>(), sdev.as<double>(),
-                   more ? rq.as<int>() : nullptr, rqc, org_out.as<double2>(), s, &P.ev_ipm);
-        refined += np;
-        pending += 4 * (int64_t)np;
-        int next = 0;
-        if (more) {
-          LENS_CUDA(cudaMemcpyAsync(&next, rqc, sizeof(int), cudaMemcpyDeviceToHost, s));
-          LENS_CUDA(cudaStreamSynchronize(s));
-        }
-        // this level's queue and corners feed the next one
-        parents_keep = std::move(rq);
-        org_keep = std::move(org_out);
-        parents = parents_keep.as<int>();
-        org_in = org_keep.as<double2>();
-        np = next;
-        hc *= 0.5;
-      }
-      P.work = work;
-    }
-  }
-  ipm_finish_map(map32.as<float>(), rowdiff.as<float>(), npx, npy, map_out, flushed, false, s);
-  mark();
-  double hs[16];
-  int64_t hw[16];
-  read_words(sdev.as<int64_t>(), 16, hw, s);
-  std::memcpy(hs, hw, sizeof(hs));
-  double msd = 0, msi = 0;
-  for (size_t k = 0; k + 1 < ev.size(); ++k) {
-    float ms = 0;
-    cudaEventElapsedTime(&ms, ev[k], ev[k + 1]);
-    if (k % 2 == 0) msd += ms; else msi += ms;
-  }
-  for (auto e : ev) cudaEventDestroy(e);
-  // every corner of every chunk must have been owned by exactly one leaf
-  double expect_rays = 0;
-  for (int64_t r0 = 0; r0 < ny; r0 += rows)
-    expect_rays += (double)(std::min<int64_t>(rows, ny - r0) + 1) * (double)(nx + 1);
-  if (hs[12] != expect_rays)
-    fail(LENS_ECUDA, "internal: leaves covered " + std::to_string(hs[12]) + " of " +
-                         std::to_string(expect_rays) + " grid rays");
-  double mse = 0, msk = 0;
-  for (auto& e : P.ev_eval) { float ms = 0; cudaEventElapsedTime(&ms, e.first, e.second); mse += ms; }
-  for (auto& e : P.ev_ipm) { float ms = 0; cudaEventElapsedTime(&ms, e.first, e.second); msk += ms; }
-  double msf = 0;
-  for (auto& e : P.ev_fused) { float ms = 0; cudaEventElapsedTime(&ms, e.first, e.second); msf += ms; }
-  if (stats) {
-    stats->cells = (double)nx * (double)ny;
-    stats->area_total = stats->cells * ip.a_cell;
-    stats->area_in_map = ip.a_cell * hs[2];
-    stats->area_outside = ip.a_cell * hs[3];
-    stats->area_dropped = ip.a_cell * hs[6];
-    stats->area_degenerate = ip.a_cell * hs[7];
-    stats->cells_dropped = hs[4];
-    stats->cells_degenerate = hs[5];
-    stats->chunks = chunks;
-    stats->ms_deflect = msd;
-    stats->ms_ipm = msi;
-    stats->rays = hs[12];
-    stats->p2p_pairs = hs[13];
-    stats->m2p_evals = hs[14];
-    stats->ipm_updates = hs[8];
-    stats->cells_queued = hs[9];
-    stats->cells_ext = hs[10];
-    stats->ms_eval_kernel = mse;
-    stats->ms_ipm_kernel = msk;
-    stats->launches = launch_count() - l0;
-    stats->cells_refined = (double)refined;
-    stats->fused = fused ? 1 : 0;
-    stats->ms_fused_kernel = msf;
-    stats->rays_evaluated = fused ? hs[15] : hs[12];
+  // The first try of an unasked call may find that the memory is not there: the
+  // corner and queue buffers, or what the chunks and refinement levels need beside them.
+  try {
+    map_pass(P, *grid, ip, rows, flush_cells, refine_levels, fused, map_out, stats, s);
+  } catch (const Error& e) {
+    if (!unasked || e.status != LENS_ENOMEM) throw;
+    map_pass(P, *grid, ip, rows_from_memory(), flush_cells, refine_levels, fused, map_out, stats, s);
   }
   LENS_API_END
 }

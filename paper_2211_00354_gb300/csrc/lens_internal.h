@@ -31,6 +31,8 @@ void check_cuda(cudaError_t e, const char* what);
 void after_launch(const char* name);
 // Counts allocations (LENS_FAULT=alloc@K); throws LENS_EFAULT_INJECTED when due.
 void fault_point_alloc();
+// free device memory, or what LENS_FAULT=memory@BYTES leaves of it
+size_t free_memory();
 // kernels launched so far by this process (through LENS_LAUNCHED)
 long long launch_count();
 

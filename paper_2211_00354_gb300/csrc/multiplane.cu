@@ -303,8 +303,7 @@ extern "C" lens_status lens_multiplane_ipm_map(const lens_plane* planes, int npl
     const int64_t nx = grid->nx, ny = grid->ny;
     int64_t max_cells = max_cells_per_chunk;
     if (max_cells == 0) {
-      size_t fr = 0, tot = 0;
-      LENS_CUDA(cudaMemGetInfo(&fr, &tot));
+      const size_t fr = free_memory();
       // per corner: entry, two positions, plane output, K deflections, the
       // pixel corner; within a quarter of free memory
       const double per = 16.0 * (4 + ps.K) + 16.0 + 4.0;
