@@ -69,11 +69,13 @@ __device__ __forceinline__ void fill_inv(double* inv, int n) {
 
 // sum of ln d2 over positive d2: exponents summed as integers, mantissas
 // multiplied (each in [1, 2), so up to kLogRun of them stay in range); zeros are
-// left out, subnormal and non-finite values take their own logarithm.
+// left out, subnormal and non-finite values take their own logarithm.  The sum of the
+// exponents is kept as 2^16 e16 + e: a near field of millions of stars goes beyond 32
+// bits, a run does not.
 constexpr int kLogRun = 512;
 struct LogSum {
   double prod = 1.0, rest = 0.0;
-  int e = 0, n = 0;
+  int e16 = 0, e = 0, n = 0;
   __device__ __forceinline__ void add(double d2) {
     const int hi = __double2hiint(d2);
     if ((unsigned)hi - 0x00100000u < 0x7ff00000u - 0x00100000u) {
@@ -87,11 +89,13 @@ struct LogSum {
   __device__ __forceinline__ void fold() {  // prod back to [1, 2)
     const int hi = __double2hiint(prod);
     e += (hi >> 20) - 1023;
-    prod = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(prod));
+    e16 += e >> 16;
+    e &= 0xffff;
     n = 0;
+    prod = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(prod));
   }
   __device__ __forceinline__ double value() const {
-    return rest + fma((double)e, 0.69314718055994530942, log(prod));  // ln 2
+    return rest + fma((double)(65536ll * e16 + e), 0.69314718055994530942, log(prod));  // ln 2
   }
 };
 
