@@ -38,9 +38,10 @@ __device__ __forceinline__ float2 cfma(float2 a, float2 b, float2 c) {
 template <typename C, typename R> __host__ __device__ __forceinline__ C cscale(C a, R s) {
   C z; z.x = a.x * s; z.y = a.y * s; return z;
 }
-// 1/x for x > 0: the hardware's coarse reciprocal (relative error within 2^-23)
-// and one third-order Newton step, y (1 + e + e^2) with e = 1 - x y: the residual
-// e^3 is below 2^-69, so the result is within an ulp or so of the last rounding.
+// 1/x for x > 0: the hardware's coarse reciprocal (the PTX ISA has rcp.approx.ftz.f64 read
+// and return the upper 20 mantissa bits: a relative error of about 2^-20) and one
+// third-order Newton step, y (1 + e + e^2) with e = 1 - x y: the residual e^3 is about
+// 2^-60 against the last rounding's 2^-53, so the result is within an ulp.
 // Three float64 operations where the compiler's division takes about ten, on a
 // pipe that gives a warp one instruction per ~77 cycles and sub-partition.  Outside
 // the range where the seed is normal (and for 0, infinities, NaN) it divides.
