@@ -564,7 +564,7 @@ def config_line(args):
         tf = eval_flops / (ms_eval / 1e3) / 1e12
         line["eval_roofline"] = {"bound": "alu", "achieved": tf, "peak": fp32_peak,
                                  "unit": "TFLOP/s", "frac": tf / fp32_peak, "ms": ms_eval}
-        line["roofline"] = dict(line["eval_roofline"], kernel="k_eval32 (fused L2P+P2P+M2P)",
+        line["roofline"] = dict(line["eval_roofline"], kernel="k_eval_quads (fused L2P+P2P+M2P)",
                                 traffic=None)
         line["phase_ms"] = {"build": sum(i_["ms_build"] for i_ in infos) / K,
                             "tree": sum(i_["ms_tree"] for i_ in infos) / K}

@@ -32,7 +32,9 @@
  *   - A star exactly at a ray contributes nothing to that ray.
  *   - Environment LENS_FAULT=alloc@K or launch@K makes the K-th internal
  *     allocation or kernel launch of the process fail with
- *     LENS_EFAULT_INJECTED (host-side fault injection for tests).
+ *     LENS_EFAULT_INJECTED, and LENS_FAULT=memory@BYTES lets the library's
+ *     own pool give out BYTES at a time, LENS_ENOMEM beyond (host-side fault
+ *     injection for tests).
  */
 #ifndef LENS_H
 #define LENS_H
@@ -118,7 +120,7 @@ typedef struct {
   double p2p_pairs;    /* ray-star pairs summed directly (U lists) */
   double m2p_evals;    /* ray-box multipole evaluations (W lists) */
   double ipm_updates;  /* (cell, pixel) map increments */
-  double cells_queued; /* cells sent to the warp-per-cell path */
+  double cells_queued; /* cells of boxes over 4 x 4 pixels and ill-conditioned cells */
   double cells_ext;    /* of those, ill-conditioned cells redone in float-float (~48 bits) */
   double ms_eval_kernel;
   double ms_ipm_kernel;

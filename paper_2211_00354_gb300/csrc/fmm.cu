@@ -313,7 +313,8 @@ inline size_t downward_smem_per_box(int p) {
 
 // NW warps a box: 1 (kWarpsPerBlock boxes a block) or kFarWarps (one box a block, for up
 // to kFarFewBoxes active boxes, which as a warp each leave most of the pipes idle:
-// 33 boxes of p 24 72 -> 17 us, 329 of p 16 42 -> 22).  A box's sums are the same, term by term, for both.
+// 33 boxes of p 24 72 -> 17 us, 329 of p 16 42 -> 22; 4 * 152 is one warp a box on every
+// sub-partition of the chip's SMs).  A box's sums are the same, term by term, for both.
 constexpr int kFarWarps = 8;
 constexpr int64_t kFarFewBoxes = 4 * 152;
 
