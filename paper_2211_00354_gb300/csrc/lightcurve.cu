@@ -288,18 +288,6 @@ __global__ void k_lc_ray_cell(const double* __restrict__ y, int64_t m, SampleGri
   if (c >= 0) agg_inc(&cnt[c], c);
 }
 
-// positions in the rays' order; a ray that is not near is put beyond every cell's
-// neighbours
-__global__ void k_lc_ray_pos(const double* __restrict__ y, int64_t m, SampleGrid G, RayGrid R,
-                             Pos* __restrict__ yp) {
-  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (r >= m) return;
-  Pos p;
-  if (ray_part(G, R, y[2 * r], y[2 * r + 1], p) < 0)
-    p = Pos{make_float4(0.f, 0.f, 0.f, 0.f), make_int2(-8, -8)};
-  yp[r] = p;
-}
-
 // positions (and ray numbers, where they are asked for) in the order of the parts
 __global__ void k_lc_ray_fill(const double* __restrict__ y, int64_t m, const int* __restrict__ partof,
                               const int64_t* __restrict__ off, unsigned long long* __restrict__ cur,
@@ -416,16 +404,26 @@ __global__ void k_lc_sample_coef(const double* __restrict__ s, const int* __rest
 // samples of the 3 x 3 cells around it.  Bound by instruction issue, as the forward pass.
 // In the order of the rays, with every ray's cell by divisions: 1140 us for 3e6 rays and
 // 2048 samples (1.4e6 of them near), now 458.
+// Not ORDERED: all m rays as they come, their positions formed here.
 constexpr int kGradThreads = 128;
+template <bool ORDERED>
 __global__ void __launch_bounds__(kGradThreads)
-k_lc_grad(const Pos* __restrict__ yp, const int64_t* __restrict__ num, int64_t near, SampleGrid G,
-          const float4* __restrict__ so, const float2* __restrict__ coef, ExpTab T, ff ninv2s2, ff cut2,
-          float cutf, double* __restrict__ gy) {
+k_lc_grad(const Pos* __restrict__ yp, const int64_t* __restrict__ num, const double* __restrict__ rays,
+          int64_t m, SampleGrid G, RayGrid R, const float4* __restrict__ so,
+          const float2* __restrict__ coef, ExpTab T, ff ninv2s2, ff cut2, float cutf,
+          double* __restrict__ gy) {
   __shared__ float2 sh_exp[64];
   const ExpShared X = stage_exp(T, sh_exp);
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= near) return;
-  const Pos y = yp[i];
+  if (i >= m) return;
+  Pos y;
+  if (ORDERED) {
+    y = yp[i];
+  } else if (ray_part(G, R, rays[2 * i], rays[2 * i + 1], y) < 0) {
+    gy[2 * i] = 0.0;
+    gy[2 * i + 1] = 0.0;
+    return;
+  }
   const float side = (float)G.cell;
   ff g1{0.f, 0.f}, g2{0.f, 0.f};
   const Cut C{ninv2s2, cut2, near_cut2(cutf, side)};
@@ -449,7 +447,7 @@ k_lc_grad(const Pos* __restrict__ yp, const int64_t* __restrict__ num, int64_t n
       }
     }
   }
-  const int64_t r = num ? num[i] : i;
+  const int64_t r = ORDERED ? num[i] : i;
   gy[2 * r] = ff_to_double(g1);
   gy[2 * r + 1] = ff_to_double(g2);
 }
@@ -511,11 +509,14 @@ struct RayParts {
   int64_t near = 0;
 };
 
-// the gradient of few rays takes them as they come: the counting, its scan and read-back
-// cost more than the order saves (300 samples: 100 rays 259 -> 204 us, 5000 rays the same)
+// The gradient takes the rays as they come where there are few of them, few samples for a
+// ray to look at (9 cells' worth, on average over the grid), or few pairs of both: the
+// counting, its scan and read-back cost more than the order saves.  Random rays, as they come
+// and in order: 3e6 and 1 sample a ray 255 and 966 us, 3 samples 298 and 344, 13 samples
+// 618 and 358; 5000 and 64 samples 177 and 186, 256 samples 370 and 284; 3e4 and 16 samples
+// 131 and 171.
 constexpr int64_t kFewRays = 1 << 12;
-// rays at a time where the memory for the order is not to be had (2 MB of positions)
-constexpr int64_t kRayStep = 1 << 16;
+constexpr double kFewSamples = 8.0, kFewPairs = 1e6;
 
 RayGrid ray_grid(const SampleGrid& G, int sub) {
   const double icell = 1.0 / G.cell;
@@ -602,14 +603,8 @@ void light_curve_grad(const double* y, int64_t m, double w, const double* smp, i
                                                       coef.as<float2>());
   LENS_LAUNCHED("k_lc_sample_coef");
   static const ExpTab kExp = make_exp_tab();
-  const auto grad = [&](const Pos* yp, const int64_t* num, int64_t n, double* out) {
-    if (n == 0) return;
-    k_lc_grad<<<grid_for(n, kGradThreads), kGradThreads, 0, s>>>(
-        yp, num, n, H.G, so.as<float4>(), coef.as<float2>(), kExp, ff_of(-inv2s2),
-        ff_of(trunc * trunc * sigma * sigma), (float)(trunc * sigma), out);
-    LENS_LAUNCHED("k_lc_grad");
-  };
-  bool ordered = m > kFewRays;
+  const double seen = std::min((double)ns, 9.0 * ns / ((double)H.G.nx * H.G.ny));
+  bool ordered = m > kFewRays && seen > kFewSamples && seen * m > kFewPairs;
   RayParts B;
   try {
     if (ordered) bucket_near_rays(y, m, H.G, kMaxSub, true, da, s, B);
@@ -620,16 +615,16 @@ void light_curve_grad(const double* y, int64_t m, double w, const double* smp, i
   }
   if (ordered) {
     LENS_CUDA(cudaMemsetAsync(gy, 0, sizeof(double) * 2 * m, s));
-    grad(B.yp.as<Pos>(), B.num.as<int64_t>(), B.near, gy);
   } else {
-    const int64_t step = std::min(m, kRayStep);
-    Scratch yp(&da, sizeof(Pos) * (size_t)step);
-    for (int64_t i = 0; i < m; i += step) {
-      const int64_t n = std::min(step, m - i);
-      k_lc_ray_pos<<<grid_for(n, 256), 256, 0, s>>>(y + 2 * i, n, H.G, ray_grid(H.G, 1), yp.as<Pos>());
-      LENS_LAUNCHED("k_lc_ray_pos");
-      grad(yp.as<Pos>(), nullptr, n, gy + 2 * i);
-    }
+    B.R = ray_grid(H.G, 1);
+    B.near = m;
+  }
+  if (B.near > 0) {
+    const auto kernel = ordered ? k_lc_grad<true> : k_lc_grad<false>;
+    kernel<<<grid_for(B.near, kGradThreads), kGradThreads, 0, s>>>(
+        B.yp.as<Pos>(), B.num.as<int64_t>(), y, B.near, H.G, B.R, so.as<float4>(), coef.as<float2>(), kExp,
+        ff_of(-inv2s2), ff_of(trunc * trunc * sigma * sigma), (float)(trunc * sigma), gy);
+    LENS_LAUNCHED("k_lc_grad");
   }
   LENS_CUDA(cudaStreamSynchronize(s));
 }
