@@ -30,13 +30,21 @@ namespace lens {
 namespace {
 
 constexpr int kIpmThreads = 256;
-// 32-cell chunks per fetch of the chunk counter: at most 8 (a single address
-// serves all warps, and a fetch per chunk made it the bound of a pass without
-// B and C work), fewer where that would leave a resident warp under 8 fetches:
-// with 8 always, the 900 chunks of a refinement level went to 112 of 4864
-// warps (308 us of a 200^2-pixel window's map) and the 7.8e3 chunks of a 500^2
-// grid to 976.
-constexpr int kMaxGrab = 8;
+// 32-cell chunks per fetch of the chunk counter: at most 8 (a single address serves all
+// warps, ~2 ns a fetch: a fetch per chunk made it the bound of a pass of single-pixel cells),
+// fewer where that would leave a resident warp under kFetchesPerWarp: with 8 always, the 900
+// chunks of a refinement level went to 112 of 4864 warps (308 us of a 200^2-pixel window's
+// map). 8 fetches a warp instead of 3: 4e6 cells of single pixels 113 -> 170 us.
+constexpr int kMaxGrab = 8, kFetchesPerWarp = 3;
+// The fetches are dealt out to strips of the cells, 16 for fetches of 8 chunks and more for
+// shorter ones (kSpread chunks in all), so that the resident warps work in many places: next
+// to each other they queue up at the same pixels where a map is strongly compressed
+// (4000^2 cells of a field at high magnification on 100^2 pixels: 15.5 ms with short
+// fetches in one strip, 9.4 in strips).  Passes of more than kStripCells cells, whose corners
+// do not stay in L2, take fetches of 8 chunks in order (critical-curve map: 16 strips 744 ms
+// against 643).
+constexpr int kSpread = 128;
+constexpr int64_t kStripCells = 6 << 20;
 // Cells per chunk: 32, fewer (down to kMinLanes lanes with a cell) while that leaves fewer
 // than kChunksPerWarp chunks for a resident warp.  Most of a round's work is pixels and rows,
 // spread over all lanes whoever holds the cells, so short rounds cost little and a
@@ -69,38 +77,37 @@ __global__ void __launch_bounds__(kIpmThreads, kBlocksPerSm) k_ipm_cells(IpmArgs
   // warps of a block finish together however the large cells fall; one
   // fetch takes A.grab chunks.
   unsigned* next = reinterpret_cast<unsigned*>(A.qcount) + 1;
-  unsigned g_u = 0;
-  if (lane == 0) g_u = atomicAdd(next, 1u);
-  const int grab = A.grab;
-  int left = grab;
-  for (int64_t ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * grab; ch < nchunks;) {
+  // (the first fetch is the warp's number)
+  const unsigned warps = gridDim.x * kWarps;
+  unsigned g_u = blockIdx.x * kWarps + w;
+  for (;;) {
+    const unsigned f = __shfl_sync(0xffffffffu, g_u, 0), pos = f >> A.strips;
+    if (pos >= A.per) break;
     // the following grab is fetched while this one is processed
-    if (lane == 0 && left == grab) g_u = atomicAdd(next, 1u);
-    const int64_t idx = ch * lanes + lane;
-    const bool has = lane < lanes && idx < A.ncells;
-    int64_t c = idx;
-    PixCorner q4[4];
-    if (has) {
-      if (LIST) c = A.cell_list[idx];
-      if (QUADS) {
+    if (lane == 0) g_u = warps + atomicAdd(next, 1u);
+    int64_t ch = ((int64_t)(f - (pos << A.strips)) * A.per + pos) * A.grab;
+    const int64_t end = min64(ch + A.grab, nchunks);
+    for (; ch < end; ++ch) {
+      const int64_t idx = ch * lanes + lane;
+      const bool has = lane < lanes && idx < A.ncells;
+      int64_t c = idx;
+      PixCorner q4[4];
+      if (has) {
+        if (LIST) c = A.cell_list[idx];
+        if (QUADS) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) q4[k] = A.yc[4 * c + k];
-      } else {
-        const int64_t j = cell_row(A, (uint32_t)c);
-        const PixCorner* y0 = A.yc + (c + j);  // j W + i = c + j
-        q4[0] = y0[0];
-        q4[1] = y0[1];
-        q4[2] = y0[W + 1];
-        q4[3] = y0[W];
+          for (int k = 0; k < 4; ++k) q4[k] = A.yc[4 * c + k];
+        } else {
+          const int64_t j = cell_row(A, (uint32_t)c);
+          const PixCorner* y0 = A.yc + (c + j);  // j W + i = c + j
+          q4[0] = y0[0];
+          q4[1] = y0[1];
+          q4[2] = y0[W + 1];
+          q4[3] = y0[W];
+        }
       }
-    }
-    ipm_round<false>(A, sh[w], lane, has, c, q4, led);
-    __syncwarp();  // the next chunk overwrites this one's staging
-    if (--left > 0) {
-      ++ch;
-    } else {
-      left = grab;
-      ch = (int64_t)__shfl_sync(0xffffffffu, g_u, 0) * grab;
+      ipm_round<false>(A, sh[w], lane, has, c, q4, led);
+      __syncwarp();  // the next chunk overwrites this one's staging
     }
   }
   block_add_stats<kWarps>(A.stats, led, A.wcell);
@@ -191,13 +198,17 @@ void ipm_launch(IpmArgs& A, bool quads, int* qcount, cudaStream_t s,
   const int64_t warps = (int64_t)sms * kBlocksPerSm * kWarps;
   while (A.lanes > kMinLanes && A.ncells / A.lanes < kChunksPerWarp * warps) A.lanes /= 2;
   const int64_t chunk_blocks = (A.ncells + A.lanes * kWarps - 1) / (A.lanes * kWarps);
-  const unsigned g = (unsigned)std::min<int64_t>(chunk_blocks, (int64_t)sms * 8);
+  const unsigned g = (unsigned)std::min<int64_t>(chunk_blocks, (int64_t)sms * kBlocksPerSm);
   int L = 0;
   while ((1ll << L) < A.nx) ++L;
   A.div_s = 30 + L;
   A.div_m = A.nx > 0 ? (uint32_t)((1ull << A.div_s) / (uint64_t)A.nx + 1) : 0;
   A.grab = (int)std::max<int64_t>(
-      1, std::min<int64_t>(kMaxGrab, A.ncells / A.lanes / (warps * 8)));
+      1, std::min<int64_t>(kMaxGrab, A.ncells / A.lanes / (warps * kFetchesPerWarp)));
+  const int64_t fetches = (A.ncells + (int64_t)A.lanes * A.grab - 1) / ((int64_t)A.lanes * A.grab);
+  A.strips = 0;
+  while (A.ncells <= kStripCells && A.grab << A.strips < kSpread && fetches >> A.strips >= 8) ++A.strips;
+  A.per = (unsigned)((fetches + (1 << A.strips) - 1) >> A.strips);
   if (quads) k_ipm_cells<true><<<g, kIpmThreads, 0, s>>>(A);
   else if (A.cell_list) k_ipm_cells<false, true><<<g, kIpmThreads, 0, s>>>(A);
   else k_ipm_cells<false><<<g, kIpmThreads, 0, s>>>(A);

@@ -36,6 +36,7 @@ struct IpmArgs {
   float wcell;          // cell area in units of the grid's cell (1, or 4^-level for sub-cells)
   int* rq; int* rqcount;  // refinement: cells over the cap are queued here (NULL: dropped)
   int grab;               // k_ipm_cells: chunks per fetch of the chunk counter
+  int strips; unsigned per;  // k_ipm_cells: log2 of the strips that the fetches are dealt to, fetches a strip
   int lanes;              // k_ipm_cells: cells per chunk
   uint32_t div_m; int div_s;  // c / nx as (c div_m) >> div_s for cell ids c < 2^30
   const int* cell_list;   // k_ipm_cells: the cells to map (ids into yc's grid), or NULL: all
