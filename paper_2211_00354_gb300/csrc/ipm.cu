@@ -31,19 +31,22 @@ namespace {
 
 constexpr int kIpmThreads = 256;
 // 32-cell chunks per fetch of the chunk counter: at most 8 (a single address serves all
-// warps, ~2 ns a fetch: a fetch per chunk made it the bound of a pass of single-pixel cells),
-// fewer where that would leave a resident warp under kFetchesPerWarp: with 8 always, the 900
+// warps, ~2 ns a fetch: a fetch per chunk made it the bound of a pass without B and C work),
+// fewer where that would leave a resident warp under 8 fetches: with 8 always, the 900
 // chunks of a refinement level went to 112 of 4864 warps (308 us of a 200^2-pixel window's
-// map). 8 fetches a warp instead of 3: 4e6 cells of single pixels 113 -> 170 us.
-constexpr int kMaxGrab = 8, kFetchesPerWarp = 3;
-// The fetches are dealt out to strips of the cells, 16 for fetches of 8 chunks and more for
-// shorter ones (kSpread chunks in all), so that the resident warps work in many places: next
-// to each other they queue up at the same pixels where a map is strongly compressed
-// (4000^2 cells of a field at high magnification on 100^2 pixels: 15.5 ms with short
-// fetches in one strip, 9.4 in strips).  Passes of more than kStripCells cells, whose corners
-// do not stay in L2, take fetches of 8 chunks in order (critical-curve map: 16 strips 744 ms
-// against 643).
-constexpr int kSpread = 128;
+// map) and the 7.8e3 chunks of a 500^2 grid to 976.
+constexpr int kMaxGrab = 8, kFetches = 8;
+// A pass of kDense cells a map pixel or more: 3 fetches a warp are enough (cells of a pixel
+// or two each: 4e6 of them 340 us, with 8 fetches 498), and they are dealt out to strips of the
+// cells, 16 for fetches of 8 chunks and more for shorter ones (kSpread chunks in all), so that
+// the resident warps work in many places: next to each other they queue up at the same
+// pixels where a map is strongly compressed (4000^2 cells of a field at high magnification on
+// 100^2 pixels: 15.5 ms in one strip, 9.4 so).  Sparser passes go in order (4e6 cells, the
+// tenth of them that falls on the map's 4e6 pixels 10 pixels long: 160 us, in strips 265),
+// and so do those of more than kStripCells cells, whose corners do not stay in L2 (critical-
+// curve map: 643 ms, in strips 744).
+constexpr int kFetchesDense = 3, kSpread = 128;
+constexpr double kDense = 1.5;
 constexpr int64_t kStripCells = 6 << 20;
 // Cells per chunk: 32, fewer (down to kMinLanes lanes with a cell) while that leaves fewer
 // than kChunksPerWarp chunks for a resident warp.  Most of a round's work is pixels and rows,
@@ -203,11 +206,13 @@ void ipm_launch(IpmArgs& A, bool quads, int* qcount, cudaStream_t s,
   while ((1ll << L) < A.nx) ++L;
   A.div_s = 30 + L;
   A.div_m = A.nx > 0 ? (uint32_t)((1ull << A.div_s) / (uint64_t)A.nx + 1) : 0;
+  const bool dense = (double)A.ncells >= kDense * A.ip.npx * A.ip.npy;
   A.grab = (int)std::max<int64_t>(
-      1, std::min<int64_t>(kMaxGrab, A.ncells / A.lanes / (warps * kFetchesPerWarp)));
+      1, std::min<int64_t>(kMaxGrab, A.ncells / A.lanes / (warps * (dense ? kFetchesDense : kFetches))));
   const int64_t fetches = (A.ncells + (int64_t)A.lanes * A.grab - 1) / ((int64_t)A.lanes * A.grab);
   A.strips = 0;
-  while (A.ncells <= kStripCells && A.grab << A.strips < kSpread && fetches >> A.strips >= 8) ++A.strips;
+  if (dense && A.ncells <= kStripCells)
+    while (A.grab << A.strips < kSpread && fetches >> A.strips >= 8) ++A.strips;
   A.per = (unsigned)((fetches + (1 << A.strips) - 1) >> A.strips);
   if (quads) k_ipm_cells<true><<<g, kIpmThreads, 0, s>>>(A);
   else if (A.cell_list) k_ipm_cells<false, true><<<g, kIpmThreads, 0, s>>>(A);
